@@ -379,7 +379,7 @@ int fppg_batch_load(fppg_batch *b);
  * with the fastest force kernel, the triangle search on 8 or 16 CTAs per SM
  * or -- search CTAs 0 -- one thread per queued particle on 16 CTAs per SM;
  * then, with the fastest of those, the two ways of ordering the cell keys
- * (a full stable sort, or the incremental repair of the previous order,
+ * (a full stable sort, or the counting sort over the fine keys,
  * fppg_batch_set_incremental), then the two orders of the grid rows
  * (fppg_batch_set_cell_order), keeps the fastest and restores the particle
  * state afterwards.  The choice is cached per (particle-count bucket,
@@ -389,20 +389,21 @@ int fppg_batch_load(fppg_batch *b);
  * particles between the force loop's two partial sums, so it agrees with
  * row-major rows up to FP32 rounding (a plain body set to the same row
  * order gives the batch's bits).  Outputs (nullable): chosen variant,
- * block size, search CTAs, ordering (1 incremental), row order and the
+ * block size, search CTAs, ordering (1 counting sort), row order and the
  * measured ms per iteration (0 when taken from the cache). */
 int fppg_batch_autotune(fppg_batch *b, int32_t iters, int32_t *variant, int32_t *block, int32_t *search_ctas,
                         int32_t *incremental, int32_t *cell_order, double *ms_per_iter);
 /* How the cell keys are put in order every iteration (Sec. 3.1.3): 0 a full
- * stable radix sort of every key; 1 the previous order repaired -- the
- * particles whose key changed since the last grid build are sorted alone and
- * merged with the others, which keep their order.  Both give the one order by
- * (key, particle id), so the results are the same bits; the incremental form
- * moves less data once few keys change per iteration (large groups start
- * with it).  Drops a captured graph.  FPPG_ERR_ARG for other values. */
+ * stable radix sort of every key; 1 (the start) a counting sort over the
+ * dense fine keys, which gives the start table and the order together: the
+ * keys are counted as they are made, and particles that share a key are
+ * ranked by id.  Both give the one order by (key, particle id), so the
+ * results are the same bits.  The counting sort's work for a particle grows
+ * with the number that share its key, as its pairs do.  Drops a captured
+ * graph.  FPPG_ERR_ARG for other values. */
 int fppg_batch_set_incremental(fppg_batch *b, int32_t incremental);
 /* The same for the single body of a handle (its fppg_relax, fppg_stats and
- * debug calls); a body of at least 2^21 particles starts incremental. */
+ * debug calls). */
 int fppg_set_incremental(fppg_ctx *ctx, int32_t incremental);
 /* Order of the neighbour grid's rows in the cell key (Sec. 3.1.3 sorts
  * particles by cell; Eq. 9 gives the Morton code of a cell):
@@ -419,8 +420,7 @@ int fppg_set_incremental(fppg_ctx *ctx, int32_t incremental);
  * FP32 rounding of the two partial sums a row's slots are split between
  * (by the parity of their absolute position); the keys and the permutation
  * follow the order.  The rank table of every grid is built on first use
- * (FPPG_ERR_ARG above 2^26 rows).  The previous order of the keys is
- * forgotten.  fppg_set_cell_order for the body of a handle,
+ * (FPPG_ERR_ARG above 2^26 rows).  fppg_set_cell_order for the body of a handle,
  * fppg_batch_set_cell_order for a batch (bodies of a batch take the
  * batch's order). */
 #define FPPG_ORDER_ROWS 0
@@ -469,12 +469,11 @@ int fppg_device_sm_count(int32_t *sms);
 /* Bounds checks.  A library built with -DFPPG_CHECKED (the `checked`
  * build of paper_2501_03056_gb300._build) checks, in the hot-path kernels,
  * every index it computes before using it: the sorted ids and fine keys of
- * the gather, each grid row's slot range of the force pass, the search
- * queue's slots and entries, the candidate triangles of the searches, the
- * compaction positions and merge splits of the incremental order.  A
- * failed check skips the access and ORs its code into a device word:
- * 1 gather, 2 slot range, 4 queue slot, 8 queue entry, 16 candidate
- * triangle, 32 merge split, 64 compaction position.  fppg_check_status
+ * the gather, the slots of the counting sort, each grid row's slot range of
+ * the force pass, the search queue's slots and entries, the candidate
+ * triangles of the searches.  A failed check skips the access and ORs its
+ * code into a device word: 1 gather or slot, 2 slot range, 4 queue slot,
+ * 8 queue entry, 16 candidate triangle.  fppg_check_status
  * returns that word in *word and clears it (0 in the normal build, where
  * the checks compile away), and *checked (nullable) = 1 for the checked
  * build.  FPPG_ERR_ARG for word NULL; FPPG_ERR_CUDA when the word cannot be

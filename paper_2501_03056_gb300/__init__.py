@@ -216,8 +216,8 @@ class Body:
         self._chk(lib().fppg_set_projection_rule(self._h, 1 if cascade else 0))
 
     def set_incremental(self, on: bool):
-        """Order the keys by repairing the previous order (True) or by a full
-        stable sort (False); both give the same bits."""
+        """Order the keys by the counting sort over the fine keys (True) or by
+        a full stable radix sort (False); both give the same bits."""
         self._chk(lib().fppg_set_incremental(self._h, int(bool(on))))
 
     def set_cell_order(self, order: int):
@@ -583,8 +583,8 @@ class Batch:
         self._chk(lib().fppg_batch_set_cell_order(self._h, int(order)))
 
     def set_incremental(self, on: bool):
-        """Order the keys by repairing the previous order (True) or by a full
-        stable sort (False); both give the same bits."""
+        """Order the keys by the counting sort over the fine keys (True) or by
+        a full stable radix sort (False); both give the same bits."""
         self._chk(lib().fppg_batch_set_incremental(self._h, int(bool(on))))
 
     def set_mobile_classes(self, classes):

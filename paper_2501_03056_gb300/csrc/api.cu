@@ -45,7 +45,7 @@ struct fppg_ctx {
         return nullptr;
     }
     int64_t n_ghost = 0;           // the last n_ghost particles are ghosts (fppg_set_ghost_count)
-    int split_buf = -1;            // grid buffer of the last fppg_relax_forces, until its step
+    bool split = false;            // after fppg_relax_forces, until its step
     // device staging of the host particle arrays of set / get, kept between
     // calls (both synchronise the stream before they return)
     void *stage = nullptr;
@@ -379,7 +379,7 @@ int fppg_set_particles(fppg_ctx *ctx, const float *xyz_host, const int32_t *cls_
     }
     Group &g = ctx->group;
     ctx->has_particles = false;     // until the new set is complete
-    ctx->split_buf = -1;
+    ctx->split = false;
     ctx->n_ghost = 0;
     if (n != g.d.N || !g.d.pos) {
         int r = g.alloc_particles(n, ctx->err);
@@ -591,12 +591,13 @@ int fppg_relax_forces(fppg_ctx *ctx, float *amax_host) {
     uint32_t a = 0u;
     if (ctx->n > 0) {
         Group &g = ctx->group;
-        ctx->split_buf = build_grid(g, ctx->stream);
+        build_grid(g, ctx->stream);
+        ctx->split = true;
         forces(g, ctx->stream, nullptr);
         CUDA_OR(ctx->err, cudaMemcpyAsync(&a, g.d.amax, sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
         CUDA_OR(ctx->err, cudaStreamSynchronize(ctx->stream));
     } else {
-        ctx->split_buf = 0;
+        ctx->split = true;
     }
     memcpy(amax_host, &a, sizeof(float));
     return FPPG_OK;
@@ -604,16 +605,15 @@ int fppg_relax_forces(fppg_ctx *ctx, float *amax_host) {
 
 int fppg_relax_step(fppg_ctx *ctx, float amax) {
     if (!ctx) return FPPG_ERR_ARG;
-    if (ctx->split_buf < 0) return fail(ctx->err, FPPG_ERR_STATE, "fppg_relax_step needs a fppg_relax_forces first");
+    if (!ctx->split) return fail(ctx->err, FPPG_ERR_STATE, "fppg_relax_step needs a fppg_relax_forces first");
     if (!(amax >= 0.f) || !std::isfinite(amax)) return fail(ctx->err, FPPG_ERR_ARG, "amax must be finite, >= 0");
-    const int buf = ctx->split_buf;
-    ctx->split_buf = -1;
+    ctx->split = false;
     if (ctx->n == 0) return FPPG_OK;
     Group &g = ctx->group;
     uint32_t a;
     memcpy(&a, &amax, sizeof(a));
     CUDA_OR(ctx->err, cudaMemcpyAsync(g.d.amax, &a, sizeof(uint32_t), cudaMemcpyHostToDevice, ctx->stream));
-    step_and_project(g, ctx->stream, buf);
+    step_and_project(g, ctx->stream);
     CUDA_OR(ctx->err, cudaStreamSynchronize(ctx->stream));
     return FPPG_OK;
 }
@@ -638,10 +638,11 @@ int fppg_debug_grid(fppg_ctx *ctx, uint32_t *key_host, uint32_t *perm_host, uint
         if (n_cells) *n_cells = 0;
         return FPPG_OK;
     }
-    int buf = build_grid(g, ctx->stream);
+    build_grid(g, ctx->stream);
     std::vector<uint32_t> ks(n), perm(n);
-    CUDA_OR(ctx->err, cudaMemcpyAsync(ks.data(), g.d.key[buf], 4 * n, cudaMemcpyDeviceToHost, ctx->stream));
-    CUDA_OR(ctx->err, cudaMemcpyAsync(perm.data(), g.d.id[buf], 4 * n, cudaMemcpyDeviceToHost, ctx->stream));
+    CUDA_OR(ctx->err, cudaMemcpyAsync(ks.data(), sorted_keys(g.d, ctx->stream), 4 * n, cudaMemcpyDeviceToHost,
+                                      ctx->stream));
+    CUDA_OR(ctx->err, cudaMemcpyAsync(perm.data(), g.d.id_s, 4 * n, cudaMemcpyDeviceToHost, ctx->stream));
     // the dense start table: cell c holds the slots [fstart[8c], fstart[8c + 8])
     std::vector<uint32_t> table((size_t)kSlabs * (size_t)g.d.total_cells + 1);
     CUDA_OR(ctx->err, cudaMemcpyAsync(table.data(), g.d.fstart, sizeof(uint32_t) * table.size(),
@@ -676,9 +677,9 @@ int fppg_debug_forces(fppg_ctx *ctx, float *acc_host, int32_t *count_host, float
     CUDA_OR(ctx->err, dev_malloc(&dacc, sizeof(float) * 3 * n));
     CUDA_OR(ctx->err, dev_malloc(&dcnt_s, sizeof(int32_t) * n));
     CUDA_OR(ctx->err, dev_malloc(&dcnt, sizeof(int32_t) * n));
-    int buf = build_grid(g, ctx->stream);
+    build_grid(g, ctx->stream);
     forces(g, ctx->stream, dcnt_s);
-    unpermute(g, buf, ctx->stream, dacc, dcnt_s, dcnt);
+    unpermute(g, ctx->stream, dacc, dcnt_s, dcnt);
     uint32_t am = 0;
     if (acc_host) CUDA_OR(ctx->err, cudaMemcpyAsync(acc_host, dacc, sizeof(float) * 3 * n, cudaMemcpyDeviceToHost, ctx->stream));
     if (count_host)
@@ -1135,13 +1136,6 @@ std::mutex g_tune_mu;
 std::map<TuneKey, TuneVal> g_tune_cache;
 } // namespace
 
-// switch the ordering of the keys; entering the incremental form forgets
-// the previous order (its arrays may be stale after full sorts)
-static void set_ordering(Group &g, bool incremental, cudaStream_t s) {
-    if (incremental && !g.d.incremental) g.invalidate_order(s);
-    g.d.incremental = incremental;
-}
-
 int fppg_batch_autotune(fppg_batch *b, int32_t iters, int32_t *variant, int32_t *block, int32_t *search_ctas,
                         int32_t *incremental, int32_t *cell_order, double *ms_per_iter) {
     NvtxRange nvtx_("fppg_batch_autotune");
@@ -1161,7 +1155,7 @@ int fppg_batch_autotune(fppg_batch *b, int32_t iters, int32_t *variant, int32_t 
     while ((int64_t)1 << (nb + 1) <= std::max<int64_t>(d.N, 1)) nb++;
     const TuneKey key{nb, d.N ? (int)(10 * nv / d.N) : 0, prop.name};
     TuneVal best{g.force_variant, g.force_block, g.search_thread ? 0 : g.search_blocks / std::max(sms, 1),
-                 d.incremental ? 1 : 0, g.cell_order};
+                 d.counted ? 1 : 0, g.cell_order};
     double best_ms = 0.0;
     bool cached = false;
     {
@@ -1194,7 +1188,7 @@ int fppg_batch_autotune(fppg_batch *b, int32_t iters, int32_t *variant, int32_t 
             g.force_block = tb;
             g.search_thread = sc == 0;
             g.search_blocks = (sc == 0 ? 16 : sc) * sms;
-            set_ordering(g, inc != 0, s);
+            d.counted = inc != 0;
             if (co != g.cell_order) {
                 const int r = g.set_cell_order(co, s, b->err);
                 if (r) return r == 1 ? FPPG_ERR_ARG : (r == 3 ? FPPG_ERR_OOM : FPPG_ERR_CUDA);
@@ -1250,7 +1244,7 @@ int fppg_batch_autotune(fppg_batch *b, int32_t iters, int32_t *variant, int32_t 
     g.force_block = best.block;
     g.search_thread = best.search_ctas == 0;
     g.search_blocks = (best.search_ctas == 0 ? 16 : best.search_ctas) * sms;
-    set_ordering(g, best.incremental != 0, s);
+    d.counted = best.incremental != 0;
     if (best.cell_order != g.cell_order) {
         const int r = g.set_cell_order(best.cell_order, s, b->err);
         if (r) return r == 1 ? FPPG_ERR_ARG : (r == 3 ? FPPG_ERR_OOM : FPPG_ERR_CUDA);
@@ -1333,20 +1327,18 @@ int fppg_device_sm_count(int32_t *sms) {
 
 int fppg_set_incremental(fppg_ctx *ctx, int32_t incremental) {
     if (!ctx || incremental < 0 || incremental > 1) return FPPG_ERR_ARG;
-    set_ordering(ctx->group, incremental != 0, ctx->stream);
-    CUDA_OR(ctx->err, cudaGetLastError());
+    ctx->group.d.counted = incremental != 0;
     return FPPG_OK;
 }
 
 int fppg_batch_set_incremental(fppg_batch *b, int32_t incremental) {
     if (!b || incremental < 0 || incremental > 1) return FPPG_ERR_ARG;
     Group &g = b->group;
-    set_ordering(g, incremental != 0, b->stream);
+    g.d.counted = incremental != 0;
     if (g.graph) {
         cudaGraphExecDestroy(g.graph);
         g.graph = nullptr;
     }
-    CUDA_OR(b->err, cudaGetLastError());
     return FPPG_OK;
 }
 
@@ -1358,7 +1350,7 @@ int fppg_batch_set_cell_order(fppg_batch *b, int32_t order) {
 }
 
 int32_t fppg_batch_kernels_per_iter(const fppg_batch *b) {
-    // keys, 3 per radix pass, gather, the start scan, force, step, search
+    // the grid build, force, step, search
     return b ? grid_kernels(b->group.d) + 3 : -1;
 }
 

@@ -258,10 +258,11 @@ void Group::release_particles() {
     DevGroup &g = d;
     void *ptrs[] = {g.pos,    g.cons,   g.cons_s,   g.key[0], g.key[1],  g.id[0],   g.id[1],  g.pos_s,
                     g.pos_p,  g.cert,   g.acc_s,    g.hist,   g.coef_s,  g.work,    g.fstart, g.bstart,
-                    g.amax,   g.maxdisp, g.work_count, g.totals};
+                    g.amax,   g.maxdisp, g.work_count, g.totals, g.cnt, g.tiles, g.tile_base, g.scan_tmp};
     for (void *p : ptrs)
         if (p) cudaFree(p);
-    free_order_state();
+    g.cnt = g.tiles = g.tile_base = g.scan_tmp = nullptr;
+    g.id_s = g.key_s = nullptr;
     g.pos = g.pos_s = g.pos_p = g.cert = g.acc_s = nullptr;
     g.cons = g.cons_s = nullptr;
     g.key[0] = g.key[1] = g.id[0] = g.id[1] = nullptr;
@@ -275,58 +276,6 @@ int Group::alloc_particles(int64_t N, std::string &err) {
     const int r = alloc_particles_once(N, err);
     if (r) release_particles();   // no half-allocated group: the next call starts over
     return r;
-}
-
-void Group::free_order_state() {
-    DevGroup &g = d;
-    void *ptrs[] = {g.key_id, g.chg_bits, g.keep_bits, g.tile_cnt, g.tile_pos, g.ck[0], g.ck[1], g.cv[0],
-                    g.cv[1],  g.uk,       g.uv,        g.split,    g.counts,   g.scan_tmp_n};
-    for (void *p : ptrs)
-        if (p) cudaFree(p);
-    g.key_id = g.chg_bits = g.keep_bits = g.tile_cnt = g.tile_pos = nullptr;
-    g.uk = g.uv = g.split = g.counts = g.scan_tmp_n = nullptr;
-    g.ck[0] = g.ck[1] = g.cv[0] = g.cv[1] = nullptr;
-}
-
-__global__ void k_iota_u32(uint32_t *__restrict__ a, int64_t n) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) a[i] = (uint32_t)i;
-}
-
-// The arrays of the incremental ordering: the previous order starts as the
-// identity over ids with no key recorded, so the first grid build sorts
-// every particle.  Allocated with the particles.
-int Group::alloc_order_state(std::string &err) {
-    DevGroup &g = d;
-    free_order_state();
-    const size_t n1 = (size_t)std::max<int64_t>(g.N, 1);
-    const int64_t nblk = (std::max<int64_t>(g.N, 1) + 2047) / 2048;
-    CKA(dev_malloc(&g.key_id, sizeof(uint32_t) * n1));
-    // tiles of 2048 (those of the compactions), 32 flags a word
-    const int64_t ntile = (std::max<int64_t>(g.N, 1) + 2047) / 2048;
-    const size_t nword = (size_t)(ntile * 64);
-    CKA(dev_malloc(&g.chg_bits, sizeof(uint32_t) * nword));
-    CKA(dev_malloc(&g.keep_bits, sizeof(uint32_t) * nword));
-    CKA(dev_malloc(&g.tile_cnt, sizeof(uint32_t) * (size_t)(2 * ntile)));
-    CKA(dev_malloc(&g.tile_pos, sizeof(uint32_t) * (size_t)(2 * ntile)));
-    for (int k = 0; k < 2; k++) {
-        CKA(dev_malloc(&g.ck[k], sizeof(uint32_t) * n1));
-        CKA(dev_malloc(&g.cv[k], sizeof(uint32_t) * n1));
-    }
-    CKA(dev_malloc(&g.uk, sizeof(uint32_t) * n1));
-    CKA(dev_malloc(&g.uv, sizeof(uint32_t) * n1));
-    CKA(dev_malloc(&g.split, sizeof(uint32_t) * (size_t)(nblk + 2)));
-    CKA(dev_malloc(&g.counts, 2 * sizeof(uint32_t)));
-    CKA(dev_malloc(&g.scan_tmp_n, sizeof(uint32_t) * (size_t)scan_tmp_elems(2 * ntile)));
-    CKA(cudaMemset(g.key_id, 0xff, sizeof(uint32_t) * n1));
-    k_iota_u32<<<(unsigned)((n1 + 255) / 256), 256>>>(g.id[0], (int64_t)n1);
-    CKA(cudaGetLastError());
-    CKA(cudaDeviceSynchronize());
-    return 0;
-}
-
-void Group::invalidate_order(cudaStream_t s) {
-    if (d.key_id && d.N > 0) cudaMemsetAsync(d.key_id, 0xff, sizeof(uint32_t) * (size_t)d.N, s);
 }
 
 int Group::alloc_particles_once(int64_t N, std::string &err) {
@@ -368,17 +317,19 @@ int Group::alloc_particles_once(int64_t N, std::string &err) {
     CKA(dev_malloc(&g.hist, sizeof(uint32_t) * kMaxDigits * (size_t)g.n_tiles));
     if (!g.totals) CKA(dev_malloc(&g.totals, sizeof(uint32_t) * kMaxDigits));
     if (!g.fstart) {
-        // dense start table of every fine key (+1), the counts it is scanned
-        // from (zero between iterations) and the scan's block sums
-        const size_t f1 = (size_t)kSlabs * (size_t)std::max<int64_t>(g.total_cells, 1) + 1;
-        CKA(dev_malloc(&g.fstart, sizeof(uint32_t) * f1));
-        CKA(dev_malloc(&g.bstart, sizeof(uint32_t) * (size_t)(start_blocks((int64_t)f1) + 1)));
-    }
-    // the incremental ordering for large groups (the autotuner may switch)
-    {
-        const int r = alloc_order_state(err);
-        if (r) return r;
-        g.incremental = N >= kIncrementalMinN;
+        // dense start table of every fine key (+1), and the counts it is
+        // scanned from (zero between grid builds)
+        const int64_t f1 = kSlabs * std::max<int64_t>(g.total_cells, 1) + 1, nt = count_tiles(f1);
+        CKA(dev_malloc(&g.fstart, sizeof(uint32_t) * (size_t)f1));
+        CKA(dev_malloc(&g.bstart, sizeof(uint32_t) * (size_t)(start_blocks(f1) + 1)));
+        CKA(dev_malloc(&g.cnt, sizeof(uint32_t) * (size_t)f1));
+        CKA(dev_malloc(&g.tiles, sizeof(uint32_t) * (size_t)nt));
+        CKA(cudaMemset(g.cnt, 0, sizeof(uint32_t) * (size_t)f1));
+        if (nt > kScanTiles) {
+            CKA(dev_malloc(&g.tile_base, sizeof(uint32_t) * (size_t)nt));
+            CKA(dev_malloc(&g.scan_tmp, sizeof(uint32_t) * (size_t)scan_tmp_elems(nt)));
+        }
+        g.counted = true;    // the faster form at every size measured (the autotuner may switch)
     }
     if (!g.amax) {
         CKA(dev_malloc(&g.amax, sizeof(uint32_t) * (size_t)std::max(g.B, 1)));
@@ -428,7 +379,6 @@ int Group::set_cell_order(int order, cudaStream_t s, std::string &err) {
     cell_order = order;
     d.morton_rows = order != 0;
     for (size_t i = 0; i < hp.size(); i++) hp[i].row_rank = order ? d.row_rank + row_off[i] : nullptr;
-    invalidate_order(s);
     return upload_params(s, err);
 }
 
@@ -443,7 +393,7 @@ void Group::free_all() {
     DevGroup &g = d;
     void *ptrs[] = {g.params, g.row_rank, g.pos, g.cons, g.cons_s, g.key[0], g.key[1], g.id[0], g.id[1], g.pos_s, g.pos_p, g.cert,
                     g.acc_s, g.fstart, g.bstart, g.amax, g.maxdisp, g.hist, g.totals, g.coef_s, g.work,
-                    g.work_count};
+                    g.work_count, g.cnt, g.tiles, g.tile_base, g.scan_tmp};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (owns_mesh) {

@@ -130,15 +130,10 @@ struct Group {
     int alloc_particles(int64_t N, std::string &err);   // on failure: nothing allocated, N = 0
     int alloc_particles_once(int64_t N, std::string &err);
     void release_particles();
-    int alloc_order_state(std::string &err);
-    void free_order_state();
-    // forget the previous order (the next grid build sorts every key); used
-    // when the incremental ordering is switched on
-    void invalidate_order(cudaStream_t s);
     int upload_params(cudaStream_t s, std::string &err);
     // the rank tables of the grids of hp (built once), then every body's
-    // parameters pointed at its table (order 1) or at none (order 0); the
-    // previous order of the keys is forgotten.  Uploads the parameters.
+    // parameters pointed at its table (order 1) or at none (order 0).
+    // Uploads the parameters.
     int set_cell_order(int order, cudaStream_t s, std::string &err);
     void free_all();
     ~Group() { free_all(); }
@@ -161,34 +156,32 @@ uint32_t check_word_take();
 // the bits of y and z interleaved, z's above y's at every level
 void morton_row_ranks(int ny, int nz, std::vector<uint32_t> &rank);
 
-// groups of at least this many particles start with the incremental ordering
-constexpr int64_t kIncrementalMinN = 1 << 21;
-
 // event records per timed iteration: before A1, after A3, A4, A5 and A6
 constexpr int kPhaseEvents = 5;
 // one relaxation iteration of every body of the group (A1-A6)
 void iterate(Group &g, cudaStream_t s, bool energy_mode, int32_t *count_dbg = nullptr);
-// A5-A6 (step, then the projections) after a grid build that returned buf
-// and a force pass; amax is whatever the device holds
-void step_and_project(Group &g, cudaStream_t s, int buf);
+// A5-A6 (step, then the projections) after a grid build and a force pass;
+// amax is whatever the device holds
+void step_and_project(Group &g, cudaStream_t s);
 // particles [first_ghost, N) become ghosts, the others not (the ghost bit of w)
 void tag_ghosts(Group &g, int64_t first_ghost, cudaStream_t s);
-// A1-A3 only (keys, sort, gather + cell ranges); returns the buffer index
-// holding the sorted keys / ids
-int build_grid(Group &g, cudaStream_t s);
+// A1-A3 only (keys, order, gather + cell ranges)
+void build_grid(Group &g, cudaStream_t s);
+// the sorted keys of the last grid build (device memory, until the next)
+const uint32_t *sorted_keys(DevGroup &d, cudaStream_t s);
 // the same on bare device arrays (no Group): A1-A3, A4, back to id order
-int build_grid_dev(DevGroup &d, cudaStream_t s);
+void build_grid_dev(DevGroup &d, cudaStream_t s);
 // kernel launches of one grid build (A1-A3)
 int grid_kernels(const DevGroup &d);
 void forces_dev(DevGroup &d, int block, int variant, cudaStream_t s, int32_t *count_s = nullptr,
                 int32_t *tested_s = nullptr);
-void unpermute_dev(DevGroup &d, int buf, cudaStream_t s, float *acc_out, const int32_t *count_s, int32_t *count_out);
+void unpermute_dev(DevGroup &d, cudaStream_t s, float *acc_out, const int32_t *count_s, int32_t *count_out);
 // A4 into acc_s (and counts when non-null)
 void forces(Group &g, cudaStream_t s, int32_t *count_s, int32_t *cand_s = nullptr, int32_t *tested_s = nullptr);
 // energy-descent acceleration -dE/dx into acc_s
 void energy_accel(Group &g, cudaStream_t s);
 // debug helpers
-void unpermute(Group &g, int buf, cudaStream_t s, float *acc_out, const int32_t *count_s, int32_t *count_out);
+void unpermute(Group &g, cudaStream_t s, float *acc_out, const int32_t *count_s, int32_t *count_out);
 void project_points(Group &g, const float *y, const int32_t *cls, const int32_t *cons_in, int64_t n, float *x,
                     int32_t *cons_out, int32_t *ok, cudaStream_t s);
 // uniformity statistics into host doubles (see fppg_stats_t)

@@ -397,14 +397,14 @@ int energy(Group &g, const Body &b, const float *y_dev, const float *verts_dev, 
     float4 *saved = d.pos;
     k_project_frozen<<<nblocks(N), TPB, 0, s>>>(y_dev, d.pos, d.cons, N, V, b.d_tris, es.xs);
     d.pos = es.xs;
-    int buf = build_grid(g, s);
+    build_grid(g, s);
     d.pos = saved;
     k_rho<<<nblocks(N + 1), TPB, 0, s>>>(d.pos_s, d.pos_p, N, d.params, d.fstart, d.coef_s, es.e_s);
     k_sum_fixed<<<kSumBlocks, TPB, 0, s>>>(es.e_s, N, es.part);
     k_sum_fixed<<<1, TPB, 0, s>>>(es.part, kSumBlocks, es.part + kSumBlocks);
     if (gy || gV) {
         k_grad<<<nblocks(N), TPB, 0, s>>>(d.pos_s, d.pos_p, N, d.params, d.fstart, d.coef_s, 1.f, d.acc_s, nullptr);
-        k_vjp<<<nblocks(N), TPB, 0, s>>>(d.acc_s, d.id[buf], N, y_dev, d.pos, d.cons, V, b.d_tris, b.nv, gy,
+        k_vjp<<<nblocks(N), TPB, 0, s>>>(d.acc_s, d.id_s, N, y_dev, d.pos, d.cons, V, b.d_tris, b.nv, gy,
                                           gV ? es.vk[0] : nullptr, es.vcon);
         if (gV) {
             cudaMemsetAsync(gV, 0, sizeof(float) * 3 * (size_t)b.nv, s);

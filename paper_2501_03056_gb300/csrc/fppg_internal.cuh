@@ -153,19 +153,14 @@ struct DevGroup {
     float4 *acc_s = nullptr;
     uint32_t *fstart = nullptr;   // F + 1 entries (F = kSlabs * total_cells)
     uint32_t *bstart = nullptr;   // start_blocks(F + 1) + 1 entries
-    // incremental ordering (the previous iteration's order repaired, see
-    // order_incremental); null unless incremental is set
-    bool incremental = false;
-    uint32_t *key_id = nullptr;    // by id: fine key at the last grid build (~0: none)
-    uint32_t *chg_bits = nullptr;  // by id: key changed, one bit each (bit i & 31 of word i >> 5)
-    uint32_t *keep_bits = nullptr; // by previous slot: key kept, one bit each
-    uint32_t *tile_cnt = nullptr;  // set bits of every tile of 2048: the changed tiles, then the kept ones
-    uint32_t *tile_pos = nullptr;  // their exclusive scan
-    uint32_t *ck[2] = {nullptr, nullptr}, *cv[2] = {nullptr, nullptr};   // changed (key, id), radix ping-pong
-    uint32_t *uk = nullptr, *uv = nullptr;   // kept (key, id) in previous order
-    uint32_t *split = nullptr;     // merge tile splits
-    uint32_t *counts = nullptr;    // [0] changed, [1] kept
-    uint32_t *scan_tmp_n = nullptr; // scan_tmp_elems(2 x tiles) entries
+    // the order by (key, id) of the last grid build
+    uint32_t *id_s = nullptr;      // ids (one of the arrays above)
+    uint32_t *key_s = nullptr;     // sorted keys (radix form only; else sorted_keys)
+    // counted form (a counting sort over the fine keys): counts per fine key
+    // (0 between builds), counts per tile of kCountTile keys, their exclusive
+    // sums when there are more than kScanTiles
+    bool counted = false;
+    uint32_t *cnt = nullptr, *tiles = nullptr, *tile_base = nullptr, *scan_tmp = nullptr;
     uint32_t *amax = nullptr;
     uint32_t *maxdisp = nullptr;
     int4 *work = nullptr;          // search queue {key slot, trial point}, N entries, then N uint2
@@ -264,8 +259,6 @@ enum CheckCode : uint32_t {
     kChkQueue = 4u,      // a search-queue slot outside [0, N)
     kChkEntry = 8u,      // a queued key slot outside [0, N)
     kChkTri = 16u,       // a candidate triangle outside the body's triangles
-    kChkMerge = 32u,     // a merge tile's split outside its lists
-    kChkCompact = 64u,   // a compaction position outside [0, N)
 };
 #ifdef FPPG_CHECKED
 __device__ bool fppg_check_failed(uint32_t code);
@@ -290,6 +283,13 @@ __device__ inline uint32_t grid_row_of(const AsmParams &A, int y, int z) {
 // the fine keys in blocks of 256 for building the start table (relax.cu)
 constexpr int kStartBlock = 256;
 constexpr int64_t start_blocks(int64_t f1) { return (f1 + kStartBlock - 1) / kStartBlock; }
+
+// tiles of the counts per fine key (relax.cu): up to kFewTiles of them every
+// block adds up the counts before its own tile itself (28 vectors a thread
+// at most, less than the launch that saves them); up to kScanTiles the tile
+// sums (64 a thread at most); above that their scan is read
+constexpr int kCountTile = 4096, kFewTiles = 8, kScanTiles = 16384;
+constexpr int64_t count_tiles(int64_t f1) { return (f1 + kCountTile - 1) / kCountTile; }
 
 struct GridPoint {
     float t[3];
@@ -420,10 +420,6 @@ int radix_sort_u32(uint32_t *keys[2], uint32_t *vals[2], bool iota_vals, int64_t
                    uint32_t *totals, cudaStream_t s);
 int radix_sort_u64(uint64_t *keys[2], uint32_t *vals[2], bool iota_vals, int64_t n, int bits, uint32_t *hist,
                    uint32_t *totals, cudaStream_t s);
-// the same with the count read from device memory (*n_dev <= n_max; the
-// launches and the histogram are sized for n_max; values given)
-int radix_sort_u32_dev(uint32_t *keys[2], uint32_t *vals[2], int64_t n_max, const uint32_t *n_dev, int bits,
-                       uint32_t *hist, uint32_t *totals, cudaStream_t s);
 int64_t radix_tiles(int64_t n);
 // radix passes for keys of `bits` bits and their digit width (*digit_bits);
 // the histogram holds kMaxDigits rows of radix_tiles(n)
@@ -434,12 +430,7 @@ constexpr int kMaxDigits = 256;
 void exclusive_scan_u32(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *total_dev, uint32_t *tmp,
                         int64_t tmp_elems, cudaStream_t s);
 int64_t scan_tmp_elems(int64_t n);
-// the same scan of counts that are cleared (set to 0) as they are read, so
-// the count array starts the next accumulation at zero
-void exclusive_scan_u32_clear(uint32_t *in, uint32_t *out, int64_t n, uint32_t *tmp, int64_t tmp_elems,
-                              cudaStream_t s);
-// kernel launches of exclusive_scan_u32 (no total) / _clear on n elements
+// kernel launches of exclusive_scan_u32 (no total) on n elements
 int scan_launches(int64_t n);
-int scan_clear_launches(int64_t n);
 
 } // namespace fppg

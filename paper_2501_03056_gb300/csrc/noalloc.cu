@@ -178,9 +178,9 @@ extern "C" int fppg_forces_static(const float *xyz_dev, const int32_t *cls_dev, 
     }
     if (n > 0) {
         k_pack_static<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(xyz_dev, cls_dev, n, d.pos, error);
-        const int buf = build_grid_dev(d, s);
+        build_grid_dev(d, s);
         forces_dev(d, 256, 0, s);
-        unpermute_dev(d, buf, s, acc_dev, nullptr, nullptr);
+        unpermute_dev(d, s, acc_dev, nullptr, nullptr);
         // a launch that failed to start is not reported by the synchronise
         // below: ask for it here
         const cudaError_t le = cudaGetLastError();

@@ -1,13 +1,12 @@
 // The relaxation hot path (Algorithm 1, Sec. 3.3) for a group of bodies.
 //
 // Per iteration, all bodies at once:
-//   k_keys          A1  cell key per particle (FP32 rule, no contraction);
-//                       zeroes the per-body amax / max-move
-//   radix sort      A2  stable (key, id) sort, 8-bit digits
-//   k_gather        A3  positions and constraint ids in key order
-//   start table     A3  the dense table of the first slot of every fine key,
-//                       from the sorted keys (block starts, then a binary
-//                       search per fine key inside its block's slots)
+//   grid build  A1-A3  cell key per particle (FP32 rule, no contraction), the
+//                      order by (key, id), positions and constraint ids in
+//                      that order, the dense table of the first slot of
+//                      every fine key: a counting sort (k_keys_count ..
+//                      k_rank_gather), or k_keys, a stable radix sort,
+//                      k_gather and the table from the sorted keys
 //   k_force         A4  Eq. 15 over the 3 x 3 rows of 3 cells around the
 //                       particle (each row is one contiguous slot range),
 //                       amax per body by a labelled warp max + atomicMax
@@ -108,6 +107,14 @@ __device__ inline void block_labelled_max(uint32_t *dst, int label, float v, int
     }
 }
 
+// the sort key: 8 (key_base + cell) + x-slab, with the grid row in the row order
+__device__ inline uint32_t fine_key_of(const AsmParams &A, float x, float y, float z) {
+    const int fx = fine_coord(x, A.ng_o[0], A.ng_inv, A.ng_n[0]);
+    const int cy = cell_coord(y, A.ng_o[1], A.ng_inv, A.ng_n[1]);
+    const int cz = cell_coord(z, A.ng_o[2], A.ng_inv, A.ng_n[2]);
+    return kSlabs * A.key_base + (uint32_t)fx + kSlabs * (uint32_t)A.ng_n[0] * grid_row(A, cy, cz);
+}
+
 // ---- A1 ----------------------------------------------------------------------
 __global__ void __launch_bounds__(TPB) k_keys(const float4 *__restrict__ pos, int64_t N,
                                               const AsmParams *__restrict__ P, uint32_t *__restrict__ key,
@@ -124,317 +131,278 @@ __global__ void __launch_bounds__(TPB) k_keys(const float4 *__restrict__ pos, in
     }
     if (i >= N) return;
     float4 p = pos[i];
-    const AsmParams &A = P[body_of(p.w)];
-    const int fx = fine_coord(p.x, A.ng_o[0], A.ng_inv, A.ng_n[0]);
-    const int cy = cell_coord(p.y, A.ng_o[1], A.ng_inv, A.ng_n[1]);
-    const int cz = cell_coord(p.z, A.ng_o[2], A.ng_inv, A.ng_n[2]);
-    key[i] = kSlabs * A.key_base + (uint32_t)fx +
-             kSlabs * (uint32_t)A.ng_n[0] * grid_row(A, cy, cz);
+    key[i] = fine_key_of(P[body_of(p.w)], p.x, p.y, p.z);
 }
 
-// ---- A1-A2, incremental form ---------------------------------------------------
-// A particle moves at most h / 16 per iteration, so from one grid build to
-// the next only a few per cent of the fine keys change (under 1 % once the
-// relaxation settles).  The incremental form keeps the last (key, id) order
-// and repairs it: the particles whose key changed are sorted alone (radix,
-// count on the device), the others keep their relative order, and the two
-// sorted lists are merged by (key, id).  The result is the one order by
-// (key, id), the same permutation as the stable sort of every key; with a
-// stale or foreign previous order every key counts as changed and the
-// repair is a full sort.
+// ---- A1-A3, counted form --------------------------------------------------------
+// A counting sort over the dense fine keys: the keys are counted as they are
+// made (every particle keeps its place in the arrival order of its key), the
+// counts' exclusive scan is the start table itself, the ids go to start +
+// arrival, and inside each key -- 2.2 particles on a lattice of spacing dx --
+// the gather ranks them by id.  The result is the one order by (key, id),
+// the same permutation as the stable sort of every key:
+//   k_keys_count   keys, arrival places, counts per key
+//   k_tile_sums    counts per tile of 4096 keys (more than kFewTiles tiles)
+//   k_count_starts the start table from the counts; each block adds up what
+//                  lies before it, so no block waits for another
+//   k_place        ids by key, in arrival order; the counts back to 0
+//   k_rank_gather  ids by (key, id); positions and constraints in that order
+// A key shared by m particles costs each of them m comparisons here, far
+// below what its pairs cost in the force pass.
 
-// The flags of both compactions are bits (bit i & 31 of word i >> 5: 1/32 of
-// the bytes of a flag array, small enough to stay in L2).  A block handles a
-// tile of kOrdTile items, kOrdItems per thread at stride TPB (item tile0 +
-// TPB j + thread): fewer, longer blocks than one item per thread, whose
-// launch cost would exceed the work of these light passes.  Word j of warp w
-// holds items tile0 + TPB j + 32 w + (0..31); every tile counts its set
-// bits.  One exclusive scan of the 2 x tiles counts (the changed tiles by
-// id, then the kept tiles by previous slot) places every tile; inside a tile
-// a bit's rank is the set bits of the earlier words and lanes.
-constexpr int kOrdItems = 8, kOrdTile = TPB * kOrdItems, kOrdWords = kOrdItems * (TPB / 32);
-static_assert(kOrdWords == 64, "tile_ranks scans two word counts per lane");
-static_assert(kOrdTile == 2048, "the order state (Group::alloc_order_state) has tiles of 2048");
+__global__ void __launch_bounds__(TPB) k_keys_count(const float4 *__restrict__ pos, int64_t N,
+                                                    const AsmParams *__restrict__ P, uint32_t *__restrict__ key,
+                                                    uint32_t *__restrict__ place, uint32_t *__restrict__ cnt) {
+    const int64_t i = (int64_t)blockIdx.x * TPB + threadIdx.x;
+    if (i >= N) return;
+    const float4 p = pos[i];
+    const uint32_t k = fine_key_of(P[body_of(p.w)], p.x, p.y, p.z);
+    key[i] = k;
+    place[i] = atomicAdd(cnt + k, 1u);
+}
 
-// the word counts of a tile, summed: its number of set bits
-__device__ inline void store_tile_count(uint32_t cnt, int64_t N, uint32_t *__restrict__ tile_cnt, uint32_t *wcnt) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) wcnt[w] = cnt;
+// the counts of a tile of kCountTile keys as 16-byte vectors, vector q of a
+// thread at keys f0 + 4 (q TPB + thread) .. + 3 (0 past F1)
+constexpr int kCountVec = kCountTile / (4 * TPB);
+
+__device__ inline uint4 load_counts(const uint32_t *__restrict__ cnt, int64_t f, int64_t F1) {
+    if (f + 4 <= F1) return *reinterpret_cast<const uint4 *>(cnt + f);
+    return make_uint4(f < F1 ? cnt[f] : 0u, f + 1 < F1 ? cnt[f + 1] : 0u, f + 2 < F1 ? cnt[f + 2] : 0u, 0u);
+}
+
+__device__ inline uint32_t sum4(const uint4 &a) { return a.x + a.y + a.z + a.w; }
+
+__global__ void __launch_bounds__(TPB) k_tile_sums(const uint32_t *__restrict__ cnt, int64_t F1,
+                                                   uint32_t *__restrict__ tiles) {
+    __shared__ uint32_t wsum[TPB / 32];
+    const int64_t f0 = (int64_t)blockIdx.x * kCountTile;
+    uint32_t v = 0u;
+#pragma unroll
+    for (int q = 0; q < kCountVec; q++) v += sum4(load_counts(cnt, f0 + 4 * (q * TPB + (int)threadIdx.x), F1));
+    v = __reduce_add_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = v;
     __syncthreads();
-    if (threadIdx.x == 0 && (int64_t)blockIdx.x * kOrdTile < N) {
-        uint32_t t = 0;
-        for (int q = 0; q < TPB / 32; q++) t += wcnt[q];
-        tile_cnt[blockIdx.x] = t;
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int q = 1; q < TPB / 32; q++) v += wsum[q];
+        tiles[blockIdx.x] = v;
     }
 }
 
-// key of every particle (the rule of k_keys), compared with the key it had
-// at the last grid build: the changed bits by id and their tile counts;
-// key_id updated
-__global__ void __launch_bounds__(TPB) k_keys_inc(const float4 *__restrict__ pos, int64_t N,
-                                                  const AsmParams *__restrict__ P, uint32_t *__restrict__ key_id,
-                                                  uint32_t *__restrict__ chg_bits, uint32_t *__restrict__ tile_cnt,
-                                                  uint32_t *__restrict__ amax, uint32_t *__restrict__ maxdisp, int B,
-                                                  uint32_t *__restrict__ work_count) {
-    __shared__ uint32_t wcnt[TPB / 32];
-    const int64_t g = (int64_t)blockIdx.x * TPB + threadIdx.x;
-    if (g < B) {
-        amax[g] = 0u;
-        maxdisp[g] = 0u;
-    }
-    if (g == 0) {
-        work_count[0] = 0u;
-        work_count[1] = 0u;
-    }
-    const int64_t i0 = (int64_t)blockIdx.x * kOrdTile + threadIdx.x;
-    float4 p[kOrdItems];
-    uint32_t old[kOrdItems];
-#pragma unroll
-    for (int j = 0; j < kOrdItems; j++) {
-        const int64_t i = i0 + (int64_t)j * TPB;
-        p[j] = i < N ? pos[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-        old[j] = i < N ? key_id[i] : 0u;
-    }
-    uint32_t cnt = 0;
-#pragma unroll
-    for (int j = 0; j < kOrdItems; j++) {
-        const int64_t i = i0 + (int64_t)j * TPB;
-        bool changed = false;
-        if (i < N) {
-            const AsmParams &A = P[body_of(p[j].w)];
-            const int fx = fine_coord(p[j].x, A.ng_o[0], A.ng_inv, A.ng_n[0]);
-            const int cy = cell_coord(p[j].y, A.ng_o[1], A.ng_inv, A.ng_n[1]);
-            const int cz = cell_coord(p[j].z, A.ng_o[2], A.ng_inv, A.ng_n[2]);
-            const uint32_t k = kSlabs * A.key_base + (uint32_t)fx +
-                               kSlabs * (uint32_t)A.ng_n[0] * grid_row(A, cy, cz);
-            changed = k != old[j];
-            if (changed) key_id[i] = k;
-        }
-        const uint32_t word = __ballot_sync(~0u, changed);
-        if ((threadIdx.x & 31) == 0 && i < N) chg_bits[i >> 5] = word;   // i is a multiple of 32 in lane 0
-        cnt += __popc(word);
-    }
-    store_tile_count(cnt, N, tile_cnt, wcnt);
-}
-
-// the kept bits by previous slot (the particle in slot k kept its key) and
-// their tile counts
-__global__ void __launch_bounds__(TPB) k_keep_bits(const uint32_t *__restrict__ prev_id,
-                                                   const uint32_t *__restrict__ chg_bits, int64_t N,
-                                                   uint32_t *__restrict__ keep_bits,
-                                                   uint32_t *__restrict__ tile_cnt) {
-    __shared__ uint32_t wcnt[TPB / 32];
-    const int64_t k0 = (int64_t)blockIdx.x * kOrdTile + threadIdx.x;
-    uint32_t id[kOrdItems];
-#pragma unroll
-    for (int j = 0; j < kOrdItems; j++) {
-        const int64_t k = k0 + (int64_t)j * TPB;
-        id[j] = k < N ? prev_id[k] : 0u;
-    }
-    uint32_t cnt = 0;
-#pragma unroll
-    for (int j = 0; j < kOrdItems; j++) {
-        const int64_t k = k0 + (int64_t)j * TPB;
-        const bool kept = k < N && FPPG_CHECK(id[j] < N, kChkCompact) &&
-                          !((chg_bits[id[j] >> 5] >> (id[j] & 31)) & 1u);
-        const uint32_t word = __ballot_sync(~0u, kept);
-        if ((threadIdx.x & 31) == 0 && k < N) keep_bits[k >> 5] = word;
-        cnt += __popc(word);
-    }
-    store_tile_count(cnt, N, tile_cnt, wcnt);
-}
-
-// this thread's words of a tile (word j of its warp) and, for each, the rank
-// of its own bit among the tile's set bits in item order (j, then warp, then
-// lane); sc: kOrdWords shared words
-__device__ inline void tile_ranks(const uint32_t *__restrict__ bits, int64_t tile0, int64_t N,
-                                  uint32_t (&word)[kOrdItems], uint32_t (&rank)[kOrdItems], uint32_t *sc) {
+// fstart[f] = the number of particles with a fine key below f, for f in
+// [0, F] (cnt: F1 = F + 1 entries, the last 0).  One tile per block, which
+// adds up what lies before it: the tile sums (scanned = 0), one entry of
+// their exclusive scan (scanned = 1), or with tiles null the counts
+// themselves.  Also resets the per-body maxima and the search queue.
+__global__ void __launch_bounds__(TPB) k_count_starts(const uint32_t *__restrict__ cnt,
+                                                      const uint32_t *__restrict__ tiles, int scanned, int64_t F1,
+                                                      uint32_t *__restrict__ fstart, uint32_t *__restrict__ amax,
+                                                      uint32_t *__restrict__ maxdisp, int B,
+                                                      uint32_t *__restrict__ work_count) {
+    constexpr int kWarps = TPB / 32;
+    static_assert(kCountVec * kWarps == 32, "one lane per (vector, warp) sum");
+    __shared__ uint32_t s_sum[32], s_pre[kWarps];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int j = 0; j < kOrdItems; j++) {
-        const int64_t i0 = tile0 + (int64_t)j * TPB + 32 * w;
-        word[j] = i0 < N ? bits[i0 >> 5] : 0u;
+    for (int64_t b = (int64_t)blockIdx.x * TPB + threadIdx.x; b < B; b += (int64_t)gridDim.x * TPB) {
+        amax[b] = 0u;
+        maxdisp[b] = 0u;
     }
-    if (lane == 0)
+    if (blockIdx.x == 0 && threadIdx.x < 2) work_count[threadIdx.x] = 0u;
+    const int64_t f0 = (int64_t)blockIdx.x * kCountTile;
+    uint4 v[kCountVec];
 #pragma unroll
-        for (int j = 0; j < kOrdItems; j++) sc[j * (TPB / 32) + w] = __popc(word[j]);
-    __syncthreads();
-    if (w == 0) {
-        // exclusive scan of the 64 word counts, two per lane
-        const uint32_t a = sc[2 * lane], b = sc[2 * lane + 1];
-        uint32_t v = a + b;
+    for (int q = 0; q < kCountVec; q++) v[q] = load_counts(cnt, f0 + 4 * (q * TPB + (int)threadIdx.x), F1);
+    uint32_t pre = 0u;   // this thread's share of what lies before the tile
+    if (!tiles) {
+        for (int64_t f = 4 * (int64_t)threadIdx.x; f < f0; f += 4 * TPB)
+            pre += sum4(*reinterpret_cast<const uint4 *>(cnt + f));
+    } else if (scanned) {
+        if (threadIdx.x == 0) pre = tiles[blockIdx.x];
+    } else {
+#pragma unroll 4
+        for (uint32_t t = threadIdx.x; t < blockIdx.x; t += TPB) pre += tiles[t];
+    }
+    pre = __reduce_add_sync(0xffffffffu, pre);
+    if (lane == 0) s_pre[w] = pre;
+    // inclusive sums over the warp of every vector
+    uint32_t inc[kCountVec];
+#pragma unroll
+    for (int q = 0; q < kCountVec; q++) {
+        inc[q] = sum4(v[q]);
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(~0u, v, o);
-            if (lane >= o) v += t;
+            const uint32_t t = __shfl_up_sync(0xffffffffu, inc[q], o);
+            if (lane >= o) inc[q] += t;
         }
-        const uint32_t ex = v - a - b;
-        sc[2 * lane] = ex;
-        sc[2 * lane + 1] = ex + a;
+        if (lane == 31) s_sum[q * kWarps + w] = inc[q];
     }
     __syncthreads();
-    const uint32_t lt = lanemask_lt();
+    // every warp scans the 32 (vector, warp) sums for itself
+    uint32_t all = s_sum[lane];
+    const uint32_t own = all;
 #pragma unroll
-    for (int j = 0; j < kOrdItems; j++) rank[j] = sc[j * (TPB / 32) + w] + __popc(word[j] & lt);
-}
-
-// the changed particles, in id order: (key, id) at their positions
-__global__ void __launch_bounds__(TPB) k_compact_changed(const uint32_t *__restrict__ chg_bits,
-                                                         const uint32_t *__restrict__ tile_pos,
-                                                         const uint32_t *__restrict__ key_id, int64_t N,
-                                                         uint32_t *__restrict__ ck, uint32_t *__restrict__ cv) {
-    __shared__ uint32_t sc[kOrdWords];
-    const int64_t tile0 = (int64_t)blockIdx.x * kOrdTile;
-    uint32_t word[kOrdItems], rank[kOrdItems];
-    tile_ranks(chg_bits, tile0, N, word, rank, sc);
-    const uint32_t p0 = tile_pos[blockIdx.x];
-    const int lane = threadIdx.x & 31;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, all, o);
+        if (lane >= o) all += t;
+    }
+    all -= own;
+    uint32_t base = 0u;
 #pragma unroll
-    for (int j = 0; j < kOrdItems; j++) {
-        if (!((word[j] >> lane) & 1u)) continue;
-        const int64_t i = tile0 + (int64_t)j * TPB + threadIdx.x;
-        const uint32_t p = p0 + rank[j];
-        if (!FPPG_CHECK(p < N, kChkCompact)) continue;
-        ck[p] = key_id[i];
-        cv[p] = (uint32_t)i;
+    for (int q = 0; q < kWarps; q++) base += s_pre[q];
+#pragma unroll
+    for (int q = 0; q < kCountVec; q++) {
+        const int64_t f = f0 + 4 * (q * TPB + (int)threadIdx.x);
+        uint32_t r = base + __shfl_sync(0xffffffffu, all, q * kWarps + w) + inc[q] - sum4(v[q]);
+        uint4 o;
+        o.x = r;
+        o.y = r += v[q].x;
+        o.z = r += v[q].y;
+        o.w = r += v[q].z;
+        if (f + 4 <= F1) {
+            *reinterpret_cast<uint4 *>(fstart + f) = o;
+        } else {
+            if (f < F1) fstart[f] = o.x;
+            if (f + 1 < F1) fstart[f + 1] = o.y;
+            if (f + 2 < F1) fstart[f + 2] = o.z;
+        }
     }
 }
 
-// the kept slots of the previous order, compacted (still sorted); the kept
-// tiles' positions follow the changed tiles' (nb tiles of each), so they
-// start at the number of changed particles, tile_pos[nb]
-__global__ void __launch_bounds__(TPB) k_compact_kept(const uint32_t *__restrict__ keep_bits,
-                                                      const uint32_t *__restrict__ tile_pos, int64_t nb,
-                                                      const uint32_t *__restrict__ prev_key,
-                                                      const uint32_t *__restrict__ prev_id, int64_t N,
-                                                      uint32_t *__restrict__ uk, uint32_t *__restrict__ uv) {
-    __shared__ uint32_t sc[kOrdWords];
-    const int64_t tile0 = (int64_t)blockIdx.x * kOrdTile;
-    uint32_t word[kOrdItems], rank[kOrdItems];
-    tile_ranks(keep_bits, tile0, N, word, rank, sc);
-    const uint32_t p0 = tile_pos[nb + blockIdx.x] - tile_pos[nb];
-    const int lane = threadIdx.x & 31;
+// ids by key, in arrival order; the counts set back to 0 for the next build
+__global__ void __launch_bounds__(TPB) k_place(const uint32_t *__restrict__ key, const uint32_t *__restrict__ place,
+                                               const uint32_t *__restrict__ fstart, int64_t N,
+                                               uint32_t *__restrict__ id_a, uint32_t *__restrict__ cnt, int64_t F1) {
+    const int64_t i = (int64_t)blockIdx.x * TPB + threadIdx.x;
+    const int64_t nv = F1 / 4;
+    for (int64_t f = i; f < nv; f += (int64_t)gridDim.x * TPB)
+        reinterpret_cast<uint4 *>(cnt)[f] = make_uint4(0u, 0u, 0u, 0u);
+    if (i < F1 - 4 * nv) cnt[4 * nv + i] = 0u;
+    if (i >= N) return;
+    const uint32_t k = fstart[key[i]] + place[i];
+    if (FPPG_CHECK(k < N, kChkGather)) id_a[k] = (uint32_t)i;
+}
+
+// One particle at slot k of the key order, written on its own: position,
+// slot-pair halves, constraint, id
+__device__ inline void put_slot(uint32_t k, const float4 &q, uint32_t id, int32_t c, int64_t N,
+                                float4 *__restrict__ pos_s, float4 *__restrict__ pos_p, uint32_t *__restrict__ id_s,
+                                int32_t *__restrict__ cons_s) {
+    pos_s[k] = q;
+    id_s[k] = id;
+    cons_s[k] = c;
+    float *a = reinterpret_cast<float *>(pos_p + (k >> 1)) + (k & 1u);
+    float *b = reinterpret_cast<float *>(pos_p + (N + 1) / 2 + (k >> 1)) + (k & 1u);
+    a[0] = q.x;
+    a[2] = q.y;
+    b[0] = q.z;
+    b[2] = q.w;
+}
+
+// A block takes kGatherItems TPB consecutive places of the arrival order.
+// Each particle is ranked by id among those of its key and goes to start +
+// rank: within the block's slots through shared memory (stored coalesced),
+// else -- a key that crosses the block's edge -- straight to its slot.  Bound
+// by memory: 68 B per particle, with a chain of four dependent loads (id,
+// position, start, the key's ids).  Two particles per thread keep more of
+// them in flight once the blocks fill the chip (18.9 M particles: 278 -> 250
+// us, 7.1 M: 107 -> 97 us); below that one (42 k: 3.1 against 3.9 us).
+constexpr int64_t kGatherTwoMinN = 1 << 20;
+
+template <int kGatherItems>
+__global__ void __launch_bounds__(TPB) k_rank_gather(const uint32_t *__restrict__ id_a,
+                                                     const AsmParams *__restrict__ P,
+                                                     const uint32_t *__restrict__ fstart,
+                                                     const float4 *__restrict__ pos, const int32_t *__restrict__ cons,
+                                                     int64_t N, float4 *__restrict__ pos_s, float4 *__restrict__ pos_p,
+                                                     uint32_t *__restrict__ id_s, int32_t *__restrict__ cons_s) {
+    constexpr int kGatherTile = kGatherItems * TPB;
+    __shared__ float4 s_pos[kGatherTile];
+    __shared__ uint32_t s_id[kGatherTile];
+    __shared__ int32_t s_cons[kGatherTile];
+    constexpr uint32_t kNone = 0xffffffffu;
+    const int64_t k0 = (int64_t)blockIdx.x * kGatherTile;
+    uint32_t id[kGatherItems], s[kGatherItems], e[kGatherItems];
+    float4 q[kGatherItems];
+    int32_t c[kGatherItems];
 #pragma unroll
-    for (int j = 0; j < kOrdItems; j++) {
-        if (!((word[j] >> lane) & 1u)) continue;
-        const int64_t k = tile0 + (int64_t)j * TPB + threadIdx.x;
-        const uint32_t p = p0 + rank[j];
-        if (!FPPG_CHECK(p < N, kChkCompact)) continue;
-        uk[p] = prev_key[k];
-        uv[p] = prev_id[k];
+    for (int u = 0; u < kGatherItems; u++) {
+        const int64_t k = k0 + u * TPB + threadIdx.x;
+        s_id[u * TPB + threadIdx.x] = kNone;
+        id[u] = k < N ? id_a[k] : kNone;
+        if (k < N && !FPPG_CHECK(id[u] < N, kChkGather)) id[u] = kNone;
     }
-}
-
-// counts[0] = changed particles, counts[1] = kept slots, from the scan of
-// the 2 nb tile counts
-__global__ void k_order_counts(const uint32_t *__restrict__ tile_cnt, const uint32_t *__restrict__ tile_pos,
-                               int64_t nb, uint32_t *__restrict__ counts) {
-    const uint32_t c = tile_pos[nb];
-    counts[0] = c;
-    counts[1] = tile_pos[2 * nb - 1] + tile_cnt[2 * nb - 1] - c;
-}
-
-// merge of the kept list u (U items) and the sorted changed list c (C
-// items), U + C = N, in (key, id) order; ids are distinct, so the order is
-// strict and the merge unique
-constexpr int kMergeThreads = 256, kMergeItems = 8, kMergeTile = kMergeThreads * kMergeItems;
-
-__device__ inline bool kv_less(uint32_t ka, uint32_t ia, uint32_t kb, uint32_t ib) {
-    return ka < kb || (ka == kb && ia < ib);
-}
-
-// split[b]: how many u items the first min(b tile, N) outputs take
-__global__ void k_merge_splits(const uint32_t *__restrict__ uk, const uint32_t *__restrict__ uv,
-                               const uint32_t *__restrict__ ck, const uint32_t *__restrict__ cv,
-                               const uint32_t *__restrict__ counts, int64_t N, int nblk,
-                               uint32_t *__restrict__ split) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b > nblk) return;
-    const int64_t C = counts[0], U = counts[1];
-    const int64_t d = min((int64_t)b * kMergeTile, N);
-    int64_t lo = max((int64_t)0, d - C), hi = min(d, U);
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        const int64_t j = d - 1 - mid;
-        if (kv_less(uk[mid], uv[mid], ck[j], cv[j])) lo = mid + 1;
-        else hi = mid;
-    }
-    split[b] = (uint32_t)lo;
-}
-
-// one tile of kMergeTile outputs per block: its u and c items staged in
-// shared memory, then kMergeItems outputs per thread
-__global__ void __launch_bounds__(kMergeThreads) k_merge(const uint32_t *__restrict__ uk,
-                                                         const uint32_t *__restrict__ uv,
-                                                         const uint32_t *__restrict__ ck,
-                                                         const uint32_t *__restrict__ cv,
-                                                         const uint32_t *__restrict__ split, int64_t N,
-                                                         uint32_t *__restrict__ out_key,
-                                                         uint32_t *__restrict__ out_id) {
-    __shared__ uint32_t sk[kMergeTile], si[kMergeTile];
-    const int64_t d0 = (int64_t)blockIdx.x * kMergeTile, d1 = min(d0 + kMergeTile, N);
-    const int64_t i0 = split[blockIdx.x], i1 = split[blockIdx.x + 1];
-    const int64_t j0 = d0 - i0, j1 = d1 - i1;
-    // (nu + nc = d1 - d0 <= kMergeTile: the staging fits when both are >= 0)
-    if (!FPPG_CHECK(i0 <= i1 && j0 <= j1 && j0 >= 0, kChkMerge)) return;
-    const int nu = (int)(i1 - i0), nc = (int)(j1 - j0), n = nu + nc;
-    {
-        // all loads of a thread issued before the first store (one round trip)
-        uint32_t lk[kMergeItems], li[kMergeItems];
 #pragma unroll
-        for (int r = 0; r < kMergeItems; r++) {
-            const int q = (int)threadIdx.x + r * kMergeThreads;
-            lk[r] = li[r] = 0u;
-            if (q < nu) {
-                lk[r] = uk[i0 + q];
-                li[r] = uv[i0 + q];
-            } else if (q < n) {
-                lk[r] = ck[j0 + q - nu];
-                li[r] = cv[j0 + q - nu];
-            }
+    for (int u = 0; u < kGatherItems; u++)
+        if (id[u] != kNone) {
+            q[u] = pos[id[u]];
+            c[u] = cons[id[u]];
         }
 #pragma unroll
-        for (int r = 0; r < kMergeItems; r++) {
-            const int q = (int)threadIdx.x + r * kMergeThreads;
-            if (q < n) {
-                sk[q] = lk[r];
-                si[q] = li[r];
-            }
+    for (int u = 0; u < kGatherItems; u++)
+        if (id[u] != kNone) {
+            // (the key again: cheaper than a gather of the stored one)
+            const uint32_t f = fine_key_of(P[body_of(q[u].w)], q[u].x, q[u].y, q[u].z);
+            s[u] = fstart[f];
+            e[u] = fstart[f + 1u];
+        }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kGatherItems; u++) {
+        if (id[u] == kNone) continue;
+        uint32_t slot = s[u];
+        if (e[u] - s[u] > 1u && FPPG_CHECK(s[u] <= e[u] && e[u] <= N, kChkGather))
+            for (uint32_t j = s[u]; j < e[u]; j++) slot += id_a[j] < id[u] ? 1u : 0u;
+        const int64_t l = (int64_t)slot - k0;
+        if (l >= 0 && l < kGatherTile) {
+            s_pos[l] = q[u];
+            s_id[l] = id[u];
+            s_cons[l] = c[u];
+        } else {
+            put_slot(slot, q[u], id[u], c[u], N, pos_s, pos_p, id_s, cons_s);
         }
     }
     __syncthreads();
-    const int dt = min((int)threadIdx.x * kMergeItems, n);
-    int lo = max(0, dt - nc), hi = min(dt, nu);
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        const int j = dt - 1 - mid;
-        if (kv_less(sk[mid], si[mid], sk[nu + j], si[nu + j])) lo = mid + 1;
-        else hi = mid;
-    }
-    int i = lo, j = dt - lo;
-    uint32_t rk[kMergeItems], ri[kMergeItems];
 #pragma unroll
-    for (int q = 0; q < kMergeItems; q++) {
-        if (dt + q < n) {
-            const bool take_u = j >= nc || (i < nu && kv_less(sk[i], si[i], sk[nu + j], si[nu + j]));
-            const int src = take_u ? i++ : nu + j++;
-            rk[q] = sk[src];
-            ri[q] = si[src];
+    for (int u = 0; u < kGatherItems; u++) {
+        const int l = u * TPB + (int)threadIdx.x;
+        const int64_t k = k0 + l;
+        const uint32_t mine = s_id[l];
+        // the padding of an odd count: a finite point of no class (its thread
+        // is in the last block: an odd N is no multiple of the tile)
+        const bool pad = k == N && (N & 1);
+        const bool here = mine != kNone || pad;
+        const float4 v = mine != kNone ? s_pos[l] : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (mine != kNone) {
+            pos_s[k] = v;
+            id_s[k] = mine;
+            cons_s[k] = s_cons[l];
+        }
+        // slot pairs: the two slots sit in neighbouring lanes, which swap
+        // their points and write one half each (as in k_gather); a slot whose
+        // partner is written elsewhere writes its own four values
+        const float ox = __shfl_xor_sync(0xffffffffu, v.x, 1), oy = __shfl_xor_sync(0xffffffffu, v.y, 1);
+        const float oz = __shfl_xor_sync(0xffffffffu, v.z, 1), ow = __shfl_xor_sync(0xffffffffu, v.w, 1);
+        const bool both = __shfl_xor_sync(0xffffffffu, here ? 1 : 0, 1) != 0 && here;
+        if (both) {
+            if ((k & 1) == 0) pos_p[k >> 1] = make_float4(v.x, ox, v.y, oy);
+            else pos_p[(N + 1) / 2 + (k >> 1)] = make_float4(oz, v.z, ow, v.w);
+        } else if (here) {
+            float *a = reinterpret_cast<float *>(pos_p + (k >> 1)) + (k & 1);
+            float *b = reinterpret_cast<float *>(pos_p + (N + 1) / 2 + (k >> 1)) + (k & 1);
+            a[0] = v.x;
+            a[2] = v.y;
+            b[0] = v.z;
+            b[2] = v.w;
         }
     }
-    // the tile's outputs back through shared memory, then stored coalesced
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < kMergeItems; q++)
-        if (dt + q < n) {
-            sk[dt + q] = rk[q];
-            si[dt + q] = ri[q];
-        }
-    __syncthreads();
-    for (int q = threadIdx.x; q < n; q += kMergeThreads) {
-        out_key[d0 + q] = sk[q];
-        out_id[d0 + q] = si[q];
-    }
+}
+
+// the sorted keys (diagnostics)
+__global__ void __launch_bounds__(TPB) k_sorted_keys(const uint32_t *__restrict__ id_s,
+                                                     const uint32_t *__restrict__ key, int64_t N,
+                                                     uint32_t *__restrict__ out) {
+    const int64_t k = (int64_t)blockIdx.x * TPB + threadIdx.x;
+    if (k < N) out[k] = key[id_s[k]];
 }
 
 // ---- A3 ----------------------------------------------------------------------
@@ -1694,54 +1662,63 @@ __global__ void k_class_sums(const float4 *__restrict__ pos_s, const float *__re
 } // namespace
 
 // ---- host driver ----------------------------------------------------------------
-// A1-A2 of the incremental form; the order ends in key[0] / id[0], which is
-// also the previous order it starts from
-static void order_incremental(DevGroup &d, cudaStream_t s) {
-    const int64_t N = d.N;
-    const int64_t nb = nblocks(N, kOrdTile);
-    k_keys_inc<<<std::max<unsigned>(nb, nblocks(d.B)), TPB, 0, s>>>(d.pos, N, d.params, d.key_id, d.chg_bits,
-                                                                     d.tile_cnt, d.amax, d.maxdisp, d.B,
-                                                                     d.work_count);
-    if (N == 0) return;
-    k_keep_bits<<<nb, TPB, 0, s>>>(d.id[0], d.chg_bits, N, d.keep_bits, d.tile_cnt + nb);
-    exclusive_scan_u32(d.tile_cnt, d.tile_pos, 2 * nb, nullptr, d.scan_tmp_n, scan_tmp_elems(2 * nb), s);
-    k_order_counts<<<1, 1, 0, s>>>(d.tile_cnt, d.tile_pos, nb, d.counts);
-    k_compact_changed<<<nb, TPB, 0, s>>>(d.chg_bits, d.tile_pos, d.key_id, N, d.ck[0], d.cv[0]);
-    const int cb = radix_sort_u32_dev(d.ck, d.cv, N, d.counts, d.key_bits, d.hist, d.totals, s);
-    k_compact_kept<<<nb, TPB, 0, s>>>(d.keep_bits, d.tile_pos, nb, d.key[0], d.id[0], N, d.uk, d.uv);
-    const int nblk = (int)((N + kMergeTile - 1) / kMergeTile);
-    k_merge_splits<<<(nblk + 1 + 255) / 256, 256, 0, s>>>(d.uk, d.uv, d.ck[cb], d.cv[cb], d.counts, N, nblk,
-                                                          d.split);
-    k_merge<<<nblk, kMergeThreads, 0, s>>>(d.uk, d.uv, d.ck[cb], d.cv[cb], d.split, N, d.key[0], d.id[0]);
+// A1-A3 of the counted form: key[0] the keys and id[0] the arrival places by
+// id, id[1] the ids in arrival order, key[1] the ids in key order
+static void build_counted(DevGroup &d, cudaStream_t s) {
+    const int64_t F1 = kSlabs * d.total_cells + 1, nt = count_tiles(F1);
+    k_keys_count<<<nblocks(d.N), TPB, 0, s>>>(d.pos, d.N, d.params, d.key[0], d.id[0], d.cnt);
+    const uint32_t *tiles = nullptr;
+    if (nt > kFewTiles) {
+        k_tile_sums<<<(unsigned)nt, TPB, 0, s>>>(d.cnt, F1, d.tiles);
+        tiles = d.tiles;
+    }
+    if (nt > kScanTiles) {
+        exclusive_scan_u32(d.tiles, d.tile_base, nt, nullptr, d.scan_tmp, scan_tmp_elems(nt), s);
+        tiles = d.tile_base;
+    }
+    k_count_starts<<<(unsigned)nt, TPB, 0, s>>>(d.cnt, tiles, nt > kScanTiles, F1, d.fstart, d.amax, d.maxdisp, d.B,
+                                                d.work_count);
+    d.id_s = d.key[1];
+    k_place<<<nblocks(d.N), TPB, 0, s>>>(d.key[0], d.id[0], d.fstart, d.N, d.id[1], d.cnt, F1);
+    if (d.N < kGatherTwoMinN)
+        k_rank_gather<1><<<nblocks(d.N), TPB, 0, s>>>(d.id[1], d.params, d.fstart, d.pos, d.cons, d.N, d.pos_s,
+                                                      d.pos_p, d.id_s, d.cons_s);
+    else
+        k_rank_gather<2><<<nblocks(d.N, 2 * TPB), TPB, 0, s>>>(d.id[1], d.params, d.fstart, d.pos, d.cons, d.N,
+                                                               d.pos_s, d.pos_p, d.id_s, d.cons_s);
 }
 
-int build_grid_dev(DevGroup &d, cudaStream_t s) {
-    int buf = 0;
-    if (d.incremental) {
-        order_incremental(d, s);
-    } else {
-        k_keys<<<nblocks(std::max<int64_t>(d.N, d.B)), TPB, 0, s>>>(d.pos, d.N, d.params, d.key[0], d.amax,
-                                                                     d.maxdisp, d.B, d.work_count);
-        buf = radix_sort_u32(d.key, d.id, true, d.N, d.key_bits, d.hist, d.totals, s);
+void build_grid_dev(DevGroup &d, cudaStream_t s) {
+    if (d.counted) {
+        build_counted(d, s);
+        return;
     }
-    k_gather<<<nblocks(d.N), TPB, 0, s>>>(d.id[buf], d.pos, d.N, d.pos_s, d.pos_p, d.cons, d.cons_s);
+    k_keys<<<nblocks(std::max<int64_t>(d.N, d.B)), TPB, 0, s>>>(d.pos, d.N, d.params, d.key[0], d.amax, d.maxdisp, d.B,
+                                                                 d.work_count);
+    const int buf = radix_sort_u32(d.key, d.id, true, d.N, d.key_bits, d.hist, d.totals, s);
+    d.id_s = d.id[buf];
+    d.key_s = d.key[buf];
+    k_gather<<<nblocks(d.N), TPB, 0, s>>>(d.id_s, d.pos, d.N, d.pos_s, d.pos_p, d.cons, d.cons_s);
     // the start table from the sorted keys
     const int64_t F1 = kSlabs * d.total_cells + 1;
     const int64_t nblk = start_blocks(F1);
-    k_key_block_starts<<<nblocks(d.N + 1), TPB, 0, s>>>(d.key[buf], d.N, nblk, d.bstart);
-    k_fine_starts<<<(unsigned)nblk, kStartBlock, 0, s>>>(d.key[buf], d.bstart, F1, d.fstart);
-    return buf;
+    k_key_block_starts<<<nblocks(d.N + 1), TPB, 0, s>>>(d.key_s, d.N, nblk, d.bstart);
+    k_fine_starts<<<(unsigned)nblk, kStartBlock, 0, s>>>(d.key_s, d.bstart, F1, d.fstart);
+}
+
+const uint32_t *sorted_keys(DevGroup &d, cudaStream_t s) {
+    if (!d.counted) return d.key_s;
+    k_sorted_keys<<<nblocks(d.N), TPB, 0, s>>>(d.id_s, d.key[0], d.N, d.id[1]);   // the arrival order is used up
+    return d.id[1];
 }
 
 int grid_kernels(const DevGroup &d) {
-    const int tail = 3;    // gather, block starts, fine-key starts
-    if (!d.incremental) return 1 + 3 * d.passes + tail;
-    // keys, keep bits, the scan of the tile counts and the counts, 2
-    // compactions, the changed list's radix passes, merge splits and merge
-    return 2 + scan_launches(2 * (int64_t)nblocks(d.N, kOrdTile)) + 1 + 2 + 3 * d.passes + 2 + tail;
+    if (!d.counted) return 1 + 3 * d.passes + 3;   // keys, radix passes, gather, block starts, fine-key starts
+    const int64_t nt = count_tiles(kSlabs * d.total_cells + 1);
+    return 4 + (nt > kFewTiles ? 1 : 0) + (nt > kScanTiles ? scan_launches(nt) : 0);
 }
 
-int build_grid(Group &g, cudaStream_t s) { return build_grid_dev(g.d, s); }
+void build_grid(Group &g, cudaStream_t s) { build_grid_dev(g.d, s); }
 
 void forces_dev(DevGroup &d, int tb, int variant, cudaStream_t s, int32_t *count_s, int32_t *tested_s) {
     const unsigned nbk = (unsigned)std::max<int64_t>((d.N + tb - 1) / tb, 1);
@@ -1784,10 +1761,9 @@ void iterate(Group &g, cudaStream_t s, bool energy_mode, int32_t *count_dbg) {
     if (timed) cudaStreamIsCapturing(s, &cap);
     const unsigned flags = cap == cudaStreamCaptureStatusActive ? cudaEventRecordExternal : 0u;
     if (timed) cudaEventRecordWithFlags(g.ev[g.ev_used], s, flags);
-    int buf;
     {
         NvtxRange r("A1-A3 grid");
-        buf = build_grid(g, s);
+        build_grid(g, s);
     }
     if (timed) cudaEventRecordWithFlags(g.ev[g.ev_used + 1], s, flags);
     {
@@ -1797,15 +1773,15 @@ void iterate(Group &g, cudaStream_t s, bool energy_mode, int32_t *count_dbg) {
     }
     if (timed) cudaEventRecordWithFlags(g.ev[g.ev_used + 2], s, flags);
     NvtxRange r("A5-A6 step and search");
-    k_step<<<nblocks(d.N), TPB, 0, s>>>(d.pos_s, d.acc_s, d.id[buf], d.N, d.params, d.amax, d.pos, d.cons, g.mesh,
+    k_step<<<nblocks(d.N), TPB, 0, s>>>(d.pos_s, d.acc_s, d.id_s, d.N, d.params, d.amax, d.pos, d.cons, g.mesh,
                                          d.maxdisp, d.work, queue_ranges(d), d.work_count, d.cert, d.cons_s);
     if (timed) cudaEventRecordWithFlags(g.ev[g.ev_used + 3], s, flags);
     if (g.search_thread)
-        k_search_thread<<<g.search_blocks, TPB, 0, s>>>(d.pos_s, d.id[buf], d.params, d.pos, d.cons, g.mesh,
+        k_search_thread<<<g.search_blocks, TPB, 0, s>>>(d.pos_s, d.id_s, d.params, d.pos, d.cons, g.mesh,
                                                         d.maxdisp, d.work, queue_ranges(d), d.work_count, d.N,
                                                         d.cert);
     else
-        k_search<<<g.search_blocks, TPB, 0, s>>>(d.pos_s, d.id[buf], d.params, d.pos, d.cons, g.mesh, d.maxdisp,
+        k_search<<<g.search_blocks, TPB, 0, s>>>(d.pos_s, d.id_s, d.params, d.pos, d.cons, g.mesh, d.maxdisp,
                                                  d.work, queue_ranges(d), d.work_count, d.N, d.cert);
     if (timed) {
         cudaEventRecordWithFlags(g.ev[g.ev_used + 4], s, flags);
@@ -1813,17 +1789,17 @@ void iterate(Group &g, cudaStream_t s, bool energy_mode, int32_t *count_dbg) {
     }
 }
 
-void step_and_project(Group &g, cudaStream_t s, int buf) {
+void step_and_project(Group &g, cudaStream_t s) {
     DevGroup &d = g.d;
     if (d.N == 0) return;
-    k_step<<<nblocks(d.N), TPB, 0, s>>>(d.pos_s, d.acc_s, d.id[buf], d.N, d.params, d.amax, d.pos, d.cons, g.mesh,
+    k_step<<<nblocks(d.N), TPB, 0, s>>>(d.pos_s, d.acc_s, d.id_s, d.N, d.params, d.amax, d.pos, d.cons, g.mesh,
                                          d.maxdisp, d.work, queue_ranges(d), d.work_count, d.cert, d.cons_s);
     if (g.search_thread)
-        k_search_thread<<<g.search_blocks, TPB, 0, s>>>(d.pos_s, d.id[buf], d.params, d.pos, d.cons, g.mesh,
+        k_search_thread<<<g.search_blocks, TPB, 0, s>>>(d.pos_s, d.id_s, d.params, d.pos, d.cons, g.mesh,
                                                         d.maxdisp, d.work, queue_ranges(d), d.work_count, d.N,
                                                         d.cert);
     else
-        k_search<<<g.search_blocks, TPB, 0, s>>>(d.pos_s, d.id[buf], d.params, d.pos, d.cons, g.mesh, d.maxdisp,
+        k_search<<<g.search_blocks, TPB, 0, s>>>(d.pos_s, d.id_s, d.params, d.pos, d.cons, g.mesh, d.maxdisp,
                                                  d.work, queue_ranges(d), d.work_count, d.N, d.cert);
 }
 
@@ -1840,13 +1816,13 @@ void tag_ghosts(Group &g, int64_t first_ghost, cudaStream_t s) {
     if (g.d.N > 0) k_tag_ghosts<<<nblocks(g.d.N), TPB, 0, s>>>(g.d.pos, g.d.N, first_ghost);
 }
 
-void unpermute_dev(DevGroup &d, int buf, cudaStream_t s, float *acc_out, const int32_t *count_s,
+void unpermute_dev(DevGroup &d, cudaStream_t s, float *acc_out, const int32_t *count_s,
                    int32_t *count_out) {
-    k_unpermute<<<nblocks(d.N), TPB, 0, s>>>(d.acc_s, d.id[buf], d.N, acc_out, count_s, count_out);
+    k_unpermute<<<nblocks(d.N), TPB, 0, s>>>(d.acc_s, d.id_s, d.N, acc_out, count_s, count_out);
 }
 
-void unpermute(Group &g, int buf, cudaStream_t s, float *acc_out, const int32_t *count_s, int32_t *count_out) {
-    unpermute_dev(g.d, buf, s, acc_out, count_s, count_out);
+void unpermute(Group &g, cudaStream_t s, float *acc_out, const int32_t *count_s, int32_t *count_out) {
+    unpermute_dev(g.d, s, acc_out, count_s, count_out);
 }
 
 void project_points(Group &g, const float *y, const int32_t *cls, const int32_t *cons_in, int64_t n, float *x,
