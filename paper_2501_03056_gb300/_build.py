@@ -30,6 +30,7 @@ UNITS = {
     "body.cu": [],
     "relax.cu": [],
     "energy.cu": [],
+    "stats.cu": [],
     "api.cu": [],
     "noalloc.cu": [],
     "mapping.cu": ["-fmad=false", "-Xcompiler", "-ffp-contract=off"],

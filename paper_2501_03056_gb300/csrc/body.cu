@@ -258,7 +258,7 @@ void Group::release_particles() {
     DevGroup &g = d;
     void *ptrs[] = {g.pos,    g.cons,   g.cons_s,   g.key[0], g.key[1],  g.id[0],   g.id[1],  g.pos_s,
                     g.pos_p,  g.cert,   g.acc_s,    g.hist,   g.coef_s,  g.work,    g.fstart, g.bstart,
-                    g.amax,   g.maxdisp, g.work_count, g.totals, g.cnt, g.tiles, g.tile_base, g.scan_tmp};
+                    g.amax,   g.maxdisp, g.work_count, g.totals, g.cnt, g.tiles, g.tile_base, g.scan_tmp, g.stat};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     g.cnt = g.tiles = g.tile_base = g.scan_tmp = nullptr;
@@ -268,6 +268,7 @@ void Group::release_particles() {
     g.key[0] = g.key[1] = g.id[0] = g.id[1] = nullptr;
     g.hist = g.fstart = g.bstart = g.amax = g.maxdisp = g.work_count = g.totals = nullptr;
     g.coef_s = nullptr;
+    g.stat = nullptr;
     g.work = nullptr;
     g.N = 0;
 }
@@ -281,7 +282,7 @@ int Group::alloc_particles(int64_t N, std::string &err) {
 int Group::alloc_particles_once(int64_t N, std::string &err) {
     DevGroup &g = d;
     void *old[] = {g.pos,   g.cons,  g.cons_s, g.key[0], g.key[1], g.id[0], g.id[1],
-                   g.pos_s, g.pos_p, g.cert,   g.acc_s,  g.hist,   g.coef_s, g.work};
+                   g.pos_s, g.pos_p, g.cert,   g.acc_s,  g.hist,   g.coef_s, g.work, g.stat};
     for (void *p : old)
         if (p) cudaFree(p);
     g.pos = g.pos_s = g.pos_p = g.cert = g.acc_s = nullptr;
@@ -289,6 +290,7 @@ int Group::alloc_particles_once(int64_t N, std::string &err) {
     g.key[0] = g.key[1] = g.id[0] = g.id[1] = nullptr;
     g.hist = nullptr;
     g.coef_s = nullptr;
+    g.stat = nullptr;
     g.work = nullptr;
     g.N = N;
     const size_t n1 = (size_t)std::max<int64_t>(N, 1);
@@ -309,6 +311,7 @@ int Group::alloc_particles_once(int64_t N, std::string &err) {
     CKA(cudaMemset(g.cert, 0, sizeof(float4) * n1));
     CKA(dev_malloc(&g.acc_s, sizeof(float4) * n1));
     CKA(dev_malloc(&g.coef_s, sizeof(float) * (n1 + 1)));
+    CKA(dev_malloc(&g.stat, sizeof(double) * (size_t)stat_scratch(N)));
     CKA(dev_malloc(&g.work, (sizeof(int4) + sizeof(uint2)) * n1));   // queue entries, then their ranges
     if (!g.work_count) {
         CKA(dev_malloc(&g.work_count, 2 * sizeof(uint32_t)));
@@ -393,7 +396,7 @@ void Group::free_all() {
     DevGroup &g = d;
     void *ptrs[] = {g.params, g.row_rank, g.pos, g.cons, g.cons_s, g.key[0], g.key[1], g.id[0], g.id[1], g.pos_s, g.pos_p, g.cert,
                     g.acc_s, g.fstart, g.bstart, g.amax, g.maxdisp, g.hist, g.totals, g.coef_s, g.work,
-                    g.work_count, g.cnt, g.tiles, g.tile_base, g.scan_tmp};
+                    g.work_count, g.cnt, g.tiles, g.tile_base, g.scan_tmp, g.stat};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (owns_mesh) {

@@ -185,6 +185,7 @@ void unpermute(Group &g, cudaStream_t s, float *acc_out, const int32_t *count_s,
 void project_points(Group &g, const float *y, const int32_t *cls, const int32_t *cons_in, int64_t n, float *x,
                     int32_t *cons_out, int32_t *ok, cudaStream_t s);
 // uniformity statistics into host doubles (see fppg_stats_t)
+int64_t stat_scratch(int64_t n);
 int stats(Group &g, cudaStream_t s, double *mean, double *sd, double *minpair, double *maxdisp, int64_t *cnt,
           std::string &err);
 // initial particles of Sec. 3.2 into the group (features, surface, volume)

@@ -178,8 +178,9 @@ struct DevGroup {
     uint32_t *occ = nullptr;
     uint32_t *drank = nullptr, *coff = nullptr;
     int32_t *cand = nullptr;
-    // energy scratch
+    // energy scratch (the statistics keep their kernel sums there)
     float *coef_s = nullptr;
+    double *stat = nullptr;    // statistics: stat_scratch(N) doubles
 };
 
 // the candidate-list range of each search-queue entry, stored after the

@@ -1602,63 +1602,6 @@ __global__ void k_project_points(const float *__restrict__ y, const int32_t *__r
     }
 }
 
-// ---- statistics -------------------------------------------------------------------
-// kernel sum rho = W(0) + sum of W over masked neighbours; per-class sums in
-// FP64; smallest masked pair distance over mobile particles
-__global__ void __launch_bounds__(TPB) k_density(const float4 *__restrict__ pos_s, int64_t N,
-                                                 const AsmParams *__restrict__ P, const uint32_t *__restrict__ fstart,
-                                                 float *__restrict__ rho_s, uint32_t *__restrict__ minpair) {
-    const int64_t k = (int64_t)blockIdx.x * TPB + threadIdx.x;
-    if (k >= N) return;
-    const float4 p = pos_s[k];
-    const int cls = cls_of(p.w);
-    const AsmParams &A = P[body_of(p.w)];
-    const uint32_t mbits = acts_on_bits(cls);
-    const int nx = A.ng_n[0], ny = A.ng_n[1], nz = A.ng_n[2];
-    const int cx = cell_coord(p.x, A.ng_o[0], A.ng_inv, nx);
-    const int cy = cell_coord(p.y, A.ng_o[1], A.ng_inv, ny);
-    const int cz = cell_coord(p.z, A.ng_o[2], A.ng_inv, nz);
-    float rho = 0.f, rmin2 = FLT_MAX;
-    for (int z = max(cz - 1, 0); z <= min(cz + 1, nz - 1); z++)
-        for (int y = max(cy - 1, 0); y <= min(cy + 1, ny - 1); y++) {
-            const uint32_t row = A.key_base + (uint32_t)nx * grid_row(A, y, z);
-            uint32_t s, e;
-            cells_slots(fstart, row, max(cx - 1, 0), min(cx + 1, nx - 1), s, e);
-            for (uint32_t j = s; j < e; j++) {
-                const float4 q = pos_s[j];
-                const float dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z;
-                const float r2 = dist2_rn(dx, dy, dz);
-                if (r2 < A.R2 && (int64_t)j != k && (mbits & __float_as_uint(q.w)) != 0u) {
-                    const float r = sqrtf(r2);
-                    const float qh = r * A.half_inv_h;   // q / 2
-                    const float t = 1.f - qh;
-                    rho += t * t * t * t * (4.f * qh + 1.f);
-                    rmin2 = fminf(rmin2, r2);
-                }
-            }
-        }
-    rho_s[k] = A.alpha * (rho + 1.f);
-    if (is_mobile(cls, A) && !is_ghost(p.w) && rmin2 < FLT_MAX) atomicMin(minpair, __float_as_uint(sqrtf(rmin2)));
-}
-
-__global__ void k_class_sums(const float4 *__restrict__ pos_s, const float *__restrict__ rho_s, int64_t N,
-                             const double *__restrict__ mean, double *__restrict__ sums) {
-    // sums[0..2] sum rho, [3..5] sum (rho - mean)^2 when mean != null, [6..8] count
-    const int64_t k = (int64_t)blockIdx.x * TPB + threadIdx.x;
-    if (k >= N) return;
-    const float w = pos_s[k].w;
-    int c = cls_of(w);
-    if (c > kClsF || is_ghost(w)) return;
-    double r = rho_s[k];
-    if (mean) {
-        double d = r - mean[c];
-        atomicAdd(sums + 3 + c, d * d);
-    } else {
-        atomicAdd(sums + c, r);
-        atomicAdd(sums + 6 + c, 1.0);
-    }
-}
-
 } // namespace
 
 // ---- host driver ----------------------------------------------------------------
@@ -1828,59 +1771,6 @@ void unpermute(Group &g, cudaStream_t s, float *acc_out, const int32_t *count_s,
 void project_points(Group &g, const float *y, const int32_t *cls, const int32_t *cons_in, int64_t n, float *x,
                     int32_t *cons_out, int32_t *ok, cudaStream_t s) {
     k_project_points<<<nblocks(32 * n), TPB, 0, s>>>(y, cls, cons_in, n, g.d.params, g.mesh, x, cons_out, ok);
-}
-
-int stats(Group &g, cudaStream_t s, double *mean, double *sd, double *minpair, double *maxdisp, int64_t *cnt,
-          std::string &err) {
-    DevGroup &d = g.d;
-    double *sums = nullptr;
-    uint32_t *mp = nullptr;
-    float *rho = nullptr;
-    if (dev_malloc(&sums, 12 * sizeof(double)) != cudaSuccess || dev_malloc(&mp, 8) != cudaSuccess ||
-        dev_malloc(&rho, sizeof(float) * std::max<int64_t>(d.N, 1)) != cudaSuccess) {
-        err = "stats: out of device memory";
-        cudaFree(sums);
-        cudaFree(mp);
-        return 3;
-    }
-    cudaMemsetAsync(sums, 0, 12 * sizeof(double), s);
-    uint32_t big = 0x7f7fffffu;
-    cudaMemcpyAsync(mp, &big, 4, cudaMemcpyHostToDevice, s);
-    uint32_t md = 0;
-    cudaMemcpyAsync(&md, d.maxdisp, 4, cudaMemcpyDeviceToHost, s);
-    if (d.N > 0) {
-        build_grid(g, s);
-        k_density<<<nblocks(d.N), TPB, 0, s>>>(d.pos_s, d.N, d.params, d.fstart, rho, mp);
-        k_class_sums<<<nblocks(d.N), TPB, 0, s>>>(d.pos_s, rho, d.N, nullptr, sums);
-    }
-    double h[12];
-    cudaMemcpyAsync(h, sums, sizeof(h), cudaMemcpyDeviceToHost, s);
-    cudaStreamSynchronize(s);
-    for (int c = 0; c < 3; c++) mean[c] = h[6 + c] > 0 ? h[c] / h[6 + c] : 0.0;
-    cudaMemcpyAsync(sums + 9, mean, 3 * sizeof(double), cudaMemcpyHostToDevice, s);
-    if (d.N > 0) k_class_sums<<<nblocks(d.N), TPB, 0, s>>>(d.pos_s, rho, d.N, sums + 9, sums);
-    uint32_t mph = 0;
-    cudaMemcpyAsync(h, sums, sizeof(h), cudaMemcpyDeviceToHost, s);
-    cudaMemcpyAsync(&mph, mp, 4, cudaMemcpyDeviceToHost, s);
-    cudaError_t e = cudaStreamSynchronize(s);
-    for (int c = 0; c < 3; c++) {
-        sd[c] = h[6 + c] > 0 ? std::sqrt(h[3 + c] / h[6 + c]) : 0.0;
-        cnt[c] = (int64_t)h[6 + c];
-    }
-    float mpf, mdf;
-    memcpy(&mpf, &mph, 4);
-    memcpy(&mdf, &md, 4);
-    const float dx = g.hp[0].dx;
-    *minpair = mph == big ? INFINITY : (double)mpf / dx;
-    *maxdisp = (double)mdf / dx;
-    cudaFree(sums);
-    cudaFree(mp);
-    cudaFree(rho);
-    if (e != cudaSuccess) {
-        err = std::string("stats: ") + cudaGetErrorString(e);
-        return 4;
-    }
-    return 0;
 }
 
 } // namespace fppg

@@ -262,8 +262,8 @@ int radix_sort_impl(K *keys[2], uint32_t *vals[2], bool iota_vals, int64_t n, in
 
 // ---- exclusive scan (set-up work) -----------------------------------------
 // 16 entries per thread, 4096 per block; entries move as 16-byte vectors
-// when both arrays are 16-byte aligned (VEC), else one by one.  in == out is allowed (each thread reads its entries
-// before it writes them).
+// when both arrays are 16-byte aligned (VEC), else one by one.  in == out is
+// allowed (each thread reads its entries before it writes them).
 constexpr int SCAN_ITEMS = 16;
 constexpr int SCAN_BLOCK = RT * SCAN_ITEMS;
 
@@ -285,9 +285,7 @@ __global__ void __launch_bounds__(RT) k_scan_block(const uint32_t *in, uint32_t 
         }
     } else {
 #pragma unroll
-        for (int i = 0; i < SCAN_ITEMS; i++) {
-            v[i] = base + i < n ? in[base + i] : 0u;
-        }
+        for (int i = 0; i < SCAN_ITEMS; i++) v[i] = base + i < n ? in[base + i] : 0u;
     }
 #pragma unroll
     for (int i = 0; i < SCAN_ITEMS; i++) s += v[i];
