@@ -113,6 +113,43 @@ __global__ void k_set_body(float4 *__restrict__ pos, int64_t n, int body) {
     pos[i] = p;
 }
 
+// The states of up to kMoveBodies bodies moved between a batch and the bodies'
+// own arrays in one launch: item first[q] + k is particle k of the q-th body
+// of the table, at off[q] + k in the batch.  Two copies and a kernel for each
+// body were bound by their launches: store of 64 bodies (7.1 M particles) and
+// its waits 1.1 -> 0.2 ms of a pass, of eight (76 k) 0.12 -> 0.03 ms.
+constexpr int kMoveBodies = 96;
+struct BodyMove {
+    float4 *pos[kMoveBodies];
+    int32_t *cons[kMoveBodies];
+    int64_t first[kMoveBodies + 1], off[kMoveBodies];
+    int body[kMoveBodies];
+    int n;
+};
+static_assert(sizeof(BodyMove) <= 4000, "kernel parameters hold 4 KB");
+
+__global__ void __launch_bounds__(256) k_move_bodies(const __grid_constant__ BodyMove m, float4 *__restrict__ pos,
+                                                     int32_t *__restrict__ cons, bool store) {
+    const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (t >= m.first[m.n]) return;
+    int lo = 0, hi = m.n - 1;          // the last body whose first item is <= t
+    while (lo < hi) {
+        const int c = (lo + hi + 1) >> 1;
+        if (m.first[c] <= t) lo = c;
+        else hi = c - 1;
+    }
+    const int64_t k = t - m.first[lo], i = m.off[lo] + k;
+    float4 p = store ? pos[i] : m.pos[lo][k];
+    p.w = __uint_as_float((__float_as_uint(p.w) & 0xffu) | (store ? 0u : (uint32_t)m.body[lo] << 8));
+    if (store) {
+        m.pos[lo][k] = p;
+        m.cons[lo][k] = cons[i];
+    } else {
+        pos[i] = p;
+        cons[i] = m.cons[lo][k];
+    }
+}
+
 inline unsigned nb(int64_t n) { return (unsigned)std::max<int64_t>((n + 255) / 256, 1); }
 
 // f(begin, end) over [0, n) in chunks on up to 32 host threads (at least 2^20
@@ -1084,41 +1121,54 @@ int fppg_batch_force_ms(fppg_batch *b, double *ms) {
     return r;
 }
 
+// copies the state of the batch's bodies into their own arrays (store) or
+// back from them, kMoveBodies bodies to a launch
+static int batch_move(fppg_batch *b, bool store) {
+    DevGroup &d = b->group.d;
+    BodyMove m;
+    m.n = 0;
+    int64_t items = 0;
+    auto launch = [&]() {
+        if (m.n == 0) return;
+        k_move_bodies<<<nb(items), 256, 0, b->stream>>>(m, d.pos, d.cons, store);
+        m.n = 0;
+        items = 0;
+    };
+    for (size_t i = 0; i < b->ctxs.size(); i++) {
+        DevGroup &c = b->ctxs[i]->group.d;
+        // (a body whose count changed since: no more than either side holds)
+        const int64_t cn = std::min(b->ctxs[i]->n, b->off[i + 1] - b->off[i]);
+        if (!cn) continue;
+        m.first[m.n] = items;
+        m.off[m.n] = b->off[i];
+        m.body[m.n] = (int)i;
+        m.pos[m.n] = c.pos;
+        m.cons[m.n] = c.cons;
+        m.n++;
+        items += cn;
+        m.first[m.n] = items;
+        if (m.n == kMoveBodies) launch();
+    }
+    launch();
+    CUDA_OR(b->err, cudaGetLastError());
+    return FPPG_OK;
+}
+
 int fppg_batch_store(fppg_batch *b) {
     if (!b) return FPPG_ERR_ARG;
-    cudaStream_t s = b->stream;
-    DevGroup &d = b->group.d;
-    for (size_t i = 0; i < b->ctxs.size(); i++) {
-        fppg_ctx *c = b->ctxs[i];
-        const int64_t cn = c->n;
-        if (!cn) continue;
-        CUDA_OR(b->err, cudaMemcpyAsync(c->group.d.pos, d.pos + b->off[i], sizeof(float4) * cn,
-                                        cudaMemcpyDeviceToDevice, s));
-        CUDA_OR(b->err, cudaMemcpyAsync(c->group.d.cons, d.cons + b->off[i], sizeof(int32_t) * cn,
-                                        cudaMemcpyDeviceToDevice, s));
-        k_set_body<<<nb(cn), 256, 0, s>>>(c->group.d.pos, cn, 0);
-    }
-    CUDA_OR(b->err, cudaStreamSynchronize(s));
+    const int r = batch_move(b, true);
+    if (r) return r;
+    CUDA_OR(b->err, cudaStreamSynchronize(b->stream));
     return FPPG_OK;
 }
 
 int fppg_batch_load(fppg_batch *b) {
     if (!b) return FPPG_ERR_ARG;
-    cudaStream_t s = b->stream;
-    DevGroup &d = b->group.d;
-    for (size_t i = 0; i < b->ctxs.size(); i++) {
-        fppg_ctx *c = b->ctxs[i];
-        const int64_t cn = c->n;
-        if (cn != b->off[i + 1] - b->off[i]) return fail(b->err, FPPG_ERR_STATE, "a body changed its particle count");
-        if (!cn) continue;
-        CUDA_OR(b->err, cudaMemcpyAsync(d.pos + b->off[i], c->group.d.pos, sizeof(float4) * cn,
-                                        cudaMemcpyDeviceToDevice, s));
-        CUDA_OR(b->err, cudaMemcpyAsync(d.cons + b->off[i], c->group.d.cons, sizeof(int32_t) * cn,
-                                        cudaMemcpyDeviceToDevice, s));
-        k_set_body<<<nb(cn), 256, 0, s>>>(d.pos + b->off[i], cn, (int)i);
-    }
-    CUDA_OR(b->err, cudaGetLastError());
-    return FPPG_OK;
+    // (nothing is loaded when a body's count changed)
+    for (size_t i = 0; i < b->ctxs.size(); i++)
+        if (b->ctxs[i]->n != b->off[i + 1] - b->off[i])
+            return fail(b->err, FPPG_ERR_STATE, "a body changed its particle count");
+    return batch_move(b, false);
 }
 
 namespace {
