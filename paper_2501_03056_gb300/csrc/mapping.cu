@@ -3,17 +3,29 @@
 // Compiled with -fmad=false: the ray-parity arithmetic is evaluated exactly
 // in the written order, so inside / outside is decided as by any other IEEE
 // implementation of the same formulas.
-//   k_column_parity  one warp per (x, y) column of the triangle grid: the
-//                    +z ray of Fig. 6 from every cell centre (displaced by
-//                    (1.234567e-6, 2.345678e-6) dx in x, y so it never meets
-//                    an edge or vertex exactly) against the triangles binned
-//                    into the column, each triangle counted once
-//   k_dilate_axis    Chebyshev distance <= band to a cell with triangles,
-//                    by three one-axis dilations of the occupancy bitmap
-//   k_map_cells      per cell in key order: a cell with triangles maps its
-//                    centre to the nearest triangle of the cell whose foot
-//                    is inside (else it is discarded, Fig. 9b); an empty
-//                    cell inside the body gives a volume particle
+// Cell sets are bitmaps of rows padded to whole words: bit x & 31 of word
+// (x >> 5) + W (y + ny z), W = ceil(nx / 32), so that a word is 32 columns or
+// 32 cells of a row, and words in order are cells in key order.  Work that
+// belongs to the surface runs over the occupied cells only (C_compact).
+//   k_crossings      +z rays of Fig. 6 from the cell centres of every column
+//                    (displaced by (1.234567e-6, 2.345678e-6) dx in x, y so
+//                    they meet no edge or vertex exactly) against the
+//                    triangles of the occupied cells, each triangle once per
+//                    column: a crossing toggles the cells below it, noted at
+//                    the highest one
+//   k_inside_words   the parity of the crossings above every cell, 32 columns
+//                    at a time (exclusive or down the columns)
+//   k_dilate_x/_yz   Chebyshev distance <= band to a cell with triangles, by
+//                    three one-axis dilations
+//   k_surface_cells  a cell with triangles maps its centre to the nearest
+//                    triangle of the cell whose foot is inside (else it is
+//                    discarded, Fig. 9b)
+//   k_word_counts    surface cells and empty inside cells per word; their
+//                    scan gives the particles' places in key order
+//   k_emit_surface, k_emit_volume
+// A body of C cells moves C / 8 bytes a pass instead of C to 4 C: the gear
+// turned in space (1.7e8 cells, 2.9 M particles) 12.0 -> 0.9 ms of kernels, most of
+// it the FP64 barycentric tests of k_crossings (0.5 ms).
 #include <cfloat>
 #include <cmath>
 
@@ -22,21 +34,39 @@
 namespace fppg {
 namespace {
 
-constexpr int kColBuf = 256;   // crossing candidates per column and warp
+constexpr uint32_t kColEntries = 256;   // crossed triangle entries a column may hold
 
 __device__ inline bool bit_of(const uint32_t *m, uint64_t c) { return (m[c >> 5] >> (c & 31u)) & 1u; }
-
-__device__ inline double centre(const float *o, int a, int i, double dx) {
-    return (double)(float)((double)o[a] + ((double)i + 0.5) * dx);
-}
 
 struct MapGrid {
     float o[3];
     int n[3];
+    int W;                 // words of a row
     double dx;
+    const float *mid[3];   // cell centres along each axis (k_centres)
     uint32_t hash_mask;
     float edge_tol;
 };
+
+// the cell centres along the axes, evaluated in FP64 once instead of by every
+// cell (the FP64 units are far slower than the rest of this path)
+__global__ void __launch_bounds__(256) k_centres(MapGrid g, float *__restrict__ out) {
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    const int a = i < g.n[0] ? 0 : i < g.n[0] + g.n[1] ? 1 : 2;
+    const int k = i - (a > 0 ? g.n[0] : 0) - (a > 1 ? g.n[1] : 0);
+    if (k < g.n[a]) out[i] = (float)((double)g.o[a] + ((double)k + 0.5) * g.dx);
+}
+
+__device__ inline size_t word_of(const MapGrid &g, int x, int y, int z) {
+    return (size_t)(x >> 5) + (size_t)g.W * ((size_t)y + (size_t)g.n[1] * (size_t)z);
+}
+
+__device__ inline void cell_of_key(const MapGrid &g, uint32_t key, int &x, int &y, int &z) {
+    x = (int)(key % (uint32_t)g.n[0]);
+    const uint32_t r = key / (uint32_t)g.n[0];
+    y = (int)(r % (uint32_t)g.n[1]);
+    z = (int)(r / (uint32_t)g.n[1]);
+}
 
 __device__ inline bool cell_tris(const uint2 *hrng, const uint4 *compact, const MapGrid &g, int x, int y, int z,
                                  uint32_t &beg, uint32_t &len) {
@@ -54,105 +84,134 @@ __device__ inline bool cell_tris(const uint2 *hrng, const uint4 *compact, const 
     return false;
 }
 
-__global__ void __launch_bounds__(256) k_column_parity(const float *__restrict__ V, const int32_t *__restrict__ T,
-                                                       const uint32_t *__restrict__ occ, const uint2 *__restrict__ hrng,
-                                                       const uint4 *__restrict__ compact,
-                                                       const int32_t *__restrict__ tlist, MapGrid g,
-                                                       uint8_t *__restrict__ inside, uint32_t *__restrict__ error) {
-    __shared__ int32_t s_tri[8][kColBuf];
-    __shared__ double s_z[8][kColBuf];
-    __shared__ int s_cnt[8];
-    const int w = threadIdx.x / 32, lane = threadIdx.x & 31;
-    const int64_t col = (int64_t)blockIdx.x * 8 + w;
-    if (col >= (int64_t)g.n[0] * g.n[1]) return;                 // whole warp
-    const int x = (int)(col % g.n[0]), y = (int)(col / g.n[0]);
-    const double qx = centre(g.o, 0, x, g.dx) + 1.234567e-6 * g.dx;
-    const double qy = centre(g.o, 1, y, g.dx) + 2.345678e-6 * g.dx;
-    if (lane == 0) s_cnt[w] = 0;
-    __syncwarp();
-    bool overflow = false;
-    for (int z0 = 0; z0 < g.n[2]; z0 += 32) {
-        const int z = z0 + lane;
-        uint32_t beg = 0, len = 0;
-        if (z < g.n[2]) {
-            const uint64_t key = (uint64_t)x + (uint64_t)g.n[0] * ((uint64_t)y + (uint64_t)g.n[1] * (uint64_t)z);
-            if (bit_of(occ, key)) cell_tris(hrng, compact, g, x, y, z, beg, len);
+// One thread per occupied cell.  A triangle's cells in a column are one run
+// along z, so a crossing counts at the lowest cell that lists the triangle.
+__global__ void __launch_bounds__(256) k_crossings(const float4 *__restrict__ vx,
+                                                   const uint32_t *__restrict__ occ, const uint2 *__restrict__ hrng,
+                                                   const uint4 *__restrict__ compact, int64_t ncompact,
+                                                   const int32_t *__restrict__ tlist, MapGrid g,
+                                                   uint32_t *__restrict__ toggle, uint32_t *__restrict__ entries,
+                                                   uint32_t *__restrict__ error) {
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= ncompact) return;
+    const uint4 cell = compact[i];
+    int x, y, z;
+    cell_of_key(g, cell.x, x, y, z);
+    const double qx = (double)g.mid[0][x] + 1.234567e-6 * g.dx;
+    const double qy = (double)g.mid[1][y] + 2.345678e-6 * g.dx;
+    // a nonzero quotient of these differences is far above underflow, so its
+    // sign is that of its operands: most triangles end before a division
+    auto negative = [](double num, double den) {
+        return num != 0.0 && (__double2hiint(num) ^ __double2hiint(den)) < 0;
+    };
+    for (uint32_t e = cell.y; e < cell.y + cell.z; e++) {
+        const int t = tlist[e];
+        const float4 a = vx[3 * (size_t)t], b = vx[3 * (size_t)t + 1], c = vx[3 * (size_t)t + 2];
+        const double ax = a.x, ay = a.y, bx = b.x, by = b.y, cx = c.x, cy = c.y;
+        const double d = (bx - ax) * (cy - ay) - (cx - ax) * (by - ay);
+        if (d == 0.0) continue;
+        const double m1 = (bx - qx) * (cy - qy) - (cx - qx) * (by - qy);
+        if (negative(m1, d)) continue;
+        const double m2 = (cx - qx) * (ay - qy) - (ax - qx) * (cy - qy);
+        if (negative(m2, d)) continue;
+        const double l1 = m1 / d, l2 = m2 / d;
+        const double l3 = 1.0 - l1 - l2;
+        if (l3 < 0) continue;
+        if (atomicAdd(entries + (size_t)x + (size_t)g.n[0] * (size_t)y, 1u) >= kColEntries) {
+            atomicOr(error, 1u);
+            return;
         }
-        for (uint32_t e = beg; e < beg + len; e++) {
-            const int t = tlist[e];
-            const float *a = V + 3 * T[3 * t], *b = V + 3 * T[3 * t + 1], *c = V + 3 * T[3 * t + 2];
-            const double ax = a[0], ay = a[1], bx = b[0], by = b[1], cx = c[0], cy = c[1];
-            const double d = (bx - ax) * (cy - ay) - (cx - ax) * (by - ay);
-            if (d == 0.0) continue;
-            const double l1 = ((bx - qx) * (cy - qy) - (cx - qx) * (by - qy)) / d;
-            const double l2 = ((cx - qx) * (ay - qy) - (ax - qx) * (cy - qy)) / d;
-            const double l3 = 1.0 - l1 - l2;
-            if (l1 < 0 || l2 < 0 || l3 < 0) continue;
-            const double zc = l1 * (double)a[2] + l2 * (double)b[2] + l3 * (double)c[2];
-            const int slot = atomicAdd(&s_cnt[w], 1);
-            if (slot < kColBuf) {
-                s_tri[w][slot] = t;
-                s_z[w][slot] = zc;
-            } else {
-                overflow = true;
-            }
+        bool first = true;
+        if (z > 0 && bit_of(occ, (uint64_t)cell.x - (uint64_t)g.n[0] * (uint64_t)g.n[1])) {
+            uint32_t beg = 0, len = 0;
+            if (cell_tris(hrng, compact, g, x, y, z - 1, beg, len))
+                for (uint32_t q = beg; q < beg + len && first; q++) first = tlist[q] != t;
         }
-    }
-    __syncwarp();
-    if (__any_sync(0xffffffffu, overflow)) {
-        if (lane == 0) atomicOr(error, 1u);
-        return;
-    }
-    const int m = s_cnt[w];
-    // a triangle binned into several cells of the column is counted once:
-    // an entry counts only if no earlier entry holds the same triangle
-    for (int z0 = 0; z0 < g.n[2]; z0 += 32) {
-        const int z = z0 + lane;
-        if (z >= g.n[2]) continue;
-        const double qz = centre(g.o, 2, z, g.dx);
-        int cross = 0;
-        for (int e = 0; e < m; e++) {
-            if (!(s_z[w][e] > qz)) continue;
-            bool first = true;
-            for (int f = 0; f < e && first; f++) first = s_tri[w][f] != s_tri[w][e];
-            cross += first;
-        }
-        inside[(uint64_t)x + (uint64_t)g.n[0] * ((uint64_t)y + (uint64_t)g.n[1] * (uint64_t)z)] = (uint8_t)(cross & 1);
+        if (!first) continue;
+        const double zc = l1 * (double)a.z + l2 * (double)b.z + l3 * (double)c.z;
+        // the cells whose centre lies below the crossing: 0 .. k - 1
+        int k = (int)fmin(fmax(ceil((zc - (double)g.o[2]) / g.dx - 0.5), 0.0), (double)g.n[2]);
+        while (k < g.n[2] && zc > (double)g.mid[2][k]) k++;
+        while (k > 0 && !(zc > (double)g.mid[2][k - 1])) k--;
+        if (k > 0) atomicXor(toggle + word_of(g, x, y, k - 1), 1u << (x & 31));
     }
 }
 
-// one-axis dilation by `band` cells of bitmap src into dst (bytes)
-__global__ void k_dilate_axis(const uint8_t *__restrict__ src, uint8_t *__restrict__ dst, MapGrid g, int axis,
-                              int band) {
-    const int64_t c = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    const int64_t total = (int64_t)g.n[0] * g.n[1] * g.n[2];
-    if (c >= total) return;
-    int idx[3] = {(int)(c % g.n[0]), (int)((c / g.n[0]) % g.n[1]), (int)(c / ((int64_t)g.n[0] * g.n[1]))};
-    const int64_t stride = axis == 0 ? 1 : (axis == 1 ? g.n[0] : (int64_t)g.n[0] * g.n[1]);
-    uint8_t v = 0;
-    for (int d = -band; d <= band && !v; d++) {
-        const int q = idx[axis] + d;
-        if (q < 0 || q >= g.n[axis]) continue;
-        v = src[c + (int64_t)d * stride];
+// the toggles of a column, from above: in place, bit (x, y, z) becomes the
+// parity of the crossings above its centre.  One thread per 32 columns.
+__global__ void __launch_bounds__(128) k_inside_words(uint32_t *__restrict__ m, MapGrid g) {
+    const int64_t q = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    const int64_t plane = (int64_t)g.W * g.n[1];
+    if (q >= plane) return;
+    uint32_t acc = 0u;
+    constexpr int kAhead = 8;      // words in flight
+    for (int z = g.n[2] - 1; z >= 0; z -= kAhead) {
+        uint32_t v[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; u++) v[u] = z - u >= 0 ? m[q + plane * (z - u)] : 0u;
+#pragma unroll
+        for (int u = 0; u < kAhead; u++) {
+            acc ^= v[u];
+            if (z - u >= 0) m[q + plane * (z - u)] = acc;
+        }
     }
-    dst[c] = v;
 }
 
-__global__ void k_occ_bytes(const uint32_t *__restrict__ occ, int64_t total, uint8_t *__restrict__ out) {
-    const int64_t c = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (c < total) out[c] = bit_of(occ, (uint64_t)c) ? 1 : 0;
+// the occupancy bitmap (bit = cell key) as padded rows
+__global__ void __launch_bounds__(256) k_occ_rows(const uint32_t *__restrict__ occ, int64_t occ_words, int64_t words,
+                                                  MapGrid g, uint32_t *__restrict__ out) {
+    const int64_t q = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (q >= words) return;
+    const int64_t row = (uint32_t)q / (uint32_t)g.W;
+    const int x0 = 32 * (int)(q - row * g.W), left = g.n[0] - x0;
+    const uint64_t c = (uint64_t)row * (uint64_t)g.n[0] + (uint64_t)x0;
+    const int64_t w = (int64_t)(c >> 5);
+    const uint32_t v = __funnelshift_r(occ[w], w + 1 < occ_words ? occ[w + 1] : 0u, (uint32_t)(c & 31u));
+    out[q] = left >= 32 ? v : v & ((1u << left) - 1u);
 }
 
-// nearest triangle of cell (x, y, z) whose foot of the centre is inside
+// bit x of out: some bit of src within `band` of x in the same row
+__global__ void __launch_bounds__(256) k_dilate_x(const uint32_t *__restrict__ src, uint32_t *__restrict__ dst,
+                                                  int64_t words, MapGrid g, int band) {
+    const int64_t q = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (q >= words) return;
+    const int64_t row = (uint32_t)q / (uint32_t)g.W;
+    const int w = (int)(q - row * g.W);
+    const uint32_t *r = src + row * g.W;
+    // bits 32 w + d .. 32 w + d + 31 for d = -band .. band
+    uint32_t v = 0u;
+    for (int k = w - (band + 31) / 32; k <= w + band / 32; k++) {
+        const uint32_t lo = k >= 0 && k < g.W ? r[k] : 0u, hi = k + 1 >= 0 && k + 1 < g.W ? r[k + 1] : 0u;
+        if ((lo | hi) == 0u) continue;
+        for (int sh = 0; sh < 32; sh++) {
+            const int d = 32 * (k - w) + sh;
+            if (d >= -band && d <= band) v |= __funnelshift_r(lo, hi, (uint32_t)sh);
+        }
+    }
+    const int left = g.n[0] - 32 * w;
+    dst[q] = left >= 32 ? v : v & ((1u << left) - 1u);
+}
+
+// the same along y (axis 1) or z (axis 2)
+__global__ void __launch_bounds__(256) k_dilate_yz(const uint32_t *__restrict__ src, uint32_t *__restrict__ dst,
+                                                   int64_t words, MapGrid g, int axis, int band) {
+    const int64_t q = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (q >= words) return;
+    const int64_t stride = axis == 1 ? g.W : (int64_t)g.W * g.n[1];
+    const int i = (int)(((uint32_t)q / (uint32_t)stride) % (uint32_t)g.n[axis]);
+    const int lo = max(-band, -i), hi = min(band, g.n[axis] - 1 - i);
+    uint32_t v = 0u;
+    for (int d = lo; d <= hi; d++) v |= src[q + d * stride];
+    dst[q] = v;
+}
+
+// nearest triangle of the cell (a C_compact entry) whose foot of its centre p is inside
 // (the FP32 rule of the constraint step); -1 when none
-__device__ int map_surface_cell(const float4 *__restrict__ geo, const uint2 *__restrict__ hrng,
-                                const uint4 *__restrict__ compact, const int32_t *__restrict__ tlist, const MapGrid &g,
-                                int x, int y, int z, float3 p, float &dist) {
-    uint32_t beg = 0, len = 0;
-    if (!cell_tris(hrng, compact, g, x, y, z, beg, len)) return -1;
+__device__ int map_surface_cell(const float4 *__restrict__ geo, const uint4 &cell, const int32_t *__restrict__ tlist,
+                                const MapGrid &g, float3 p, float &dist) {
     float best = FLT_MAX, bd = 0.f;
     int bt = -1;
-    for (uint32_t e = beg; e < beg + len; e++) {
+    for (uint32_t e = cell.y; e < cell.y + cell.z; e++) {
         const int t = tlist[e];
         const float4 *q = geo + 5 * (size_t)t;
         const float ux = __fsub_rn(p.x, q[0].x), uy = __fsub_rn(p.y, q[0].y), uz = __fsub_rn(p.z, q[0].z);
@@ -172,52 +231,94 @@ __device__ int map_surface_cell(const float4 *__restrict__ geo, const uint2 *__r
     return bt;
 }
 
-// pass 0: flags (surface kept / volume); pass 1: emit at the scanned slots
-template <bool EMIT>
-__global__ void k_map_cells(const float4 *__restrict__ geo, const uint2 *__restrict__ hrng,
-                            const uint4 *__restrict__ compact, const int32_t *__restrict__ tlist,
-                            const uint32_t *__restrict__ occ, const uint8_t *__restrict__ inside,
-                            const uint8_t *__restrict__ band, const uint8_t *__restrict__ inner, MapGrid g,
-                            int surface, int volume,
-                            uint32_t *__restrict__ sflag, uint32_t *__restrict__ vflag,
-                            const uint32_t *__restrict__ soff, const uint32_t *__restrict__ voff, int64_t base_s,
-                            int64_t base_v, float4 *__restrict__ pos, int32_t *__restrict__ cons,
-                            int32_t *__restrict__ cls) {
-    const int64_t c = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    const int64_t total = (int64_t)g.n[0] * g.n[1] * g.n[2];
-    if (c >= total) return;
-    const int x = (int)(c % g.n[0]), y = (int)((c / g.n[0]) % g.n[1]), z = (int)(c / ((int64_t)g.n[0] * g.n[1]));
-    const float3 p = make_float3((float)centre(g.o, 0, x, g.dx), (float)centre(g.o, 1, y, g.dx),
-                                 (float)centre(g.o, 2, z, g.dx));
-    uint32_t fs = 0, fv = 0;
-    if (bit_of(occ, (uint64_t)c)) {
-        if (surface) {
-            float d;
-            const int t = map_surface_cell(geo, hrng, compact, tlist, g, x, y, z, p, d);
-            if (t >= 0) {
-                fs = 1;
-                if (EMIT) {
-                    const float4 n = geo[5 * (size_t)t + 1];
-                    const int64_t o = base_s + soff[c];
-                    pos[o] = make_float4(p.x - d * n.x, p.y - d * n.y, p.z - d * n.z, __uint_as_float(class_bit(kClsS)));
-                    cons[o] = t;
-                    cls[o] = kClsS;
-                }
-            }
-        }
-    } else if (volume && inside[c] && (inner == nullptr || inner[c])) {
-        fv = 1;
-        if (EMIT) {
-            const int cl = (band == nullptr || band[c]) ? kClsV : kClsI;
-            const int64_t o = base_v + voff[c];
-            pos[o] = make_float4(p.x, p.y, p.z, __uint_as_float(class_bit(cl)));
-            cons[o] = -1;
-            cls[o] = cl;
-        }
-    }
-    if (!EMIT) {
-        sflag[c] = fs;
-        vflag[c] = fv;
+__device__ inline float3 cell_centre(const MapGrid &g, int x, int y, int z) {
+    return make_float3(g.mid[0][x], g.mid[1][y], g.mid[2][z]);
+}
+
+// the triangle (-1: none) and plane distance of every occupied cell's centre,
+// and the bitmap of the cells that have one
+__global__ void __launch_bounds__(256) k_surface_cells(const float4 *__restrict__ geo, const uint4 *__restrict__ compact,
+                                                       int64_t ncompact,
+                                                       const int32_t *__restrict__ tlist, MapGrid g,
+                                                       int32_t *__restrict__ tri, float *__restrict__ dist,
+                                                       uint32_t *__restrict__ sbits) {
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= ncompact) return;
+    int x, y, z;
+    cell_of_key(g, compact[i].x, x, y, z);
+    float d = 0.f;
+    const int t = map_surface_cell(geo, compact[i], tlist, g, cell_centre(g, x, y, z), d);
+    tri[i] = t;
+    dist[i] = d;
+    if (t >= 0) atomicOr(sbits + word_of(g, x, y, z), 1u << (x & 31));
+}
+
+// vbits (the inside bitmap on entry): empty cells inside, within inner
+// (nullable); the counts of surface cells, then of volume cells, per word
+__global__ void __launch_bounds__(256) k_word_counts(const uint32_t *__restrict__ rows,
+                                                     const uint32_t *__restrict__ sbits,
+                                                     const uint32_t *__restrict__ inner, int64_t words,
+                                                     uint32_t *__restrict__ vbits, uint32_t *__restrict__ cnt) {
+    const int64_t q = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (q >= words) return;
+    uint32_t v = vbits[q] & ~rows[q];
+    if (inner) v &= inner[q];
+    vbits[q] = v;
+    cnt[q] = (uint32_t)__popc(sbits[q]);
+    cnt[words + q] = (uint32_t)__popc(v);
+}
+
+__global__ void __launch_bounds__(256) k_emit_surface(const float4 *__restrict__ geo, const uint4 *__restrict__ compact,
+                                                      int64_t ncompact, const int32_t *__restrict__ tri,
+                                                      const float *__restrict__ dist,
+                                                      const uint32_t *__restrict__ sbits,
+                                                      const uint32_t *__restrict__ off, MapGrid g,
+                                                      float4 *__restrict__ pos, int32_t *__restrict__ cons) {
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= ncompact) return;
+    const int t = tri[i];
+    if (t < 0) return;
+    int x, y, z;
+    cell_of_key(g, compact[i].x, x, y, z);
+    const size_t w = word_of(g, x, y, z);
+    const size_t o = (size_t)off[w] + (size_t)__popc(sbits[w] & ((1u << (x & 31)) - 1u));
+    const float3 p = cell_centre(g, x, y, z);
+    const float4 n = geo[5 * (size_t)t + 1];
+    const float d = dist[i];
+    pos[o] = make_float4(p.x - d * n.x, p.y - d * n.y, p.z - d * n.z, __uint_as_float(class_bit(kClsS)));
+    cons[o] = t;
+}
+
+// A warp takes 32 words and emits them one after another, a lane per cell.
+// off: places counted from the first surface particle; first: the same of the
+// first volume particle.  band (nullable): V inside it, else I; cls (with
+// band): the class of every volume particle.
+__global__ void __launch_bounds__(256) k_emit_volume(const uint32_t *__restrict__ vbits,
+                                                     const uint32_t *__restrict__ off,
+                                                     const uint32_t *__restrict__ band, int64_t words, uint32_t first,
+                                                     MapGrid g, float4 *__restrict__ pos, int32_t *__restrict__ cons,
+                                                     uint8_t *__restrict__ cls) {
+    const int lane = threadIdx.x & 31;
+    const int64_t q0 = ((int64_t)blockIdx.x * 256 + threadIdx.x) & ~(int64_t)31, q = q0 + lane;
+    const uint32_t mine = q < words ? vbits[q] : 0u;
+    const uint32_t at = mine ? off[q] : 0u, near = mine ? (band ? band[q] : 0xffffffffu) : 0u;
+    uint32_t todo = __ballot_sync(0xffffffffu, mine != 0u);
+    while (todo) {
+        const int src = __ffs(todo) - 1;
+        todo &= todo - 1u;
+        const uint32_t v = __shfl_sync(0xffffffffu, mine, src), a = __shfl_sync(0xffffffffu, at, src);
+        const uint32_t b = __shfl_sync(0xffffffffu, near, src);
+        if (!((v >> lane) & 1u)) continue;
+        // (below 2^32 / 5 words: a row has at least five cells to the word)
+        const uint32_t wq = (uint32_t)(q0 + src), row = wq / (uint32_t)g.W;
+        const int x = 32 * (int)(wq - row * (uint32_t)g.W) + lane;
+        const int z = (int)(row / (uint32_t)g.n[1]), y = (int)(row - (uint32_t)z * (uint32_t)g.n[1]);
+        const uint32_t o = a + (uint32_t)__popc(v & ((1u << lane) - 1u));
+        const int cl = (b >> lane) & 1u ? kClsV : kClsI;
+        const float3 p = cell_centre(g, x, y, z);
+        pos[o] = make_float4(p.x, p.y, p.z, __uint_as_float(class_bit(cl)));
+        cons[o] = -1;
+        if (cls) cls[o - first] = (uint8_t)cl;
     }
 }
 
@@ -278,15 +379,6 @@ void Body::feature_particles(std::vector<float> &xyz, std::vector<int32_t> &cls,
     }
 }
 
-#define CKM(x)                                                                       \
-    do {                                                                             \
-        cudaError_t e_ = (x);                                                        \
-        if (e_ != cudaSuccess) {                                                     \
-            err = std::string(#x) + ": " + cudaGetErrorString(e_);                   \
-            return e_ == cudaErrorMemoryAllocation ? 3 : 4;                          \
-        }                                                                            \
-    } while (0)
-
 int map_particles(Group &g, Body &b, int surface, int volume, int features, int band_cells, int inner_cells,
                   cudaStream_t s, int64_t *n_out, std::vector<int32_t> &cls_host, std::string &err) {
     MapGrid mg;
@@ -307,101 +399,122 @@ int map_particles(Group &g, Body &b, int surface, int volume, int features, int 
     if (features && b.has_features) b.feature_particles(fxyz, fcls, fseg);
     const int64_t nf = (int64_t)fcls.size();
 
-    uint8_t *inside = nullptr, *band = nullptr, *tmp = nullptr, *inner = nullptr;
-    uint32_t *sflag = nullptr, *vflag = nullptr, *soff = nullptr, *voff = nullptr, *tot = nullptr, *scr = nullptr,
-             *error = nullptr;
+    // one block of scratch: [0, zeroed) starts at 0
+    mg.W = (mg.n[0] + 31) / 32;
+    const int64_t words = (int64_t)mg.W * mg.n[1] * mg.n[2], cols = (int64_t)mg.n[0] * mg.n[1];
+    const bool use_band = volume && band_cells > 0, use_inner = use_band && inner_cells > 0;
+    const int64_t sc = scan_tmp_elems(2 * words);
+    const int64_t zeroed = 2 * words + cols + 1;
+    const int64_t mids = (int64_t)mg.n[0] + mg.n[1] + mg.n[2];
+    const int64_t total = zeroed + mids + (use_inner ? 4 : use_band ? 3 : 0) * words + 5 * words + 2 * b.ncompact + 2 + sc;
+    uint32_t *scr = nullptr;
+    uint8_t *vcls = nullptr;
     auto cleanup = [&]() {
-        void *p[] = {inside, band, tmp, inner, sflag, vflag, soff, voff, tot, scr, error};
-        for (void *q : p)
-            if (q) cudaFree(q);
+        if (scr) cudaFree(scr);
+        if (vcls) cudaFree(vcls);
     };
-    const int64_t sc = scan_tmp_elems(cells);
-    if (dev_malloc(&inside, cells) || dev_malloc(&sflag, 4 * cells) || dev_malloc(&vflag, 4 * cells) ||
-        dev_malloc(&soff, 4 * cells) || dev_malloc(&voff, 4 * cells) || dev_malloc(&tot, 8) ||
-        dev_malloc(&scr, 4 * sc) || dev_malloc(&error, 4)) {
-        cleanup();
+    if (dev_malloc(&scr, sizeof(uint32_t) * (size_t)total)) {
         err = "map_particles: out of device memory";
         return 3;
     }
-    cudaMemsetAsync(error, 0, 4, s);
-    cudaMemsetAsync(inside, 0, cells, s);
-    if (volume)
-        k_column_parity<<<nblk((int64_t)mg.n[0] * mg.n[1], 8), 256, 0, s>>>(b.d_verts, b.d_tris, b.occ, b.hrng,
-                                                                             b.compact, b.tlist, mg, inside, error);
-    if (volume && band_cells > 0) {
-        if (dev_malloc(&band, cells) || dev_malloc(&tmp, cells)) {
-            cleanup();
-            err = "map_particles: out of device memory";
-            return 3;
-        }
-        k_occ_bytes<<<nblk(cells), 256, 0, s>>>(b.occ, cells, band);
-        for (int axis = 0; axis < 3; axis++) {
-            k_dilate_axis<<<nblk(cells), 256, 0, s>>>(band, tmp, mg, axis, band_cells);
-            std::swap(band, tmp);
-        }
-        if (inner_cells > 0) {
-            if (dev_malloc(&inner, cells)) {
-                cleanup();
-                err = "map_particles: out of device memory";
-                return 3;
-            }
-            k_occ_bytes<<<nblk(cells), 256, 0, s>>>(b.occ, cells, inner);
-            for (int axis = 0; axis < 3; axis++) {
-                k_dilate_axis<<<nblk(cells), 256, 0, s>>>(inner, tmp, mg, axis, band_cells + inner_cells);
-                std::swap(inner, tmp);
-            }
-        }
+    uint32_t *q = scr;
+    auto take = [&](int64_t n) {
+        uint32_t *r = q;
+        q += n;
+        return r;
+    };
+    uint32_t *vbits = take(words), *sbits = take(words), *entries = take(cols), *error = take(1);
+    uint32_t *rows = take(words), *cnt = take(2 * words), *off = take(2 * words);
+    uint32_t *t1 = use_band ? take(words) : nullptr, *t2 = use_band ? take(words) : nullptr;
+    uint32_t *band = use_band ? take(words) : nullptr, *inner = use_inner ? take(words) : nullptr;
+    int32_t *tri = (int32_t *)take(b.ncompact);
+    float *dist = (float *)take(b.ncompact);
+    uint32_t *tot = take(2), *tmp = take(sc);
+    float *mid = (float *)take(mids);
+    for (int k = 0, at = 0; k < 3; at += mg.n[k++]) mg.mid[k] = mid + at;
+    k_centres<<<nblk(mids), 256, 0, s>>>(mg, mid);
+    cudaMemsetAsync(scr, 0, sizeof(uint32_t) * (size_t)zeroed, s);
+    k_occ_rows<<<nblk(words), 256, 0, s>>>(b.occ, b.occ_words, words, mg, rows);
+    if (volume) {
+        k_crossings<<<nblk(b.ncompact), 256, 0, s>>>(b.vx, b.occ, b.hrng, b.compact, b.ncompact, b.tlist,
+                                                     mg, vbits, entries, error);
+        k_inside_words<<<nblk((int64_t)mg.W * mg.n[1], 128), 128, 0, s>>>(vbits, mg);
     }
-    k_map_cells<false><<<nblk(cells), 256, 0, s>>>(b.geo, b.hrng, b.compact, b.tlist, b.occ, inside, band, inner, mg,
-                                                   surface,
-                                                   volume, sflag, vflag, nullptr, nullptr, 0, 0, nullptr, nullptr,
-                                                   nullptr);
-    exclusive_scan_u32(sflag, soff, cells, tot, scr, sc, s);
-    exclusive_scan_u32(vflag, voff, cells, tot + 1, scr, sc, s);
-    uint32_t counts[2] = {0, 0}, errh = 0;
-    CKM(cudaMemcpyAsync(counts, tot, 8, cudaMemcpyDeviceToHost, s));
-    CKM(cudaMemcpyAsync(&errh, error, 4, cudaMemcpyDeviceToHost, s));
-    CKM(cudaStreamSynchronize(s));
+    auto dilate = [&](uint32_t *out, int r) {
+        k_dilate_x<<<nblk(words), 256, 0, s>>>(rows, t1, words, mg, r);
+        k_dilate_yz<<<nblk(words), 256, 0, s>>>(t1, t2, words, mg, 1, r);
+        k_dilate_yz<<<nblk(words), 256, 0, s>>>(t2, out, words, mg, 2, r);
+    };
+    if (use_band) dilate(band, band_cells);
+    if (use_inner) dilate(inner, band_cells + inner_cells);
+    if (surface)
+        k_surface_cells<<<nblk(b.ncompact), 256, 0, s>>>(b.geo, b.compact, b.ncompact, b.tlist, mg, tri, dist, sbits);
+    k_word_counts<<<nblk(words), 256, 0, s>>>(rows, sbits, inner, words, vbits, cnt);
+    exclusive_scan_u32(cnt, off, 2 * words, tot, tmp, sc, s);
+    uint32_t all = 0, first = 0, errh = 0;
+    auto ok = [&](cudaError_t e) {
+        if (e == cudaSuccess) return true;
+        err = std::string("map_particles: ") + cudaGetErrorString(e);
+        return false;
+    };
+    if (!ok(cudaMemcpyAsync(&all, tot, 4, cudaMemcpyDeviceToHost, s)) ||
+        !ok(cudaMemcpyAsync(&first, off + words, 4, cudaMemcpyDeviceToHost, s)) ||
+        !ok(cudaMemcpyAsync(&errh, error, 4, cudaMemcpyDeviceToHost, s)) || !ok(cudaStreamSynchronize(s))) {
+        cleanup();
+        return 4;
+    }
     if (errh) {
         cleanup();
         err = "map_particles: a grid column crosses more than 256 triangle entries";
         return 6;
     }
-    const int64_t ns = counts[0], nvol = counts[1], N = nf + ns + nvol;
-    int r = g.alloc_particles(N, err);
-    if (r) {
-        cleanup();
-        return r;
+    const int64_t ns = first, nvol = (int64_t)all - ns, N = nf + ns + nvol;
+    if (N != g.d.N || !g.d.pos) {
+        const int r = g.alloc_particles(N, err);
+        if (r) {
+            cleanup();
+            return r;
+        }
+    } else {
+        cudaMemsetAsync(g.d.cert, 0, sizeof(float4) * (size_t)N, s);   // as a new allocation has it
     }
-    int32_t *dcls = nullptr;
-    if (dev_malloc(&dcls, 4 * std::max<int64_t>(N, 1))) {
+    if (band && nvol && dev_malloc(&vcls, (size_t)nvol)) {
         cleanup();
         err = "map_particles: out of device memory";
         return 3;
     }
+    std::vector<float4> p4(nf);
     if (nf) {
-        std::vector<float4> p4(nf);
-        const std::vector<int32_t> &c4 = fseg;   // constraints: the segment of each feature particle
         for (int64_t i = 0; i < nf; i++) {
             uint32_t bits = class_bit(fcls[i]);
             float w;
             memcpy(&w, &bits, 4);
             p4[i] = make_float4(fxyz[3 * i], fxyz[3 * i + 1], fxyz[3 * i + 2], w);
         }
-        CKM(cudaMemcpyAsync(g.d.pos, p4.data(), sizeof(float4) * nf, cudaMemcpyHostToDevice, s));
-        CKM(cudaMemcpyAsync(g.d.cons, c4.data(), sizeof(int32_t) * nf, cudaMemcpyHostToDevice, s));
-        CKM(cudaMemcpyAsync(dcls, fcls.data(), sizeof(int32_t) * nf, cudaMemcpyHostToDevice, s));
-        CKM(cudaStreamSynchronize(s));
+        // (constraints: the segment of each feature particle)
+        if (!ok(cudaMemcpyAsync(g.d.pos, p4.data(), sizeof(float4) * nf, cudaMemcpyHostToDevice, s)) ||
+            !ok(cudaMemcpyAsync(g.d.cons, fseg.data(), sizeof(int32_t) * nf, cudaMemcpyHostToDevice, s))) {
+            cudaStreamSynchronize(s);
+            cleanup();
+            return 4;
+        }
     }
-    k_map_cells<true><<<nblk(cells), 256, 0, s>>>(b.geo, b.hrng, b.compact, b.tlist, b.occ, inside, band, inner, mg,
-                                                  surface,
-                                                  volume, nullptr, nullptr, soff, voff, nf, nf + ns, g.d.pos,
-                                                  g.d.cons, dcls);
-    cls_host.assign(N, 0);
-    if (N) CKM(cudaMemcpyAsync(cls_host.data(), dcls, 4 * N, cudaMemcpyDeviceToHost, s));
-    CKM(cudaStreamSynchronize(s));
-    cudaFree(dcls);
+    if (surface)
+        k_emit_surface<<<nblk(b.ncompact), 256, 0, s>>>(b.geo, b.compact, b.ncompact, tri, dist, sbits, off, mg,
+                                                        g.d.pos + nf, g.d.cons + nf);
+    k_emit_volume<<<nblk(words), 256, 0, s>>>(vbits, off + words, band, words, first, mg, g.d.pos + nf, g.d.cons + nf,
+                                              vcls);
+    std::vector<uint8_t> vc(band ? (size_t)nvol : 0);
+    bool done = vc.empty() || ok(cudaMemcpyAsync(vc.data(), vcls, vc.size(), cudaMemcpyDeviceToHost, s));
+    // the classes on the host: features as given, then S, then V (or as copied)
+    cls_host.resize((size_t)N);
+    std::copy(fcls.begin(), fcls.end(), cls_host.begin());
+    std::fill(cls_host.begin() + nf, cls_host.begin() + nf + ns, (int32_t)kClsS);
+    done = ok(cudaStreamSynchronize(s)) && done && ok(cudaGetLastError());
+    if (vc.empty()) std::fill(cls_host.begin() + nf + ns, cls_host.end(), (int32_t)kClsV);
+    else std::copy(vc.begin(), vc.end(), cls_host.begin() + nf + ns);
     cleanup();
+    if (!done) return 4;
     *n_out = N;
     return 0;
 }
