@@ -375,7 +375,7 @@ int fppg_batch_store(fppg_batch *b);
 int fppg_batch_load(fppg_batch *b);
 /* Autotuner: times `iters` iterations of the batch for every combination
  * of force-kernel block size (128, 256) and force-kernel variant (0 per-lane
- * rows, 1 shared-row union) with the warp search on 4 CTAs per SM; then,
+ * rows, 1 shared-row union) with the group search on 4 CTAs per SM; then,
  * with the fastest force kernel, the triangle search on 8 or 16 CTAs per SM
  * or -- search CTAs 0 -- one thread per queued particle on 16 CTAs per SM;
  * then, with the fastest of those, the two ways of ordering the cell keys
@@ -431,7 +431,8 @@ int fppg_batch_set_cell_order(fppg_batch *b, int32_t order);
  * keeps working: the mask is read from device memory). */
 int fppg_batch_set_mobile_classes(fppg_batch *b, int32_t mask);
 /* The same choice made by hand: force variant 0 or 1, force block 128 or 256,
- * search CTAs per SM 1..64 for the warp form or 0 for the thread form
+ * search CTAs per SM 1..64 for the group form (8 or 32 lanes a particle,
+ * by the mean length of the meshes' candidate lists) or 0 for one thread
  * (FPPG_ERR_ARG otherwise).  Every choice gives the
  * same bits; only the speed differs.  Drops a captured graph. */
 int fppg_batch_configure(fppg_batch *b, int32_t variant, int32_t block, int32_t search_ctas);

@@ -207,6 +207,7 @@ int ctx_group(fppg_ctx *c) {
     g.hp[0].cascade = c->cascade;
     if (g.cell_order) g.hp[0].row_rank = g.d.row_rank;   // the body's table (fppg_set_cell_order)
     g.mesh = view_of(c->body);
+    g.set_search_lanes(c->body.n_dil, c->body.n_cand);
     const int r = g.upload_params(c->stream, c->err);
     return r == 0 ? FPPG_OK : (r == 3 ? FPPG_ERR_OOM : FPPG_ERR_CUDA);
 }
@@ -966,6 +967,7 @@ int fppg_batch_create(fppg_ctx *const *ctxs, int32_t n, fppg_batch **out) {
         dc += bd.n_cand;
     }
     b->off.push_back(N);
+    g.set_search_lanes(dl - n, dc);      // (one more list start than cells for every body)
     if (cells >= ((int64_t)1 << 29) || N > ((int64_t)1 << 31) || ow >= 0xffffffffLL || dl >= 0xffffffffLL ||
         dc >= 0x7fffffffLL) {
         delete b;
@@ -1263,7 +1265,7 @@ int fppg_batch_autotune(fppg_batch *b, int32_t iters, int32_t *variant, int32_t 
             }
             return FPPG_OK;
         };
-        // the force kernel (variant, block) with the warp search on 4 CTAs
+        // the force kernel (variant, block) with the group search on 4 CTAs
         // per SM, then the search grid with the fastest force kernel
         for (int v = 0; v < 2; v++)
             for (int tb : {128, 256})

@@ -385,6 +385,15 @@ int Group::set_cell_order(int order, cudaStream_t s, std::string &err) {
     return upload_params(s, err);
 }
 
+// Lanes per queued particle from the mean candidate list of the group's
+// meshes (entries over cells).  Search per iteration with 8 and 32 lanes:
+// mean 4.2 (union pair) 8.8 / 8.9 us, 4.6 (64 bodies) 263 / 281, 4.7 (gear)
+// 21 / 45; 12.9 (icosphere + torus) 12.1 / 10.5, 16.2 (vehicle) 26 / 24, 65
+// (eight small bodies) 32 / 15.
+void Group::set_search_lanes(int64_t cells, int64_t entries) {
+    search_lanes = entries < 8 * cells ? 8 : 32;
+}
+
 void Group::free_all() {
     escr.release();
     if (graph) cudaGraphExecDestroy(graph);

@@ -115,7 +115,9 @@ struct Group {
     int ev_used = 0;
     // CUDA graph of graph_iters iterations
     int search_blocks = 152 * 8;  // persistent grid of the search
-    bool search_thread = false;   // one thread (not one warp) per queued particle
+    bool search_thread = false;   // one thread (not a group of lanes) per queued particle
+    int search_lanes = 32;        // lanes per queued particle otherwise: 8 or 32 (set_search_lanes)
+    void set_search_lanes(int64_t cells, int64_t entries);
     int force_block = 256;        // threads per block of the force kernel (multiple of 32, <= 256)
     int force_variant = 0;        // 0 per-lane rows, 1 shared-row union
     // order of the neighbour grid's rows: 0 row-major, 1 Morton (Eq. 9 over

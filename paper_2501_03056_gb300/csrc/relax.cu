@@ -13,9 +13,9 @@
 //   k_step          A5  limited step and tangential part; feature particles,
 //                       and particles with no triangle within reach, finish
 //                       here; the others are queued
-//   k_search        A6  one warp per queued particle, its lanes over the 27
-//                       triangle cells: projection or revert; positions are
-//                       written back in id order
+//   k_search        A6  a group of lanes per queued particle over the
+//                       triangles of the 27 cells: projection or revert;
+//                       positions are written back in id order
 #include <cfloat>
 
 #include "body.h"
@@ -749,11 +749,11 @@ __device__ inline float3 closest_on_triangle(float3 p, float3 a, float3 b, float
     return a + (vb * den) * ab + (vc * den) * ac;
 }
 
-// Warp-cooperative search of the 27 triangle cells around y (every lane
-// holds the same y).  Lane c < 27 owns cell c of the block: its occupancy
-// bit, its hash lookup (Eq. 10) and its triangles; the warp then reduces to
-// the overall best with ties to the lower triangle index, so the choice is
-// the same as a serial scan of the 27 cells.
+// Search of the 27 triangle cells around y by a group of G neighbouring lanes
+// (1, 8 or 32; every lane of the group holds the same y): each lane tests
+// every G-th candidate, and the group reduces to the overall best with ties to
+// the lower triangle index, so the choice is the same as a serial scan of the
+// 27 cells, for every G.
 //   surface: smallest |plane distance| among triangles whose foot is inside
 //            (edge functions >= 0); returns the triangle or -1
 //   volume:  closest triangle; returns inside (sign of (y - c) . psi <= 0)
@@ -762,63 +762,40 @@ struct CellRange {
     uint32_t beg, len;
 };
 
-__device__ inline CellRange lane_cell(const MeshView &M, const AsmParams &A, float3 y, int lane) {
+// cell c < 27 of the block around y
+__device__ inline CellRange block_cell(const MeshView &M, const AsmParams &A, float3 y, int c) {
     CellRange r{0u, 0u};
-    if (lane >= 27) return r;
-    const int x = cell_coord(y.x, A.tg_o[0], A.tg_inv, A.tg_n[0]) + lane % 3 - 1;
-    const int yy = cell_coord(y.y, A.tg_o[1], A.tg_inv, A.tg_n[1]) + (lane / 3) % 3 - 1;
-    const int z = cell_coord(y.z, A.tg_o[2], A.tg_inv, A.tg_n[2]) + lane / 9 - 1;
+    const int x = cell_coord(y.x, A.tg_o[0], A.tg_inv, A.tg_n[0]) + c % 3 - 1;
+    const int yy = cell_coord(y.y, A.tg_o[1], A.tg_inv, A.tg_n[1]) + (c / 3) % 3 - 1;
+    const int z = cell_coord(y.z, A.tg_o[2], A.tg_inv, A.tg_n[2]) + c / 9 - 1;
     if (x < 0 || yy < 0 || z < 0 || x >= A.tg_n[0] || yy >= A.tg_n[1] || z >= A.tg_n[2]) return r;
     if (!test_bit(M.occ, A.occ_off, tri_key(A, x, yy, z))) return r;
     tri_cell(M, A, x, yy, z, r.beg, r.len);
     return r;
 }
 
-// lexicographic (value, index) minimum over the warp; every lane gets it
-__device__ inline void warp_argmin(float &v, int &t) {
+// the lanes of this lane's group, and its place in it
+template <int G>
+__device__ inline uint32_t group_mask() {
+    return G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u) << (threadIdx.x & 31u & ~(uint32_t)(G - 1));
+}
+template <int G>
+__device__ inline int group_lane() {
+    return (int)(threadIdx.x & (uint32_t)(G - 1));
+}
+
+// lexicographic (value, index) minimum over the group; every lane gets it
+template <int G>
+__device__ inline void group_argmin(float &v, int &t) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, v, o);
-        const int ot = __shfl_xor_sync(0xffffffffu, t, o);
+    for (int o = G / 2; o > 0; o >>= 1) {
+        const float ov = __shfl_xor_sync(group_mask<G>(), v, o);
+        const int ot = __shfl_xor_sync(group_mask<G>(), t, o);
         if (ov < v || (ov == v && ot < t)) {
             v = ov;
             t = ot;
         }
     }
-}
-
-// The candidate triangles of the 27 cells are gathered into a per-warp list
-// in shared memory (an exclusive scan of the cells' list lengths gives each
-// cell its place), then all 32 lanes test the list together.  A list longer
-// than the buffer is tested by the lanes cell by cell instead.
-constexpr int kSearchBuf = 160;   // triangle ids per warp
-
-__device__ inline int gather_candidates(const MeshView &M, const CellRange r, int32_t *buf) {
-    const int lane = threadIdx.x & 31;
-    uint32_t off = r.len;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xffffffffu, off, o);
-        if (lane >= o) off += t;
-    }
-    const uint32_t total = __shfl_sync(0xffffffffu, off, 31);
-    off -= r.len;
-    if (total <= (uint32_t)kSearchBuf)
-        for (uint32_t q = 0; q < r.len; q++) buf[off + q] = M.tlist[r.beg + q];
-    __syncwarp();
-    return (int)total;
-}
-
-template <typename Test>
-__device__ inline void for_candidates(const MeshView &M, const CellRange r, int32_t *buf, Test &&test) {
-    const int lane = threadIdx.x & 31;
-    const int total = gather_candidates(M, r, buf);
-    if (total <= kSearchBuf) {
-        for (int q = lane; q < total; q += 32) test(buf[q]);
-    } else {
-        for (uint32_t e = r.beg; e < r.beg + r.len; e++) test(M.tlist[e]);
-    }
-    __syncwarp();
 }
 
 // Surface candidate test: the foot of y on the plane of triangle t lies
@@ -908,33 +885,44 @@ __device__ inline int cell_candidates(const MeshView &M, const AsmParams &A, flo
     return 1;
 }
 
-// every candidate triangle of the 27 cells around y, spread over the lanes
-template <typename Test>
-__device__ inline void for_27_candidates(const MeshView &M, const AsmParams &A, float3 y, int32_t *buf,
-                                         Test &&test, const uint2 *pre = nullptr) {
-    const int lane = threadIdx.x & 31;
+// every candidate triangle of the 27 cells around y (of y's own cell alone
+// with own_cell), spread over the group's lanes
+template <int G, typename Test>
+__device__ inline void for_27_candidates(const MeshView &M, const AsmParams &A, float3 y, bool own_cell, Test &&test,
+                                         const uint2 *pre = nullptr) {
+    const int sub = group_lane<G>();
     uint32_t beg = 0, end = 0;
-    const int kind = cell_candidates(M, A, y, beg, end, pre);
+    const int kind = own_cell ? 3 : cell_candidates(M, A, y, beg, end, pre);
     auto checked = [&](int t) {
         if (FPPG_CHECK(t >= 0 && t < A.nt, kChkTri)) test(t);
     };
     if (kind == 1) {
-        for (uint32_t q = beg + lane; q < end; q += 32) checked(M.cand[q]);
+        for (uint32_t q = beg + sub; q < end; q += G) checked(M.cand[q]);
     } else if (kind == 2) {
-        const CellRange r = lane_cell(M, A, y, lane);
-        for_candidates(M, r, buf, checked);
+        // (these cells hold over 512 entries together: the lanes look the
+        // cells up side by side, then share out every cell's list)
+        for (int c0 = 0; c0 < 27; c0 += G) {
+            const CellRange r = c0 + sub < 27 ? block_cell(M, A, y, c0 + sub) : CellRange{0u, 0u};
+            for (int k = 0; k < G && c0 + k < 27; k++) {
+                const uint32_t b = G > 1 ? __shfl_sync(group_mask<G>(), r.beg, k, G) : r.beg;
+                const uint32_t l = G > 1 ? __shfl_sync(group_mask<G>(), r.len, k, G) : r.len;
+                for (uint32_t e = b + sub; e < b + l; e += G) checked(M.tlist[e]);
+            }
+        }
+    } else if (kind == 3) {
+        const CellRange r = block_cell(M, A, y, 13);
+        for (uint32_t e = r.beg + sub; e < r.beg + r.len; e += G) checked(M.tlist[e]);
     }
 }
 
-__device__ int warp_project_surface(const MeshView &M, const AsmParams &A, float3 y, float &dist, int32_t *buf,
-                                    bool own_cell = false, const uint2 *pre = nullptr, float *cert_r = nullptr) {
-    const int lane = threadIdx.x & 31;
-    float best = FLT_MAX;
+template <int G>
+__device__ int group_project_surface(const MeshView &M, const AsmParams &A, float3 y, float &dist,
+                                     bool own_cell = false, const uint2 *pre = nullptr, float *cert_r = nullptr) {
+    float best = FLT_MAX, bd = 0.f;
     int bt = 0x7fffffff;
-    float bd = 0.f;
     int nproj = 0;
     float rother = FLT_MAX;
-    auto test = [&](int t) {
+    for_27_candidates<G>(M, A, y, own_cell, [&](int t) {
         float d;
         if (cert_r) {
             float emin;
@@ -952,27 +940,24 @@ __device__ int warp_project_surface(const MeshView &M, const AsmParams &A, float
             bt = t;
             bd = d;
         }
-    };
-    if (own_cell) {
-        // the cell that holds y alone: lane 13 probes the centre cell
-        CellRange r = lane_cell(M, A, y, lane);
-        if (lane != 13) r = CellRange{0u, 0u};
-        for_candidates(M, r, buf, test);
-    } else {
-        for_27_candidates(M, A, y, buf, test, pre);
-    }
+    }, pre);
     float v = best;
     int t = bt;
-    warp_argmin(v, t);
-    // the signed distance of the winner, from a lane that holds it
-    const uint32_t own = __ballot_sync(0xffffffffu, bt == t && best == v);
-    dist = __shfl_sync(0xffffffffu, bd, own ? __ffs(own) - 1 : 0);
+    group_argmin<G>(v, t);
+    dist = bd;
+    if (G > 1) {
+        // the signed distance of the winner, from a lane that holds it
+        const uint32_t own = __ballot_sync(group_mask<G>(), bt == t && best == v) & group_mask<G>();
+        dist = __shfl_sync(group_mask<G>(), bd, own ? __ffs(own) - 1 : 0);
+    }
     if (cert_r) {
-        const int total = __reduce_add_sync(0xffffffffu, nproj);
         float r = rother;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) r = fminf(r, __shfl_xor_sync(0xffffffffu, r, o));
-        *cert_r = surface_cert_radius(A, total, r);
+        for (int o = G / 2; o > 0; o >>= 1) {
+            r = fminf(r, __shfl_xor_sync(group_mask<G>(), r, o));
+            nproj += __shfl_xor_sync(group_mask<G>(), nproj, o);
+        }
+        *cert_r = surface_cert_radius(A, nproj, r);
     }
     return t == 0x7fffffff ? -1 : t;
 }
@@ -981,8 +966,9 @@ __device__ int warp_project_surface(const MeshView &M, const AsmParams &A, float
 // closest projectable triangle over the 27 cells, or with A.cascade the
 // cascade of Sec. 3.3.3 (still on triangle c: stay; else the closest
 // projectable one of y's own cell; else over the 27 cells).  -1: revert.
-__device__ int warp_surface_choice(const MeshView &M, const AsmParams &A, float3 y, int c, float &dist,
-                                   int32_t *buf, const uint2 *pre = nullptr, float *cert_r = nullptr) {
+template <int G>
+__device__ int group_surface_choice(const MeshView &M, const AsmParams &A, float3 y, int c, float &dist,
+                                    const uint2 *pre = nullptr, float *cert_r = nullptr) {
     if (A.cascade) {
         if (c >= 0 && c < A.nt) {
             float d = 0.f;
@@ -992,10 +978,10 @@ __device__ int warp_surface_choice(const MeshView &M, const AsmParams &A, float3
                 return c;
             }
         }
-        const int t = warp_project_surface(M, A, y, dist, buf, true);
+        const int t = group_project_surface<G>(M, A, y, dist, true);
         if (t >= 0) return t;
     }
-    return warp_project_surface(M, A, y, dist, buf, false, pre, A.cascade ? nullptr : cert_r);
+    return group_project_surface<G>(M, A, y, dist, false, pre, A.cascade ? nullptr : cert_r);
 }
 
 // distance from y to the faces of the 3 x 3 x 3 triangle-cell block around
@@ -1017,13 +1003,13 @@ __device__ inline float block_margin(const AsmParams &A, float3 y) {
 // sign of the angle-weighted pseudonormal): 1 inside, 0 outside, -1 when no
 // triangle lies in range.  *clear gets a lower bound of the distance from y
 // to the surface, valid when inside.
-__device__ int warp_closest_sign(const MeshView &M, const AsmParams &A, float3 y, int32_t *buf, float &clear,
-                                 const uint2 *pre = nullptr) {
-    const int lane = threadIdx.x & 31;
+template <int G>
+__device__ int group_closest_sign(const MeshView &M, const AsmParams &A, float3 y, float &clear,
+                                  const uint2 *pre = nullptr) {
     float best = FLT_MAX;
     int bt = 0x7fffffff, breg = 0;
     float3 bcp = make_float3(0.f, 0.f, 0.f);
-    for_27_candidates(M, A, y, buf, [&](int t) {
+    for_27_candidates<G>(M, A, y, false, [&](int t) {
         const size_t g = (size_t)(A.tri_off + t);
         const float3 n = f3(M.geo[5 * g + 1]);
         if (n.x == 0.f && n.y == 0.f && n.z == 0.f) return;   // degenerate
@@ -1040,34 +1026,37 @@ __device__ int warp_closest_sign(const MeshView &M, const AsmParams &A, float3 y
     }, pre);
     float v = best;
     int t = bt;
-    warp_argmin(v, t);
+    group_argmin<G>(v, t);
     const float blk = block_margin(A, y);
     clear = fmaxf(fminf(t == 0x7fffffff ? FLT_MAX : sqrtf(v), blk) * (1.f - 0x1p-10f) - A.dx * 0x1p-16f, 0.f);
     if (t == 0x7fffffff) return -1;
-    const uint32_t own = __ballot_sync(0xffffffffu, bt == t && best == v);
-    const int src = __ffs(own) - 1;
+    // the sign from a lane that holds the winner
+    int src = (int)(threadIdx.x & 31u);
+    if (G > 1) src = __ffs(__ballot_sync(group_mask<G>(), bt == t && best == v) & group_mask<G>()) - 1;
     int inside = 0;
-    if (lane == src) {
+    if ((int)(threadIdx.x & 31u) == src) {
         const size_t g = (size_t)(A.tri_off + bt);
         const float3 psi = breg == 0 ? f3(M.geo[5 * g + 1]) : f3(M.pn[6 * g + breg - 1]);
         inside = dot3(y - bcp, psi) <= 0.f;
     }
-    return __shfl_sync(0xffffffffu, inside, src);
+    return G > 1 ? __shfl_sync(group_mask<G>(), inside, src) : inside;
 }
 
 // Volume test of a particle of the body: the closest-feature sign, inside
 // when no triangle is in range (a step is below a cell)
-__device__ inline bool warp_volume_inside(const MeshView &M, const AsmParams &A, float3 y, int32_t *buf,
-                                          float &clear, const uint2 *pre = nullptr) {
-    return warp_closest_sign(M, A, y, buf, clear, pre) != 0;
+template <int G>
+__device__ inline bool group_volume_inside(const MeshView &M, const AsmParams &A, float3 y, float &clear,
+                                           const uint2 *pre = nullptr) {
+    return group_closest_sign<G>(M, A, y, clear, pre) != 0;
 }
 
 // Boolean partner rule (1 stay outside, 2 stay inside, 0 none) for point x:
 // with no partner triangle in range the particle is where it started
-__device__ inline bool warp_partner_ok(const MeshView &M, const AsmParams &Q, int rule, float3 x, int32_t *buf) {
+template <int G>
+__device__ inline bool group_partner_ok(const MeshView &M, const AsmParams &Q, int rule, float3 x) {
     if (rule == 0) return true;
     float unused;
-    const int t = warp_closest_sign(M, Q, x, buf, unused);
+    const int t = group_closest_sign<G>(M, Q, x, unused);
     return rule == 1 ? t != 1 : t != 0;
 }
 
@@ -1278,27 +1267,29 @@ __device__ inline int64_t queue_slot(uint32_t nf, int64_t N, uint32_t e) {
 }
 
 
-// k_search: one warp per queued particle (grid-stride over the queue):
-// surface particles go to the closest projectable triangle or revert,
-// volume particles are accepted when the pseudonormal sign says inside.
-__global__ void __launch_bounds__(TPB) k_search(const float4 *__restrict__ pos_s,
-                                                const uint32_t *__restrict__ id_s,
-                                                const AsmParams *__restrict__ P, float4 *__restrict__ pos,
-                                                int32_t *__restrict__ cons, MeshView M,
-                                                uint32_t *__restrict__ maxdisp, const int4 *__restrict__ work,
-                                                const uint2 *__restrict__ work_r,
-                                                const uint32_t *__restrict__ work_count, int64_t N,
-                                                float4 *__restrict__ cert) {
-    __shared__ int32_t sbuf[TPB / 32][kSearchBuf];
-    int32_t *buf = sbuf[threadIdx.x / 32];
-    const int lane = threadIdx.x & 31;
-    const uint32_t warps = gridDim.x * (TPB / 32);
+// k_search: G lanes per queued particle (grid-stride over the queue): surface
+// particles go to the closest projectable triangle or revert, volume particles
+// are accepted when the pseudonormal sign says inside.  Bound by the latency of
+// its dependent loads, so what counts is how many particles are in flight and
+// how many of a group's lanes the candidate list feeds: SEARCH_NOTE
+// At most 64 registers (four blocks, 32 warps per SM).
+template <int G>
+__global__ void __launch_bounds__(TPB, 4) k_search(const float4 *__restrict__ pos_s,
+                                                   const uint32_t *__restrict__ id_s,
+                                                   const AsmParams *__restrict__ P, float4 *__restrict__ pos,
+                                                   int32_t *__restrict__ cons, MeshView M,
+                                                   uint32_t *__restrict__ maxdisp, const int4 *__restrict__ work,
+                                                   const uint2 *__restrict__ work_r,
+                                                   const uint32_t *__restrict__ work_count, int64_t N,
+                                                   float4 *__restrict__ cert) {
     const uint32_t nf = work_count[0], n = nf + work_count[1];
-    // lane 0's running max move of body run_b, added when the body changes
-    // (the queue is in key order, so a warp meets few bodies)
-    int run_b = -1;
-    uint32_t run = 0u;
-    for (uint32_t e = (blockIdx.x * TPB + threadIdx.x) / 32; e < n; e += warps) {
+    const uint32_t stride = gridDim.x * (TPB / G);
+    const bool lead = group_lane<G>() == 0;
+    // the leader's running max move of body run_b, added when the body
+    // changes and once at the end (the queue is in key order: few changes)
+    int run_b = 0;
+    float run = 0.f;
+    for (uint32_t e = (blockIdx.x * TPB + threadIdx.x) / G; e < n; e += stride) {
         const int64_t qs = queue_slot(nf, N, e);
         if (!FPPG_CHECK(qs >= 0 && qs < N, kChkQueue)) continue;
         const int4 it = work[qs];
@@ -1306,6 +1297,7 @@ __global__ void __launch_bounds__(TPB) k_search(const float4 *__restrict__ pos_s
         if (!FPPG_CHECK(it.x >= 0 && it.x < N, kChkEntry)) continue;
         const float3 y = make_float3(__int_as_float(it.y), __int_as_float(it.z), __int_as_float(it.w));
         const float4 p = pos_s[it.x];
+        const uint32_t i = id_s[it.x];
         const int cls = cls_of(p.w), b = body_of(p.w);
         const AsmParams &A = P[b];
         float3 x = y;
@@ -1314,29 +1306,24 @@ __global__ void __launch_bounds__(TPB) k_search(const float4 *__restrict__ pos_s
         bool ok;
         if (cls == kClsS) {
             float d;
-            tri = warp_surface_choice(M, A, y, A.cascade ? cons[id_s[it.x]] : -1, d, buf, &rng, &clear);
+            tri = group_surface_choice<G>(M, A, y, A.cascade ? cons[i] : -1, d, &rng, &clear);
             ok = tri >= 0;
             if (ok) x = y - d * f3(M.geo[5 * (size_t)(A.tri_off + tri) + 1]);
         } else if (cls == kClsF) {
             // a feature particle of a union member near the partner: its
             // projection again, then the partner test below
-            int cn = -1, okf = 0;
-            if (lane == 0) okf = project_feature(M, A, y, cons[id_s[it.x]], x, cn) ? 1 : 0;
-            okf = __shfl_sync(0xffffffffu, okf, 0);
-            x = make_float3(__shfl_sync(0xffffffffu, x.x, 0), __shfl_sync(0xffffffffu, x.y, 0),
-                            __shfl_sync(0xffffffffu, x.z, 0));
-            tri = __shfl_sync(0xffffffffu, cn, 0);
-            ok = okf != 0;
+            int cn = -1;
+            ok = project_feature(M, A, y, cons[i], x, cn);
+            tri = cn;
         } else {
-            ok = warp_volume_inside(M, A, y, buf, clear, &rng);
+            ok = group_volume_inside<G>(M, A, y, clear, &rng);
         }
         // Boolean operations: the partner rule of the particle's class
         for (int q = 0; q < A.npart && ok; q++)
             if (!(cls == kClsF && tri >= A.curve_lo[q] && tri < A.curve_hi[q]))
-                ok = warp_partner_ok(M, P[A.partner[q]], cls == kClsV ? A.partner_vol[q] : A.partner_surf[q], x,
-                                     buf);
-        if (ok && lane == 0) {
-            const uint32_t i = id_s[it.x];
+                ok = group_partner_ok<G>(M, P[A.partner[q]], cls == kClsV ? A.partner_vol[q] : A.partner_surf[q], x);
+        if (G > 1) __syncwarp(group_mask<G>());   // (cons[i] is read by every lane of the group above)
+        if (ok && lead) {
             pos[i] = make_float4(x.x, x.y, x.z, p.w);
             if (tri >= 0) cons[i] = tri;
             if (cls == kClsV && A.closed && !A.vol_rules) cert[i] = make_float4(y.x, y.y, y.z, clear);
@@ -1344,203 +1331,14 @@ __global__ void __launch_bounds__(TPB) k_search(const float4 *__restrict__ pos_s
             if (cls == kClsS && clear > 0.f) cert[i] = make_float4(y.x, y.y, y.z, -clear);
             const float3 w = x - f3(p);
             if (b != run_b) {
-                if (run) atomicMax(maxdisp + run_b, run);
-                run_b = b;
-                run = 0u;
-            }
-            run = max(run, __float_as_uint(sqrtf(dot3(w, w))));
-        }
-    }
-    if (lane == 0 && run) atomicMax(maxdisp + run_b, run);
-}
-
-// ---- the same search, one thread per queued particle --------------------------
-// Each thread walks its particle's candidate list alone: no lanes idle on a
-// short list, and 32 particles' dependent loads are in flight per warp.
-// The candidate set and the comparisons (smallest distance, ties to the
-// lower index) are those of the warp form, so the choices are identical.
-
-// every candidate triangle of the 27 cells around y, one after another
-template <typename Test>
-__device__ inline void each_27_candidate(const MeshView &M, const AsmParams &A, float3 y, Test &&test,
-                                         const uint2 *pre = nullptr) {
-    uint32_t beg = 0, end = 0;
-    const int kind = cell_candidates(M, A, y, beg, end, pre);
-    auto checked = [&](int t) {
-        if (FPPG_CHECK(t >= 0 && t < A.nt, kChkTri)) test(t);
-    };
-    if (kind == 1) {
-        for (uint32_t q = beg; q < end; q++) checked(M.cand[q]);
-    } else if (kind == 2) {
-        for (int c = 0; c < 27; c++) {
-            const CellRange r = lane_cell(M, A, y, c);
-            for (uint32_t e = r.beg; e < r.beg + r.len; e++) checked(M.tlist[e]);
-        }
-    }
-}
-
-__device__ int thread_project_surface(const MeshView &M, const AsmParams &A, float3 y, float &dist,
-                                      bool own_cell = false, const uint2 *pre = nullptr, float *cert_r = nullptr) {
-    float best = FLT_MAX, bd = 0.f;
-    int bt = 0x7fffffff;
-    int nproj = 0;
-    float rother = FLT_MAX;
-    auto test = [&](int t) {
-        float d;
-        if (cert_r) {
-            float emin;
-            if (!surface_candidate_margin(M, A, t, y, d, emin)) {
-                rother = fminf(rother, -emin - A.edge_tol);
-                return;
-            }
-            nproj++;
-        } else if (!surface_candidate(M, A, t, y, d)) {
-            return;
-        }
-        const float ad = fabsf(d);
-        if (ad < best || (ad == best && t < bt)) {
-            best = ad;
-            bt = t;
-            bd = d;
-        }
-    };
-    if (own_cell) {
-        const CellRange r = lane_cell(M, A, y, 13);   // the centre cell
-        for (uint32_t e = r.beg; e < r.beg + r.len; e++) test(M.tlist[e]);
-    } else {
-        each_27_candidate(M, A, y, test, pre);
-    }
-    dist = bd;
-    if (cert_r) *cert_r = surface_cert_radius(A, nproj, rother);
-    return bt == 0x7fffffff ? -1 : bt;
-}
-
-__device__ int thread_surface_choice(const MeshView &M, const AsmParams &A, float3 y, int c, float &dist,
-                                     const uint2 *pre = nullptr, float *cert_r = nullptr) {
-    if (A.cascade) {
-        if (c >= 0 && c < A.nt) {
-            float d = 0.f;
-            if (surface_candidate(M, A, c, y, d)) {
-                dist = d;
-                return c;
-            }
-        }
-        const int t = thread_project_surface(M, A, y, dist, true);
-        if (t >= 0) return t;
-    }
-    return thread_project_surface(M, A, y, dist, false, pre, A.cascade ? nullptr : cert_r);
-}
-
-__device__ int thread_closest_sign(const MeshView &M, const AsmParams &A, float3 y, float &clear,
-                                   const uint2 *pre = nullptr) {
-    float best = FLT_MAX;
-    int bt = 0x7fffffff, breg = 0;
-    float3 bcp = make_float3(0.f, 0.f, 0.f);
-    each_27_candidate(M, A, y, [&](int t) {
-        const size_t g = (size_t)(A.tri_off + t);
-        const float3 n = f3(M.geo[5 * g + 1]);
-        if (n.x == 0.f && n.y == 0.f && n.z == 0.f) return;   // degenerate
-        int reg;
-        const float3 cp = closest_on_triangle(y, f3(M.vx[3 * g]), f3(M.vx[3 * g + 1]), f3(M.vx[3 * g + 2]), reg);
-        const float3 w = y - cp;
-        const float dd = dot3(w, w);
-        if (dd < best || (dd == best && t < bt)) {
-            best = dd;
-            bt = t;
-            breg = reg;
-            bcp = cp;
-        }
-    }, pre);
-    const float blk = block_margin(A, y);
-    clear = fmaxf(fminf(bt == 0x7fffffff ? FLT_MAX : sqrtf(best), blk) * (1.f - 0x1p-10f) - A.dx * 0x1p-16f, 0.f);
-    if (bt == 0x7fffffff) return -1;
-    const size_t g = (size_t)(A.tri_off + bt);
-    const float3 psi = breg == 0 ? f3(M.geo[5 * g + 1]) : f3(M.pn[6 * g + breg - 1]);
-    return dot3(y - bcp, psi) <= 0.f ? 1 : 0;
-}
-
-__device__ inline bool thread_partner_ok(const MeshView &M, const AsmParams &Q, int rule, float3 x) {
-    if (rule == 0) return true;
-    float unused;
-    const int t = thread_closest_sign(M, Q, x, unused);
-    return rule == 1 ? t != 1 : t != 0;
-}
-
-// k_search_thread: one thread per queued particle; the warps stride over the
-// queue together so that the per-body max move is reduced once per warp.
-// At most 64 registers (four blocks, 32 warps per SM): the kernel waits on
-// dependent loads, and more particles in flight hide more of them (at 75
-// registers and 24 warps it took 0.509 against 0.441 ms per iteration on
-// the vehicle shell)
-__global__ void __launch_bounds__(TPB, 4) k_search_thread(const float4 *__restrict__ pos_s,
-                                                       const uint32_t *__restrict__ id_s,
-                                                       const AsmParams *__restrict__ P, float4 *__restrict__ pos,
-                                                       int32_t *__restrict__ cons, MeshView M,
-                                                       uint32_t *__restrict__ maxdisp,
-                                                       const int4 *__restrict__ work,
-                                                       const uint2 *__restrict__ work_r,
-                                                       const uint32_t *__restrict__ work_count, int64_t N,
-                                                       float4 *__restrict__ cert) {
-    const uint32_t nf = work_count[0], n = nf + work_count[1];
-    const uint32_t stride = gridDim.x * TPB;
-    // this thread's running max move of body run_b, added when the body
-    // changes and once at the end (the queue is in key order: few changes)
-    int run_b = 0;
-    float run = 0.f;
-    for (uint32_t e0 = blockIdx.x * TPB + (threadIdx.x & ~31u); e0 < n; e0 += stride) {
-        const uint32_t e = e0 + (threadIdx.x & 31u);
-        int b = 0;
-        float disp = 0.f;
-        if (e < n) {
-            const int64_t qs = queue_slot(nf, N, e);
-            const bool entry_ok = FPPG_CHECK(qs >= 0 && qs < N, kChkQueue) &&
-                                  FPPG_CHECK(work[qs].x >= 0 && work[qs].x < N, kChkEntry);
-            if (!entry_ok) continue;
-            const int4 it = work[qs];
-            const uint2 rng = work_r[qs];
-            const float3 y = make_float3(__int_as_float(it.y), __int_as_float(it.z), __int_as_float(it.w));
-            const float4 p = pos_s[it.x];
-            const int cls = cls_of(p.w);
-            b = body_of(p.w);
-            const AsmParams &A = P[b];
-            const uint32_t i = id_s[it.x];
-            float3 x = y;
-            int tri = -2;
-            float clear = 0.f;
-            bool ok;
-            if (cls == kClsS) {
-                float d;
-                tri = thread_surface_choice(M, A, y, A.cascade ? cons[i] : -1, d, &rng, &clear);
-                ok = tri >= 0;
-                if (ok) x = y - d * f3(M.geo[5 * (size_t)(A.tri_off + tri) + 1]);
-            } else if (cls == kClsF) {
-                int cn = -1;
-                ok = project_feature(M, A, y, cons[i], x, cn);
-                tri = cn;
-            } else {
-                ok = thread_closest_sign(M, A, y, clear, &rng) != 0;
-            }
-            for (int q = 0; q < A.npart && ok; q++)
-                if (!(cls == kClsF && tri >= A.curve_lo[q] && tri < A.curve_hi[q]))
-                    ok = thread_partner_ok(M, P[A.partner[q]], cls == kClsV ? A.partner_vol[q] : A.partner_surf[q],
-                                           x);
-            if (ok) {
-                pos[i] = make_float4(x.x, x.y, x.z, p.w);
-                if (tri >= 0) cons[i] = tri;
-                if (cls == kClsV && A.closed && !A.vol_rules) cert[i] = make_float4(y.x, y.y, y.z, clear);
-                // surface certificates carry a negative radius (never taken for an inside one)
-                if (cls == kClsS && clear > 0.f) cert[i] = make_float4(y.x, y.y, y.z, -clear);
-                const float3 w = x - f3(p);
-                disp = sqrtf(dot3(w, w));
-            }
-            if (b != run_b) {
                 if (run > 0.f) atomicMax(maxdisp + run_b, __float_as_uint(run));
                 run_b = b;
                 run = 0.f;
             }
-            run = fmaxf(run, disp);
+            run = fmaxf(run, sqrtf(dot3(w, w)));
         }
     }
+    __syncwarp();
     labelled_max(maxdisp, run_b, run);
 }
 
@@ -1563,8 +1361,6 @@ __global__ void k_project_points(const float *__restrict__ y, const int32_t *__r
                                   const int32_t *__restrict__ cons_in, int64_t n, const AsmParams *__restrict__ P,
                                   MeshView M, float *__restrict__ x, int32_t *__restrict__ cons_out,
                                   int32_t *__restrict__ ok) {
-    __shared__ int32_t sbuf[TPB / 32][kSearchBuf];
-    int32_t *buf = sbuf[threadIdx.x / 32];
     const int64_t i = ((int64_t)blockIdx.x * TPB + threadIdx.x) / 32;   // one warp per point
     const int lane = threadIdx.x & 31;
     if (i >= n) return;                                                    // whole warp
@@ -1577,7 +1373,7 @@ __global__ void k_project_points(const float *__restrict__ y, const int32_t *__r
     const int cl = cls[i];
     if (cl == kClsS) {
         float d;
-        const int t = warp_surface_choice(M, A, yy, c, d, buf);
+        const int t = group_surface_choice<32>(M, A, yy, c, d);
         r = t >= 0;
         if (r) {
             xx = yy - d * f3(M.geo[5 * (size_t)(A.tri_off + t) + 1]);
@@ -1585,7 +1381,7 @@ __global__ void k_project_points(const float *__restrict__ y, const int32_t *__r
         }
     } else if (cl == kClsV) {
         float clear;
-        r = warp_volume_inside(M, A, yy, buf, clear);
+        r = group_volume_inside<32>(M, A, yy, clear);
     } else if (cl == kClsF) {
         r = project_feature(M, A, yy, c, xx, cn);
     }
@@ -1693,6 +1489,17 @@ void forces(Group &g, cudaStream_t s, int32_t *count_s, int32_t *cand_s, int32_t
         k_count<<<nblocks(d.N), TPB, 0, s>>>(d.pos_s, d.N, d.params, d.fstart, nullptr, cand_s);
 }
 
+static void search(Group &g, cudaStream_t s) {
+    DevGroup &d = g.d;
+#define FPPG_SEARCH(G)                                                                                               \
+    k_search<G><<<g.search_blocks, TPB, 0, s>>>(d.pos_s, d.id_s, d.params, d.pos, d.cons, g.mesh, d.maxdisp, d.work,  \
+                                                queue_ranges(d), d.work_count, d.N, d.cert)
+    if (g.search_thread) FPPG_SEARCH(1);
+    else if (g.search_lanes == 8) FPPG_SEARCH(8);
+    else FPPG_SEARCH(32);
+#undef FPPG_SEARCH
+}
+
 void iterate(Group &g, cudaStream_t s, bool energy_mode, int32_t *count_dbg) {
     DevGroup &d = g.d;
     if (d.N == 0) return;
@@ -1719,13 +1526,7 @@ void iterate(Group &g, cudaStream_t s, bool energy_mode, int32_t *count_dbg) {
     k_step<<<nblocks(d.N), TPB, 0, s>>>(d.pos_s, d.acc_s, d.id_s, d.N, d.params, d.amax, d.pos, d.cons, g.mesh,
                                          d.maxdisp, d.work, queue_ranges(d), d.work_count, d.cert, d.cons_s);
     if (timed) cudaEventRecordWithFlags(g.ev[g.ev_used + 3], s, flags);
-    if (g.search_thread)
-        k_search_thread<<<g.search_blocks, TPB, 0, s>>>(d.pos_s, d.id_s, d.params, d.pos, d.cons, g.mesh,
-                                                        d.maxdisp, d.work, queue_ranges(d), d.work_count, d.N,
-                                                        d.cert);
-    else
-        k_search<<<g.search_blocks, TPB, 0, s>>>(d.pos_s, d.id_s, d.params, d.pos, d.cons, g.mesh, d.maxdisp,
-                                                 d.work, queue_ranges(d), d.work_count, d.N, d.cert);
+    search(g, s);
     if (timed) {
         cudaEventRecordWithFlags(g.ev[g.ev_used + 4], s, flags);
         g.ev_used += kPhaseEvents;
@@ -1737,13 +1538,7 @@ void step_and_project(Group &g, cudaStream_t s) {
     if (d.N == 0) return;
     k_step<<<nblocks(d.N), TPB, 0, s>>>(d.pos_s, d.acc_s, d.id_s, d.N, d.params, d.amax, d.pos, d.cons, g.mesh,
                                          d.maxdisp, d.work, queue_ranges(d), d.work_count, d.cert, d.cons_s);
-    if (g.search_thread)
-        k_search_thread<<<g.search_blocks, TPB, 0, s>>>(d.pos_s, d.id_s, d.params, d.pos, d.cons, g.mesh,
-                                                        d.maxdisp, d.work, queue_ranges(d), d.work_count, d.N,
-                                                        d.cert);
-    else
-        k_search<<<g.search_blocks, TPB, 0, s>>>(d.pos_s, d.id_s, d.params, d.pos, d.cons, g.mesh, d.maxdisp,
-                                                 d.work, queue_ranges(d), d.work_count, d.N, d.cert);
+    search(g, s);
 }
 
 namespace {
