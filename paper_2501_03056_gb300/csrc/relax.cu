@@ -1060,22 +1060,24 @@ __device__ inline bool group_partner_ok(const MeshView &M, const AsmParams &Q, i
     return rule == 1 ? t != 1 : t != 0;
 }
 
-// closest point of the particle's feature line (all lines of the body when
-// it has none yet); ties to the lower segment
-__device__ bool project_feature(const MeshView &M, const AsmParams &A, float3 y, int cons, float3 &x, int &seg) {
-    if (A.nseg <= 0) return false;
-    int s0 = 0, s1 = A.nseg;
-    if (cons >= 0 && cons < A.nseg) {
-        const int line = __float_as_int(M.seg[3 * (size_t)(A.seg_off + cons)].w);
-        const int2 L = M.lines[A.line_off + line];
-        s0 = L.x;
-        s1 = L.x + L.y;
-    }
-    float best = FLT_MAX;
-    int bs = -1;
-    float3 bq = y;
-    for (int s = s0; s < s1; s++) {
-        const float4 *sg = M.seg + 3 * (size_t)(A.seg_off + s);
+// the segments [x, y) a feature particle projects onto: its own line's, all of
+// the body's when it has none yet
+__device__ inline int2 line_segments(const MeshView &M, const AsmParams &A, int cons) {
+    if (cons < 0 || cons >= A.nseg) return make_int2(0, max(A.nseg, 0));
+    const int line = __float_as_int(M.seg[3 * (size_t)(A.seg_off + cons)].w);
+    const int2 L = M.lines[A.line_off + line];
+    return make_int2(L.x, L.x + L.y);
+}
+
+// the closest point of segments r.x + first, r.x + first + step, ..: best
+// squared distance, segment (ties to the lower one; -1 for none) and point
+__device__ inline void closest_on_segments(const float4 *seg, int seg_off, float3 y, int2 r, int first, int step,
+                                           float &best, int &bs, float3 &bq) {
+    best = FLT_MAX;
+    bs = -1;
+    bq = y;
+    for (int s = r.x + first; s < r.y; s += step) {
+        const float4 *sg = seg + 3 * (size_t)(seg_off + s);
         const float3 a = f3(sg[0]), e = f3(sg[1]) - a;
         const float ee = dot3(e, e);
         float t = ee > 0.f ? dot3(y - a, e) / ee : 0.f;
@@ -1089,9 +1091,27 @@ __device__ bool project_feature(const MeshView &M, const AsmParams &A, float3 y,
             bq = q;
         }
     }
-    x = bq;
-    seg = bs;
-    return bs >= 0;
+}
+
+// the same over a group of G lanes that hold the same y and r: every lane
+// gets the closest of all
+template <int G>
+__device__ bool group_project_feature(const float4 *segs, int seg_off, float3 y, int2 r, float3 &x, int &seg) {
+    float best;
+    closest_on_segments(segs, seg_off, y, r, group_lane<G>(), G, best, seg, x);
+    if (G > 1) {
+        float v = best;
+        int t = seg < 0 ? 0x7fffffff : seg;
+        const int mine = t;
+        group_argmin<G>(v, t);
+        const uint32_t own = __ballot_sync(group_mask<G>(), mine == t) & group_mask<G>();
+        const int src = __ffs(own) - 1;     // (none anywhere: every lane, with its y)
+        x.x = __shfl_sync(group_mask<G>(), x.x, src);
+        x.y = __shfl_sync(group_mask<G>(), x.y, src);
+        x.z = __shfl_sync(group_mask<G>(), x.z, src);
+        seg = t == 0x7fffffff ? -1 : t;
+    }
+    return seg >= 0;
 }
 
 // some triangle of body Q within the 27 triangle cells of x (its dilated
@@ -1103,10 +1123,13 @@ __device__ inline bool near_body(const MeshView &M, const AsmParams &Q, float3 x
                             cell_coord(x.z, Q.tg_o[2], Q.tg_inv, Q.tg_n[2])));
 }
 
+// segments of a feature line that the step walks itself
+constexpr int kLaneSegments = 8;
+
 // ---- A5 + A6 -------------------------------------------------------------------
 // k_step: one thread per particle (key order): the limited step and its
-// tangential part, then the cases that need no triangle search -- feature
-// particles (their own line), volume particles with no triangle in the 27
+// tangential part, then the cases that need no search -- feature particles
+// of short lines, volume particles with no triangle in the 27
 // cells (accepted), surface particles with none (reverted).  Every other
 // particle is queued with its trial point for k_search.
 __global__ void __launch_bounds__(TPB, 5) k_step(const float4 *__restrict__ pos_s, const float4 *__restrict__ acc_s,
@@ -1145,9 +1168,17 @@ __global__ void __launch_bounds__(TPB, 5) k_step(const float4 *__restrict__ pos_
         const float3 p3 = f3(p);
         y = p3 + dr;
         if (cls == kClsF) {
+            // a long line goes to the search, whose lanes share its segments
+            // (one lane on a rim of 240 segments kept its warp here for over
+            // 10,000 instructions: the step of the gear, 2.4 M particles,
+            // 142 -> 76 us, its search 21 -> 37)
+            const int2 line = line_segments(M, A, c);
             float3 x;
-            int cn;
-            if (project_feature(M, A, y, c, x, cn)) {
+            int cn = -1;
+            float best;
+            if (line.y - line.x > kLaneSegments) queue = true;
+            else closest_on_segments(M.seg, A.seg_off, y, line, 0, 1, best, cn, x);
+            if (cn >= 0) {
                 // a partner's triangles within reach: the search tests that
                 // partner's rule on the projection (a particle on the
                 // intersection curve with a partner lies on both surfaces:
@@ -1310,11 +1341,9 @@ __global__ void __launch_bounds__(TPB, 4) k_search(const float4 *__restrict__ po
             ok = tri >= 0;
             if (ok) x = y - d * f3(M.geo[5 * (size_t)(A.tri_off + tri) + 1]);
         } else if (cls == kClsF) {
-            // a feature particle of a union member near the partner: its
-            // projection again, then the partner test below
-            int cn = -1;
-            ok = project_feature(M, A, y, cons[i], x, cn);
-            tri = cn;
+            // a feature particle of a long line, or of a union member near
+            // the partner: its projection (again), then the partner test below
+            ok = group_project_feature<G>(M.seg, A.seg_off, y, line_segments(M, A, cons[i]), x, tri);
         } else {
             ok = group_volume_inside<G>(M, A, y, clear, &rng);
         }
@@ -1383,7 +1412,7 @@ __global__ void k_project_points(const float *__restrict__ y, const int32_t *__r
         float clear;
         r = group_volume_inside<32>(M, A, yy, clear);
     } else if (cl == kClsF) {
-        r = project_feature(M, A, yy, c, xx, cn);
+        r = group_project_feature<32>(M.seg, A.seg_off, yy, line_segments(M, A, c), xx, cn);
     }
     if (!r) {
         xx = yy;

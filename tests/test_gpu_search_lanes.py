@@ -1,6 +1,7 @@
 """The triangle search with 1, 8 or 32 lanes per particle gives the same bits,
 on meshes whose candidate lists are short, long and too long to merge (their
-27 cells are probed), with both projection rules and with Boolean partners."""
+27 cells are probed), with both projection rules, with Boolean partners and
+with feature lines long enough to be searched too."""
 import numpy as np
 import pytest
 
@@ -22,6 +23,8 @@ def built():
 def bodies(kind, cascade):
     if kind == "cube":                       # lists of one or two triangles: 8 lanes
         mesh, dx = W.cube_mesh(0.5), 0.06
+    elif kind == "rims":                     # feature lines of 9 and 96 segments, in the search
+        mesh, dx = W.cylinder_mesh(0.5, 1.0, 96 if not cascade else 9, 4), 0.06
     elif kind == "sphere":                   # lists of about a hundred: 32 lanes
         mesh, dx = W.icosphere_mesh(4, 0.5), 0.08
     else:                                    # "probe": over 512 entries in the 27 cells
@@ -47,7 +50,7 @@ def bodies(kind, cascade):
 
 
 @pytest.mark.parametrize("cascade", [False, True])
-@pytest.mark.parametrize("kind", ["cube", "sphere", "probe"])
+@pytest.mark.parametrize("kind", ["cube", "rims", "sphere", "probe"])
 def test_lanes_do_not_change_the_search(kind, cascade):
     got = []
     for ctas in (0, 1, 8):
