@@ -70,4 +70,32 @@ __device__ inline PairGeo pair_geo(const float4 *__restrict__ pos_p, const float
     return o;
 }
 
+// The same for sums that take no decision on r^2: fused multiply-adds and the
+// weight max(1 - r / 2h, 0) from a saturating FMA.  CLS: the class bits are
+// wanted; else only {z, z'} of the second half is read (24 bytes a pair
+// instead of 32).
+template <bool CLS>
+__device__ inline PairGeo pair_sum_geo(const float4 *__restrict__ pos_p, const float4 *__restrict__ pos_b, uint32_t m,
+                                       float2 npx, float2 npy, float2 npz, float hih) {
+    const float4 A = pos_p[m];
+    PairGeo o;
+    float2 z;
+    if (CLS) {
+        const float4 B = pos_b[m];
+        z = make_float2(B.x, B.y);
+        o.w0 = __float_as_uint(B.z);
+        o.w1 = __float_as_uint(B.w);
+    } else {
+        z = *reinterpret_cast<const float2 *>(pos_b + m);
+        o.w0 = o.w1 = 0u;
+    }
+    o.dx = __fadd2_rn(make_float2(A.x, A.y), npx);
+    o.dy = __fadd2_rn(make_float2(A.z, A.w), npy);
+    o.dz = __fadd2_rn(z, npz);
+    o.r2 = __ffma2_rn(o.dz, o.dz, __ffma2_rn(o.dy, o.dy, __fmul2_rn(o.dx, o.dx)));
+    o.r = make_float2(sqrt_approx(o.r2.x), sqrt_approx(o.r2.y));
+    o.t = make_float2(__saturatef(fmaf(o.r.x, -hih, 1.f)), __saturatef(fmaf(o.r.y, -hih, 1.f)));
+    return o;
+}
+
 } // namespace fppg
