@@ -105,3 +105,29 @@ def test_energy_and_gradients_are_the_same_bits_on_every_run():
         assert np.array_equal(gy, runs[0][1]) and np.array_equal(gV, runs[0][2])
     assert np.abs(runs[0][2]).max() > 0
 
+
+
+def test_autograd_function_makes_the_gradients_that_are_wanted():
+    # each input alone, no gradient at all, two backwards through one forward;
+    # a change of the inputs between forward and backward is refused
+    import torch
+    from paper_2501_03056_gb300.autograd import UniformityEnergy, uniformity_energy
+    a, b, o, x32, cls, cons = shared_state(1)
+    y = torch.from_numpy(x32).cuda()
+    v = torch.from_numpy(a.verts).cuda()
+    gy, gV = torch.empty_like(y), torch.empty_like(v)
+    E = b.energy_ptr(y.data_ptr(), v.data_ptr(), gy.data_ptr(), gV.data_ptr())
+    yr, vr = y.clone().requires_grad_(True), v.clone().requires_grad_(True)
+    assert torch.equal(torch.autograd.grad(uniformity_energy(yr, v, b), yr)[0], gy)
+    assert torch.equal(torch.autograd.grad(uniformity_energy(y, vr, b), vr)[0], gV)
+    with torch.no_grad():
+        e0 = uniformity_energy(yr, vr, b)
+    assert not e0.requires_grad and float(e0) == E
+    e1 = UniformityEnergy.apply(yr, vr, b)
+    for _ in range(2):
+        got = torch.autograd.grad(3.0 * e1, (yr, vr), retain_graph=True)
+        assert torch.equal(got[0], gy * 3.0) and torch.equal(got[1], gV * 3.0)
+    with torch.no_grad():
+        yr += 0.01
+    with pytest.raises(RuntimeError, match="modified by an inplace operation"):
+        torch.autograd.grad(e1, yr)
