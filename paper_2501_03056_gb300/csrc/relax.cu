@@ -8,7 +8,9 @@
 //                      k_rank_gather), or k_keys, a stable radix sort,
 //                      k_gather and the table from the sorted keys
 //   k_force         A4  Eq. 15 over the 3 x 3 rows of 3 cells around the
-//                       particle (each row is one contiguous slot range),
+//                       particle (each row is one contiguous slot range; a
+//                       lane per particle, or one per plane of rows in small
+//                       groups),
 //                       amax per body by a labelled warp max + atomicMax
 //   k_step          A5  limited step and tangential part; feature particles,
 //                       and particles with no triangle within reach, finish
@@ -598,14 +600,38 @@ __device__ inline void force_range2(const float4 *__restrict__ pos_p, const floa
     pair_step<ALL, COUNT, true>(pos_p, pos_b, m1 - 1, s, e, npx, npy, npz, mbits, R2, hih, acc, self);
 }
 
-template <int VARIANT, bool COUNT, bool MORTON>
+// k_force, three lanes a particle: ten particles to a warp.  Particles up to
+// which it is taken: a lane's walk of ~350 slots is the launch's length while
+// the warps do not fill the chip (195 k threads at 48 registers).  One lane ->
+// three: 42 k particles 34.3 -> 19.5 us, 76 k 31.3 -> 28.5, 540 k 121 -> 147,
+// 777 k 165 -> 204; the lines through the last four cross at 118 k.
+constexpr int kSplitPerWarp = 10;
+constexpr int64_t kSplitMaxN = 100000;
+
+// (P0 + P1) + P2 of the particle's three lanes
+__device__ inline float planes_sum(float v, int lane) {
+    const int l0 = lane - lane % 3;
+    const float p0 = __shfl_sync(0xffffffffu, v, l0), p1 = __shfl_sync(0xffffffffu, v, l0 + 1);
+    return (p0 + p1) + __shfl_sync(0xffffffffu, v, l0 + 2);
+}
+
+// The sums of the three planes of rows (dz = -1, 0, 1) are formed apart and
+// added as (P0 + P1) + P2, so that SPLIT gives the same bits: three lanes share
+// a particle, a plane each.  It takes more pair steps in all (idle lanes, lanes
+// of a warp in different rows) and makes a warp's walk 2.7 times shorter.  The
+// plane's two halves are added before they join the total: three registers for
+// the totals instead of six, which keeps the one-lane form as fast as a single
+// running sum (18.9 M particles 3703 -> 3683 us; six 3792).
+template <int VARIANT, bool COUNT, bool MORTON, bool SPLIT>
 // (at most 48 registers: five 256-thread blocks per SM)
 __global__ void __launch_bounds__(TPB, 5)
     k_force(const float4 *__restrict__ pos_s, const float4 *__restrict__ pos_p, int64_t N,
             const AsmParams *__restrict__ P, const uint32_t *__restrict__ fstart, float4 *__restrict__ acc_s,
             uint32_t *__restrict__ amax, int32_t *__restrict__ count_s, int32_t *__restrict__ tested_s) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool active = k < N;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31, plane = SPLIT ? lane % 3 : 0;
+    const int64_t k = SPLIT ? (t >> 5) * kSplitPerWarp + lane / 3 : t;
+    const bool active = k < N && (!SPLIT || lane < 3 * kSplitPerWarp);
     const float4 p = active ? pos_s[k] : make_float4(0.f, 0.f, 0.f, 0.f);
     const int cls = active ? cls_of(p.w) : kClsI;
     const int b = active ? body_of(p.w) : 0;
@@ -630,8 +656,9 @@ __global__ void __launch_bounds__(TPB, 5)
         shared_row = __all_sync(0xffffffffu, mbits == 0u || rowkey == lead_row);
     }
     PairAcc acc{make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), 0};
+    float ax = 0.f, ay = 0.f, az = 0.f;                // the planes so far
     int tested = 0;
-    for (int dz = -1; dz <= 1; dz++) {
+    for (int dz = SPLIT ? plane - 1 : -1; dz <= (SPLIT ? plane - 1 : 1); dz++) {
         const int z = cz + dz;
         const float gz = row_gap(g.t[2], cz, dz, g.slack);
         for (int dy = -1; dy <= 1; dy++) {
@@ -655,16 +682,25 @@ __global__ void __launch_bounds__(TPB, 5)
             else
                 force_range2<false, COUNT>(pos_p, pos_b, npx, npy, npz, mbits, R2, hih, s, e, acc, (uint32_t)k);
         }
+        ax += acc.ax.x + acc.ax.y;
+        ay += acc.ay.x + acc.ay.y;
+        az += acc.az.x + acc.az.y;
+        acc.ax = acc.ay = acc.az = make_float2(0.f, 0.f);
+    }
+    if (SPLIT) {
+        ax = planes_sum(ax, lane);
+        ay = planes_sum(ay, lane);
+        az = planes_sum(az, lane);
     }
     float fx = 0.f, fy = 0.f, fz = 0.f, mag = 0.f;
     if (mob) {
         // the sums hold q - p: negate
-        fx = -(acc.ax.x + acc.ax.y) * A.force_scale;
-        fy = -(acc.ay.x + acc.ay.y) * A.force_scale;
-        fz = -(acc.az.x + acc.az.y) * A.force_scale;
+        fx = -ax * A.force_scale;
+        fy = -ay * A.force_scale;
+        fz = -az * A.force_scale;
         mag = sqrtf(fx * fx + fy * fy + fz * fz);
     }
-    if (active) acc_s[k] = make_float4(fx, fy, fz, mag);
+    if (active && plane == 0) acc_s[k] = make_float4(fx, fy, fz, mag);
     if (COUNT && active) {
         count_s[k] = acc.cnt;
         if (tested_s) tested_s[k] = mob ? tested : 0;
@@ -1489,25 +1525,22 @@ int grid_kernels(const DevGroup &d) {
 void build_grid(Group &g, cudaStream_t s) { build_grid_dev(g.d, s); }
 
 void forces_dev(DevGroup &d, int tb, int variant, cudaStream_t s, int32_t *count_s, int32_t *tested_s) {
-    const unsigned nbk = (unsigned)std::max<int64_t>((d.N + tb - 1) / tb, 1);
-#define FPPG_FORCE(V, C, M)                                                                                    \
-    k_force<V, C, M><<<nbk, tb, 0, s>>>(d.pos_s, d.pos_p, d.N, d.params, d.fstart, d.acc_s, d.amax, count_s,        \
-                                        tested_s)
-    if (d.morton_rows) {
-        if (count_s) {
-            if (variant == 1) FPPG_FORCE(1, true, true);
-            else FPPG_FORCE(0, true, true);
-        } else {
-            if (variant == 1) FPPG_FORCE(1, false, true);
-            else FPPG_FORCE(0, false, true);
-        }
-    } else if (count_s) {
-        if (variant == 1) FPPG_FORCE(1, true, false);
-        else FPPG_FORCE(0, true, false);
-    } else {
-        if (variant == 1) FPPG_FORCE(1, false, false);
-        else FPPG_FORCE(0, false, false);
-    }
+    const bool split = !count_s && variant == 0 && d.N <= kSplitMaxN;
+    const unsigned nbk = split ? nblocks(d.N, tb / 32 * kSplitPerWarp) : nblocks(d.N, tb);
+#define FPPG_FORCE(V, C, M, S)                                                                                       \
+    k_force<V, C, M, S><<<nbk, tb, 0, s>>>(d.pos_s, d.pos_p, d.N, d.params, d.fstart, d.acc_s, d.amax, count_s,       \
+                                           tested_s)
+#define FPPG_FORCE_ORDER(V, C, S)                                                                                    \
+    do {                                                                                                             \
+        if (d.morton_rows) FPPG_FORCE(V, C, true, S);                                                                \
+        else FPPG_FORCE(V, C, false, S);                                                                             \
+    } while (0)
+    if (split) FPPG_FORCE_ORDER(0, false, true);
+    else if (count_s && variant == 1) FPPG_FORCE_ORDER(1, true, false);
+    else if (count_s) FPPG_FORCE_ORDER(0, true, false);
+    else if (variant == 1) FPPG_FORCE_ORDER(1, false, false);
+    else FPPG_FORCE_ORDER(0, false, false);
+#undef FPPG_FORCE_ORDER
 #undef FPPG_FORCE
 }
 
