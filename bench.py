@@ -81,7 +81,7 @@ def parse():
     p.add_argument("--no-extras", action="store_true", help="skip plain / e2e / CPU legs")
     p.add_argument("--no-autotune", action="store_true", help="keep the default kernel configuration")
     p.add_argument("--config", default=None,
-                   help="force variant,block,search CTAs per SM[,incremental order 0/1[,row order 0/1]] "
+                   help="force variant,block,search CTAs per SM[,key order: 0 radix, 1 counting[,row order 0/1]] "
                         "(e.g. 0,128,4,1) instead of the autotuner")
     return p.parse_args()
 

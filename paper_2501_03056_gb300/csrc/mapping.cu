@@ -24,8 +24,8 @@
 //                    scan gives the particles' places in key order
 //   k_emit_surface, k_emit_volume
 // A body of C cells moves C / 8 bytes a pass instead of C to 4 C: the gear
-// turned in space (1.7e8 cells, 2.9 M particles) 12.0 -> 0.9 ms of kernels, most of
-// it the FP64 barycentric tests of k_crossings (0.5 ms).
+// turned in space (1.7e8 cells, 2.9 M particles) 12.0 -> 0.5 ms of kernels, the
+// largest k_crossings (0.13 ms).
 #include <cfloat>
 #include <cmath>
 
@@ -84,57 +84,141 @@ __device__ inline bool cell_tris(const uint2 *hrng, const uint4 *compact, const 
     return false;
 }
 
+// the ray of a column as FP32 pairs: hi + lo is within 2^-48 of q
+struct RayPoint {
+    float xh, xl, yh, yl;
+};
+
+__device__ inline RayPoint ray_point(double qx, double qy) {
+    const float xh = (float)qx, yh = (float)qy;
+    return RayPoint{xh, (float)(qx - (double)xh), yh, (float)(qy - (double)yh)};
+}
+
+// Whether the ray meets triangle (a, b, c) within its edges (1) or not (-1), in
+// FP32, or that FP32 does not tell (0).  m1, m2, m3 are the signed areas that
+// the edges make with q: inside they have one sign, outside two differ.  With
+// u = 2^-24 every difference below is off by at most 2 u (|its value| + |lo|)
+// <= 2 u mx, so an area by at most 12 u mx my (two products of two such
+// factors, their rounding and the subtraction's); the FP64 test's own error is
+// 2^-46 mx my.  Areas beyond 32 u mx my therefore have their signs in the FP64
+// test too: two opposite ones miss whatever the sign of its determinant, three
+// alike give it theirs.  NaN and overflow are never certain.
+__device__ inline int ray_side(const float4 &a, const float4 &b, const float4 &c, const RayPoint &q) {
+    const float ax = (a.x - q.xh) - q.xl, bx = (b.x - q.xh) - q.xl, cx = (c.x - q.xh) - q.xl;
+    const float ay = (a.y - q.yh) - q.yl, by = (b.y - q.yh) - q.yl, cy = (c.y - q.yh) - q.yl;
+    const float mx = fmaxf(fmaxf(fabsf(ax), fabsf(bx)), fabsf(cx)) + fabsf(q.xl);
+    const float my = fmaxf(fmaxf(fabsf(ay), fabsf(by)), fabsf(cy)) + fabsf(q.yl);
+    const float m1 = bx * cy - cx * by, m2 = cx * ay - ax * cy, m3 = ax * by - bx * ay;
+    const float bound = mx * my * 0x1p-19f + 1e-36f;    // (and products that underflow)
+    const bool p1 = m1 > bound, p2 = m2 > bound, p3 = m3 > bound;
+    const bool n1 = m1 < -bound, n2 = m2 < -bound, n3 = m3 < -bound;
+    if ((p1 || p2 || p3) && (n1 || n2 || n3)) return -1;
+    return (p1 && p2 && p3) || (n1 && n2 && n3) ? 1 : 0;
+}
+
+// barycentric weights of (qx, qy) in FP64; false outside.  A nonzero quotient
+// of these differences is far above underflow, so its sign is that of its
+// operands.
+__device__ inline bool ray_weights(const float4 &a, const float4 &b, const float4 &c, double qx, double qy, double &l1,
+                                   double &l2, double &l3) {
+    auto negative = [](double num, double den) {
+        return num != 0.0 && (__double2hiint(num) ^ __double2hiint(den)) < 0;
+    };
+    const double ax = a.x, ay = a.y, bx = b.x, by = b.y, cx = c.x, cy = c.y;
+    const double d = (bx - ax) * (cy - ay) - (cx - ax) * (by - ay);
+    if (d == 0.0) return false;
+    const double m1 = (bx - qx) * (cy - qy) - (cx - qx) * (by - qy);
+    if (negative(m1, d)) return false;
+    const double m2 = (cx - qx) * (ay - qy) - (ax - qx) * (cy - qy);
+    if (negative(m2, d)) return false;
+    l1 = m1 / d;
+    l2 = m2 / d;
+    l3 = 1.0 - l1 - l2;
+    return !(l3 < 0);
+}
+
+__device__ inline void ray_of(const MapGrid &g, int x, int y, double &qx, double &qy) {
+    qx = (double)g.mid[0][x] + 1.234567e-6 * g.dx;
+    qy = (double)g.mid[1][y] + 2.345678e-6 * g.dx;
+}
+
+// the crossing's height, toggled at the highest cell whose centre lies below
+__device__ inline void toggle_crossing(const MapGrid &g, uint32_t key, const float4 &a, const float4 &b,
+                                       const float4 &c, uint32_t *__restrict__ toggle) {
+    int x, y, z;
+    cell_of_key(g, key, x, y, z);
+    double qx, qy, l1, l2, l3;
+    ray_of(g, x, y, qx, qy);
+    if (!ray_weights(a, b, c, qx, qy, l1, l2, l3)) return;
+    const double zc = l1 * (double)a.z + l2 * (double)b.z + l3 * (double)c.z;
+    // zc above a float centre: so is zc rounded up.  The first k is a guess.
+    const float zu = __double2float_ru(zc);
+    int k = min((int)fminf(fmaxf(ceilf((zu - g.o[2]) / (float)g.dx - 0.5f), 0.f), (float)g.n[2]), g.n[2]);
+    while (k < g.n[2] && zu > g.mid[2][k]) k++;
+    while (k > 0 && !(zu > g.mid[2][k - 1])) k--;
+    if (k > 0) atomicXor(toggle + word_of(g, x, y, k - 1), 1u << (x & 31));
+}
+
 // One thread per occupied cell.  A triangle's cells in a column are one run
 // along z, so a crossing counts at the lowest cell that lists the triangle.
+// Bound by the FP64 units, a 64th of the FP32 rate, which a warp keeps busy for
+// one lane as for 32: the test is decided in FP32 but next to an edge, and the
+// warp's crossings are queued so that their heights are computed 32 at a time.
+// Gear turned in space, 1.7e8 cells: every test in FP64 523 us, FP32 for the misses
+// alone 470 (some lane of most warps still meets its triangle), both 129.
 __global__ void __launch_bounds__(256) k_crossings(const float4 *__restrict__ vx,
                                                    const uint32_t *__restrict__ occ, const uint2 *__restrict__ hrng,
                                                    const uint4 *__restrict__ compact, int64_t ncompact,
                                                    const int32_t *__restrict__ tlist, MapGrid g,
                                                    uint32_t *__restrict__ toggle, uint32_t *__restrict__ entries,
                                                    uint32_t *__restrict__ error) {
+    __shared__ uint2 queue[8][64];      // (cell key, triangle), 32 left over at most before 32 more
+    uint2 *const mine = queue[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (i >= ncompact) return;
-    const uint4 cell = compact[i];
+    const uint4 cell = i < ncompact ? compact[i] : make_uint4(0u, 0u, 0u, 0u);
     int x, y, z;
     cell_of_key(g, cell.x, x, y, z);
-    const double qx = (double)g.mid[0][x] + 1.234567e-6 * g.dx;
-    const double qy = (double)g.mid[1][y] + 2.345678e-6 * g.dx;
-    // a nonzero quotient of these differences is far above underflow, so its
-    // sign is that of its operands: most triangles end before a division
-    auto negative = [](double num, double den) {
-        return num != 0.0 && (__double2hiint(num) ^ __double2hiint(den)) < 0;
+    double qx, qy;
+    ray_of(g, x, y, qx, qy);
+    const RayPoint q = ray_point(qx, qy);
+    auto toggle_of = [&](uint2 v) {
+        toggle_crossing(g, v.x, vx[3 * (size_t)v.y], vx[3 * (size_t)v.y + 1], vx[3 * (size_t)v.y + 2], toggle);
     };
-    for (uint32_t e = cell.y; e < cell.y + cell.z; e++) {
-        const int t = tlist[e];
-        const float4 a = vx[3 * (size_t)t], b = vx[3 * (size_t)t + 1], c = vx[3 * (size_t)t + 2];
-        const double ax = a.x, ay = a.y, bx = b.x, by = b.y, cx = c.x, cy = c.y;
-        const double d = (bx - ax) * (cy - ay) - (cx - ax) * (by - ay);
-        if (d == 0.0) continue;
-        const double m1 = (bx - qx) * (cy - qy) - (cx - qx) * (by - qy);
-        if (negative(m1, d)) continue;
-        const double m2 = (cx - qx) * (ay - qy) - (ax - qx) * (cy - qy);
-        if (negative(m2, d)) continue;
-        const double l1 = m1 / d, l2 = m2 / d;
-        const double l3 = 1.0 - l1 - l2;
-        if (l3 < 0) continue;
-        if (atomicAdd(entries + (size_t)x + (size_t)g.n[0] * (size_t)y, 1u) >= kColEntries) {
-            atomicOr(error, 1u);
-            return;
+    int queued = 0;
+    for (uint32_t e = cell.y; __any_sync(0xffffffffu, e < cell.y + cell.z); e++) {
+        bool first = false;
+        int t = 0;
+        if (e < cell.y + cell.z) {
+            t = tlist[e];
+            const float4 a = vx[3 * (size_t)t], b = vx[3 * (size_t)t + 1], c = vx[3 * (size_t)t + 2];
+            const int side = ray_side(a, b, c, q);
+            double l1, l2, l3;
+            first = side > 0 || (side == 0 && ray_weights(a, b, c, qx, qy, l1, l2, l3));
+            if (first && atomicAdd(entries + (size_t)x + (size_t)g.n[0] * (size_t)y, 1u) >= kColEntries) {
+                atomicOr(error, 1u);
+                first = false;
+            }
+            if (first && z > 0 && bit_of(occ, (uint64_t)cell.x - (uint64_t)g.n[0] * (uint64_t)g.n[1])) {
+                uint32_t beg = 0, len = 0;
+                if (cell_tris(hrng, compact, g, x, y, z - 1, beg, len))
+                    for (uint32_t o = beg; o < beg + len && first; o++) first = tlist[o] != t;
+            }
         }
-        bool first = true;
-        if (z > 0 && bit_of(occ, (uint64_t)cell.x - (uint64_t)g.n[0] * (uint64_t)g.n[1])) {
-            uint32_t beg = 0, len = 0;
-            if (cell_tris(hrng, compact, g, x, y, z - 1, beg, len))
-                for (uint32_t q = beg; q < beg + len && first; q++) first = tlist[q] != t;
+        const uint32_t vote = __ballot_sync(0xffffffffu, first);
+        if (first) mine[queued + __popc(vote & ((1u << lane) - 1u))] = make_uint2(cell.x, (uint32_t)t);
+        queued += __popc(vote);
+        if (queued >= 32) {
+            __syncwarp();
+            toggle_of(mine[lane]);
+            queued -= 32;
+            const uint2 rest = mine[32 + lane];     // (the first `queued` of them)
+            __syncwarp();
+            if (lane < queued) mine[lane] = rest;
         }
-        if (!first) continue;
-        const double zc = l1 * (double)a.z + l2 * (double)b.z + l3 * (double)c.z;
-        // the cells whose centre lies below the crossing: 0 .. k - 1
-        int k = (int)fmin(fmax(ceil((zc - (double)g.o[2]) / g.dx - 0.5), 0.0), (double)g.n[2]);
-        while (k < g.n[2] && zc > (double)g.mid[2][k]) k++;
-        while (k > 0 && !(zc > (double)g.mid[2][k - 1])) k--;
-        if (k > 0) atomicXor(toggle + word_of(g, x, y, k - 1), 1u << (x & 31));
     }
+    __syncwarp();
+    if (lane < queued) toggle_of(mine[lane]);
 }
 
 // the toggles of a column, from above: in place, bit (x, y, z) becomes the
