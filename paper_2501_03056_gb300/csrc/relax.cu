@@ -9,8 +9,7 @@
 //                      k_gather and the table from the sorted keys
 //   k_force         A4  Eq. 15 over the 3 x 3 rows of 3 cells around the
 //                       particle (each row is one contiguous slot range; a
-//                       lane per particle, or one per plane of rows in small
-//                       groups),
+//                       lane per particle, two in small groups),
 //                       amax per body by a labelled warp max + atomicMax
 //   k_step          A5  limited step and tangential part; feature particles,
 //                       and particles with no triangle within reach, finish
@@ -600,38 +599,45 @@ __device__ inline void force_range2(const float4 *__restrict__ pos_p, const floa
     pair_step<ALL, COUNT, true>(pos_p, pos_b, m1 - 1, s, e, npx, npy, npz, mbits, R2, hih, acc, self);
 }
 
-// k_force, three lanes a particle: ten particles to a warp.  Particles up to
-// which it is taken: a lane's walk of ~350 slots is the launch's length while
-// the warps do not fill the chip (195 k threads at 48 registers).  One lane ->
-// three: 42 k particles 34.3 -> 19.5 us, 76 k 31.3 -> 28.5, 540 k 121 -> 147,
-// 777 k 165 -> 204; the lines through the last four cross at 118 k.
-constexpr int kSplitPerWarp = 10;
+// k_force with two lanes a particle.  Particles up to which it is taken: a
+// lane's walk of ~350 slots is the launch's length while the warps do not fill
+// the chip.  One lane -> two: 42 k particles 35.9 -> 19.8 us, 76 k 31.5 -> 27.3,
+// 540 k 121 -> 155, 777 k 166 -> 216; the lines through the last three cross
+// at about 125 k.
 constexpr int64_t kSplitMaxN = 100000;
 
-// (P0 + P1) + P2 of the particle's three lanes
-__device__ inline float planes_sum(float v, int lane) {
-    const int l0 = lane - lane % 3;
-    const float p0 = __shfl_sync(0xffffffffu, v, l0), p1 = __shfl_sync(0xffffffffu, v, l0 + 1);
-    return (p0 + p1) + __shfl_sync(0xffffffffu, v, l0 + 2);
+// every second slot of [j, e): the operations of pair_step (not COUNT) on one
+// half, in the same order
+__device__ inline void force_slots(const float4 *__restrict__ pos_s, const float4 &p, uint32_t mbits, float hih,
+                                   uint32_t j, uint32_t e, float sum[3]) {
+#pragma unroll 4
+    for (; j < e; j += 2) {
+        const float4 q = pos_s[j];
+        const float dx = __fadd_rn(q.x, -p.x), dy = __fadd_rn(q.y, -p.y), dz = __fadd_rn(q.z, -p.z);
+        const float r2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
+        const float t = __saturatef(__fmaf_rn(sqrt_approx(r2), -hih, 1.f));
+        const float w = (mbits & __float_as_uint(q.w)) != 0u ? __fmul_rn(__fmul_rn(t, t), t) : 0.f;
+        sum[0] = __fmaf_rn(w, dx, sum[0]);
+        sum[1] = __fmaf_rn(w, dy, sum[1]);
+        sum[2] = __fmaf_rn(w, dz, sum[2]);
+    }
 }
 
-// The sums of the three planes of rows (dz = -1, 0, 1) are formed apart and
-// added as (P0 + P1) + P2, so that SPLIT gives the same bits: three lanes share
-// a particle, a plane each.  It takes more pair steps in all (idle lanes, lanes
-// of a warp in different rows) and makes a warp's walk 2.7 times shorter.  The
-// plane's two halves are added before they join the total: three registers for
-// the totals instead of six, which keeps the one-lane form as fast as a single
-// running sum (18.9 M particles 3703 -> 3683 us; six 3792).
+// SPLIT (variant 0 without counts): two lanes a particle, one for the even and
+// one for the odd slots.  The one-lane form sums these apart, in the halves of
+// its packed sums, and adds the two at the end; so both forms give the same
+// bits.  A lane's step takes one candidate instead of two: a walk 1.8 times
+// shorter for 1.3 times the work.
 template <int VARIANT, bool COUNT, bool MORTON, bool SPLIT>
-// (at most 48 registers: five 256-thread blocks per SM)
-__global__ void __launch_bounds__(TPB, 5)
+// (at most 48 registers: five 256-thread blocks per SM; 80 in the split form,
+// whose groups do not fill the chip)
+__global__ void __launch_bounds__(TPB, SPLIT ? 3 : 5)
     k_force(const float4 *__restrict__ pos_s, const float4 *__restrict__ pos_p, int64_t N,
             const AsmParams *__restrict__ P, const uint32_t *__restrict__ fstart, float4 *__restrict__ acc_s,
             uint32_t *__restrict__ amax, int32_t *__restrict__ count_s, int32_t *__restrict__ tested_s) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int lane = threadIdx.x & 31, plane = SPLIT ? lane % 3 : 0;
-    const int64_t k = SPLIT ? (t >> 5) * kSplitPerWarp + lane / 3 : t;
-    const bool active = k < N && (!SPLIT || lane < 3 * kSplitPerWarp);
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, k = SPLIT ? t >> 1 : t;
+    const uint32_t half = threadIdx.x & 1u;
+    const bool active = k < N;
     const float4 p = active ? pos_s[k] : make_float4(0.f, 0.f, 0.f, 0.f);
     const int cls = active ? cls_of(p.w) : kClsI;
     const int b = active ? body_of(p.w) : 0;
@@ -655,10 +661,10 @@ __global__ void __launch_bounds__(TPB, 5)
         const uint32_t lead_row = __shfl_sync(0xffffffffu, rowkey, leader);
         shared_row = __all_sync(0xffffffffu, mbits == 0u || rowkey == lead_row);
     }
+    float sum[3] = {0.f, 0.f, 0.f};
     PairAcc acc{make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), 0};
-    float ax = 0.f, ay = 0.f, az = 0.f;                // the planes so far
     int tested = 0;
-    for (int dz = SPLIT ? plane - 1 : -1; dz <= (SPLIT ? plane - 1 : 1); dz++) {
+    for (int dz = -1; dz <= 1; dz++) {
         const int z = cz + dz;
         const float gz = row_gap(g.t[2], cz, dz, g.slack);
         for (int dy = -1; dy <= 1; dy++) {
@@ -677,30 +683,28 @@ __global__ void __launch_bounds__(TPB, 5)
                 s = __reduce_min_sync(0xffffffffu, s);
                 e = __reduce_max_sync(0xffffffffu, e);
             }
-            if (all_cls)
+            if (SPLIT)
+                force_slots(pos_s, p, mbits, hih, s + ((s ^ half) & 1u), e, sum);
+            else if (all_cls)
                 force_range2<true, COUNT>(pos_p, pos_b, npx, npy, npz, mbits, R2, hih, s, e, acc, (uint32_t)k);
             else
                 force_range2<false, COUNT>(pos_p, pos_b, npx, npy, npz, mbits, R2, hih, s, e, acc, (uint32_t)k);
         }
-        ax += acc.ax.x + acc.ax.y;
-        ay += acc.ay.x + acc.ay.y;
-        az += acc.az.x + acc.az.y;
-        acc.ax = acc.ay = acc.az = make_float2(0.f, 0.f);
     }
     if (SPLIT) {
-        ax = planes_sum(ax, lane);
-        ay = planes_sum(ay, lane);
-        az = planes_sum(az, lane);
+        acc.ax = make_float2(sum[0], __shfl_xor_sync(0xffffffffu, sum[0], 1));
+        acc.ay = make_float2(sum[1], __shfl_xor_sync(0xffffffffu, sum[1], 1));
+        acc.az = make_float2(sum[2], __shfl_xor_sync(0xffffffffu, sum[2], 1));
     }
     float fx = 0.f, fy = 0.f, fz = 0.f, mag = 0.f;
     if (mob) {
         // the sums hold q - p: negate
-        fx = -ax * A.force_scale;
-        fy = -ay * A.force_scale;
-        fz = -az * A.force_scale;
+        fx = -(acc.ax.x + acc.ax.y) * A.force_scale;
+        fy = -(acc.ay.x + acc.ay.y) * A.force_scale;
+        fz = -(acc.az.x + acc.az.y) * A.force_scale;
         mag = sqrtf(fx * fx + fy * fy + fz * fz);
     }
-    if (active && plane == 0) acc_s[k] = make_float4(fx, fy, fz, mag);
+    if (active && (!SPLIT || half == 0u)) acc_s[k] = make_float4(fx, fy, fz, mag);
     if (COUNT && active) {
         count_s[k] = acc.cnt;
         if (tested_s) tested_s[k] = mob ? tested : 0;
@@ -1526,7 +1530,7 @@ void build_grid(Group &g, cudaStream_t s) { build_grid_dev(g.d, s); }
 
 void forces_dev(DevGroup &d, int tb, int variant, cudaStream_t s, int32_t *count_s, int32_t *tested_s) {
     const bool split = !count_s && variant == 0 && d.N <= kSplitMaxN;
-    const unsigned nbk = split ? nblocks(d.N, tb / 32 * kSplitPerWarp) : nblocks(d.N, tb);
+    const unsigned nbk = nblocks(d.N, split ? tb / 2 : tb);
 #define FPPG_FORCE(V, C, M, S)                                                                                       \
     k_force<V, C, M, S><<<nbk, tb, 0, s>>>(d.pos_s, d.pos_p, d.N, d.params, d.fstart, d.acc_s, d.amax, count_s,       \
                                            tested_s)

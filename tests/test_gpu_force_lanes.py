@@ -1,6 +1,6 @@
-"""The pair force with three lanes per particle (small groups) gives the bits
-of the one-lane form, which the same body meets in a batch of over 100 000
-particles; sizes around a warp's ten particles and a block's eighty."""
+"""The pair force with two lanes per particle (small groups) gives the bits of
+the one-lane form, which the same body meets in a batch of over 100 000
+particles; sizes around a warp's sixteen particles and a block's 128."""
 import numpy as np
 import pytest
 
@@ -28,7 +28,7 @@ def body(n, seed):
 
 
 @pytest.mark.parametrize("morton", [False, True])
-@pytest.mark.parametrize("n", [1, 9, 10, 11, 79, 80, 81, 2500])
+@pytest.mark.parametrize("n", [1, 9, 10, 11, 15, 16, 17, 79, 80, 81, 127, 128, 129, 2500])
 def test_small_group_has_the_bits_of_a_large_one(n, morton):
     small, large = body(n, n), body(n, n)
     rest = body(100001 - n, 7)                # one past the small form's range
