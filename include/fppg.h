@@ -370,7 +370,9 @@ int fppg_batch_set_stream(fppg_batch *b, void *stream);
 int fppg_batch_relax(fppg_batch *b, int32_t n_iter, int32_t use_graph);
 int fppg_batch_set_graph_iters(fppg_batch *b, int32_t graph_iters);
 /* Copy the batch state back into its bodies, or reload it from them (after
- * fppg_set_particles on the bodies with unchanged particle counts). */
+ * fppg_set_particles on the bodies with unchanged particle counts).
+ * FPPG_ERR_STATE, with nothing moved, when a body has lost its particles to
+ * an allocation that failed. */
 int fppg_batch_store(fppg_batch *b);
 int fppg_batch_load(fppg_batch *b);
 /* Autotuner: times `iters` iterations of the batch for every combination

@@ -181,7 +181,6 @@ MeshView view_of(const Body &b) {
     return MeshView{b.geo, b.vx, b.pn, b.hrng, b.compact, b.tlist, b.seg, b.lines, b.occ, b.drank, b.coff, b.cand};
 }
 
-// (re)build the single-body group of a context
 // the staging buffer of ctx with at least `bytes` bytes
 int stage_buf(fppg_ctx *ctx, size_t bytes, void **out) {
     if (bytes > ctx->stage_bytes) {
@@ -198,6 +197,15 @@ int stage_buf(fppg_ctx *ctx, size_t bytes, void **out) {
     return FPPG_OK;
 }
 
+// after a call that failed: the arrays hold another number of particles than
+// the handle had, or none, so it has none (no call may count on the old ones)
+void forget_lost_particles(fppg_ctx *c) {
+    if (c->group.d.pos && c->group.d.N == c->n) return;
+    c->n = 0;
+    c->cls_host.clear();
+}
+
+// (re)build the single-body group of a context
 int ctx_group(fppg_ctx *c) {
     Group &g = c->group;
     g.d.B = 1;
@@ -372,7 +380,10 @@ int fppg_map_particles(fppg_ctx *ctx, const fppg_map_opts *opts, int64_t *n_out)
     int r = map_particles(ctx->group, ctx->body, opts->surface, opts->volume, opts->features, opts->band_cells,
                           opts->band_cells > 0 ? opts->inner_cells : 0, ctx->stream, &n, ctx->cls_host,
                           ctx->err);
-    if (r) return r == 1 ? FPPG_ERR_ARG : (r == 3 ? FPPG_ERR_OOM : (r == 6 ? FPPG_ERR_INTERNAL : FPPG_ERR_CUDA));
+    if (r) {
+        forget_lost_particles(ctx);
+        return r == 1 ? FPPG_ERR_ARG : (r == 3 ? FPPG_ERR_OOM : (r == 6 ? FPPG_ERR_INTERNAL : FPPG_ERR_CUDA));
+    }
     ctx->n = n;
     ctx->has_particles = true;
     if (n_out) *n_out = n;
@@ -420,7 +431,10 @@ int fppg_set_particles(fppg_ctx *ctx, const float *xyz_host, const int32_t *cls_
     ctx->n_ghost = 0;
     if (n != g.d.N || !g.d.pos) {
         int r = g.alloc_particles(n, ctx->err);
-        if (r) return r;
+        if (r) {
+            forget_lost_particles(ctx);
+            return r;
+        }
     }
     ctx->n = n;
     if ((int64_t)ctx->cls_host.size() != n) ctx->cls_host.resize((size_t)n);
@@ -1135,10 +1149,15 @@ static int batch_move(fppg_batch *b, bool store) {
         m.n = 0;
         items = 0;
     };
+    // (the kernel takes the bodies' arrays as they are: a body that lost them
+    // to a failed allocation is refused before anything is launched)
+    for (size_t i = 0; i < b->ctxs.size(); i++)
+        if (!b->ctxs[i]->has_particles && b->ctxs[i]->n == 0 && b->off[i + 1] > b->off[i])
+            return fail(b->err, FPPG_ERR_STATE, "a body of the batch lost its particles");
     for (size_t i = 0; i < b->ctxs.size(); i++) {
         DevGroup &c = b->ctxs[i]->group.d;
         // (a body whose count changed since: no more than either side holds)
-        const int64_t cn = std::min(b->ctxs[i]->n, b->off[i + 1] - b->off[i]);
+        const int64_t cn = std::min({b->ctxs[i]->n, c.N, b->off[i + 1] - b->off[i]});
         if (!cn) continue;
         m.first[m.n] = items;
         m.off[m.n] = b->off[i];
