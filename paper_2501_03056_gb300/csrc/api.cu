@@ -377,6 +377,7 @@ int fppg_map_particles(fppg_ctx *ctx, const fppg_map_opts *opts, int64_t *n_out)
         return fail(ctx->err, FPPG_ERR_ARG, "band_cells or inner_cells outside 0..64");
     int64_t n = 0;
     ctx->has_particles = false;     // until the new set is complete
+    ctx->split = false;
     int r = map_particles(ctx->group, ctx->body, opts->surface, opts->volume, opts->features, opts->band_cells,
                           opts->band_cells > 0 ? opts->inner_cells : 0, ctx->stream, &n, ctx->cls_host,
                           ctx->err);

@@ -288,6 +288,7 @@ int Group::alloc_particles_once(int64_t N, std::string &err) {
     g.pos = g.pos_s = g.pos_p = g.cert = g.acc_s = nullptr;
     g.cons = g.cons_s = nullptr;
     g.key[0] = g.key[1] = g.id[0] = g.id[1] = nullptr;
+    g.id_s = g.key_s = nullptr;     // (the last grid build's order lived in these)
     g.hist = nullptr;
     g.coef_s = nullptr;
     g.stat = nullptr;

@@ -69,3 +69,14 @@ def test_a_batch_does_not_touch_the_arrays_a_body_lost(lose):
                 call()
             assert e.value.code == pkg.ERR_STATE
     assert k > 3
+
+
+@pytest.mark.parametrize("replace", [lambda b: b.map_particles(), lose_by_setting])
+def test_a_step_needs_the_forces_of_the_particles_it_moves(replace):
+    b = body()
+    amax = b.relax_forces()
+    replace(b)
+    with pytest.raises(pkg.FPPGError) as e:
+        b.relax_step(amax)
+    assert e.value.code == pkg.ERR_STATE
+    b.relax_step(b.relax_forces())       # and then it goes on
