@@ -560,6 +560,13 @@ int map_particles(Group &g, Body &b, int surface, int volume, int features, int 
             return r;
         }
     } else {
+        // the arrays are used again: work on the old particles that is still
+        // under way on a stream the body had before ends first (a new
+        // allocation waits for it when it frees the old arrays)
+        if (!ok(cudaDeviceSynchronize())) {
+            cleanup();
+            return 4;
+        }
         cudaMemsetAsync(g.d.cert, 0, sizeof(float4) * (size_t)N, s);   // as a new allocation has it
     }
     if (band && nvol && dev_malloc(&vcls, (size_t)nvol)) {
