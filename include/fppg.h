@@ -387,7 +387,8 @@ int fppg_batch_load(fppg_batch *b);
  * state afterwards.  The choice is cached per (particle-count bucket,
  * volume-particle share, GPU name) for the life of the process; a cached
  * choice is applied without timing.  Every variant, block size, search
- * grid and ordering gives the same bits; the Morton row order moves
+ * grid and ordering gives the same bits (the keys of a crowded set, see
+ * fppg_batch_set_incremental, keep their ordering); the Morton row order moves
  * particles between the force loop's two partial sums, so it agrees with
  * row-major rows up to FP32 rounding (a plain body set to the same row
  * order gives the batch's bits).  Outputs (nullable): chosen variant,
@@ -396,13 +397,16 @@ int fppg_batch_load(fppg_batch *b);
 int fppg_batch_autotune(fppg_batch *b, int32_t iters, int32_t *variant, int32_t *block, int32_t *search_ctas,
                         int32_t *incremental, int32_t *cell_order, double *ms_per_iter);
 /* How the cell keys are put in order every iteration (Sec. 3.1.3): 0 a full
- * stable radix sort of every key; 1 (the start) a counting sort over the
- * dense fine keys, which gives the start table and the order together: the
- * keys are counted as they are made, and particles that share a key are
- * ranked by id.  Both give the one order by (key, particle id), so the
- * results are the same bits.  The counting sort's work for a particle grows
- * with the number that share its key, as its pairs do.  Drops a captured
- * graph.  FPPG_ERR_ARG for other values. */
+ * stable radix sort of every key; 1 a counting sort over the dense fine keys,
+ * which gives the start table and the order together: the keys are counted as
+ * they are made, and particles that share a key are ranked by id.  Both give
+ * the one order by (key, particle id), so the results are the same bits.  The
+ * counting sort's work for a particle grows with the number that share its
+ * key (an eighth along x of a neighbour-grid cell), so the start is 1, but 0
+ * for a set with fixed particles (I, P, ghosts, classes kept from moving) that
+ * has more than 512 particles on one key when it is given, or when its classes
+ * are fixed.  A choice made here stays, also for sets given later.  Drops a
+ * captured graph.  FPPG_ERR_ARG for other values. */
 int fppg_batch_set_incremental(fppg_batch *b, int32_t incremental);
 /* The same for the single body of a handle (its fppg_relax, fppg_stats and
  * debug calls). */

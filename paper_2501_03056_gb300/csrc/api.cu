@@ -17,6 +17,8 @@ namespace fppg {
 void set_global_error(const char *msg);
 }
 
+constexpr int kMovable = (1 << FPPG_S) | (1 << FPPG_V) | (1 << FPPG_F);
+
 struct fppg_ctx {
     Body body;
     Group group;
@@ -26,7 +28,7 @@ struct fppg_ctx {
     bool has_particles = false;
     int fixed_features = 0;
     std::vector<int32_t> cls_host;
-    int mobile_mask = (1 << FPPG_S) | (1 << FPPG_V) | (1 << FPPG_F);   // classes that move
+    int mobile_mask = kMovable;    // classes that move
     int cascade = 0;               // surface re-projection rule (fppg_set_projection_rule)
     // Boolean operations this body takes part in (fppg_boolean), in order:
     // the other operand, FPPG_UNION / FPPG_DIFFERENCE / FPPG_INTERSECTION,
@@ -44,6 +46,7 @@ struct fppg_ctx {
             if (r.other == o) return &r;
         return nullptr;
     }
+    int64_t n_still = 0;           // particles of the classes I and P, as far as they may share keys
     int64_t n_ghost = 0;           // the last n_ghost particles are ghosts (fppg_set_ghost_count)
     bool split = false;            // after fppg_relax_forces, until its step
     // device staging of the host particle arrays of set / get, kept between
@@ -205,6 +208,22 @@ void forget_lost_particles(fppg_ctx *c) {
     c->cls_host.clear();
 }
 
+// The order of the keys for the particles as they are (Group::find_crowds).
+// Moving particles repel each other and pay more for their pairs than for their
+// place, so only a set with enough fixed ones is looked at.
+int ctx_crowds(fppg_ctx *c) {
+    Group &g = c->group;
+    int64_t fixed = c->n_still + c->n_ghost;
+    const int moving = c->mobile_mask & (c->fixed_features ? ~(1 << FPPG_F) : ~0);
+    const int still = kMovable & ~moving;
+    if (still)
+        for (int32_t cl : c->cls_host) fixed += (still >> cl) & 1;
+    g.crowded = false;
+    if (fixed > (int64_t)kCrowd && g.find_crowds(c->stream, &g.crowded, c->err)) return FPPG_ERR_CUDA;
+    g.choose_order();
+    return FPPG_OK;
+}
+
 // (re)build the single-body group of a context
 int ctx_group(fppg_ctx *c) {
     Group &g = c->group;
@@ -300,15 +319,17 @@ int fppg_set_stream(fppg_ctx *ctx, void *stream) {
 int fppg_set_fixed_features(fppg_ctx *ctx, int32_t fixed) {
     if (!ctx) return FPPG_ERR_ARG;
     ctx->fixed_features = fixed ? 1 : 0;
-    return ctx_group(ctx);
+    const int r = ctx->has_particles ? ctx_crowds(ctx) : FPPG_OK;
+    return r ? r : ctx_group(ctx);
 }
 
 int fppg_set_mobile_classes(fppg_ctx *ctx, int32_t mask) {
     if (!ctx) return FPPG_ERR_ARG;
-    if (mask & ~((1 << FPPG_S) | (1 << FPPG_V) | (1 << FPPG_F)))
+    if (mask & ~kMovable)
         return fail(ctx->err, FPPG_ERR_ARG, "only S, V and F can be mobile");
     ctx->mobile_mask = mask;
-    return ctx_group(ctx);
+    const int r = ctx->has_particles ? ctx_crowds(ctx) : FPPG_OK;
+    return r ? r : ctx_group(ctx);
 }
 
 int fppg_set_projection_rule(fppg_ctx *ctx, int32_t rule) {
@@ -386,6 +407,14 @@ int fppg_map_particles(fppg_ctx *ctx, const fppg_map_opts *opts, int64_t *n_out)
         return r == 1 ? FPPG_ERR_ARG : (r == 3 ? FPPG_ERR_OOM : (r == 6 ? FPPG_ERR_INTERNAL : FPPG_ERR_CUDA));
     }
     ctx->n = n;
+    // (cells and feature points are a spacing apart; only the singular points,
+    // mesh vertices at the front with the features, can share keys)
+    ctx->n_still = 0;
+    for (int32_t c : ctx->cls_host) {
+        if (c != FPPG_F && c != FPPG_P) break;
+        ctx->n_still += c == FPPG_P;
+    }
+    if ((r = ctx_crowds(ctx))) return r;
     ctx->has_particles = true;
     if (n_out) *n_out = n;
     return ctx_group(ctx);
@@ -411,9 +440,14 @@ int fppg_set_particles(fppg_ctx *ctx, const float *xyz_host, const int32_t *cls_
     // branch-free scans (they vectorise), on several host threads: a class
     // outside 0..4, an exponent field of all ones (inf or NaN)
     std::atomic<uint32_t> bad_cls{0u}, bad_xyz{0u};
+    std::atomic<int64_t> still{0};
     host_parallel(n, [&](int64_t a, int64_t b) {
-        uint32_t bc = 0u, bx = 0u;
-        for (int64_t i = a; i < b; i++) bc |= (uint32_t)((uint32_t)cls_host[i] > 4u);
+        uint32_t bc = 0u, bx = 0u, st = 0u;
+        for (int64_t i = a; i < b; i++) {
+            bc |= (uint32_t)((uint32_t)cls_host[i] > 4u);
+            st += (uint32_t)(cls_host[i] >= FPPG_I);
+        }
+        still.fetch_add(st);
         for (int64_t i = 3 * a; i < 3 * b; i++) {
             uint32_t w;
             memcpy(&w, xyz_host + i, sizeof(w));
@@ -442,6 +476,9 @@ int fppg_set_particles(fppg_ctx *ctx, const float *xyz_host, const int32_t *cls_
     int32_t *ch = ctx->cls_host.data();
     host_parallel(n, [&](int64_t a, int64_t b) { std::copy(cls_host + a, cls_host + b, ch + a); });
     if (n > 0) k_pack<<<nb(n), 256, 0, ctx->stream>>>(dx, dc, n, 0, g.d.pos, g.d.cons);
+    ctx->n_still = still.load();
+    const int r = ctx_crowds(ctx);
+    if (r) return r;
     CUDA_OR(ctx->err, cudaStreamSynchronize(ctx->stream));
     ctx->has_particles = true;
     return ctx_group(ctx);
@@ -632,7 +669,7 @@ int fppg_set_ghost_count(fppg_ctx *ctx, int64_t n_ghost) {
     ctx->n_ghost = n_ghost;
     tag_ghosts(ctx->group, ctx->n - n_ghost, ctx->stream);
     CUDA_OR(ctx->err, cudaGetLastError());
-    return FPPG_OK;
+    return ctx_crowds(ctx);
 }
 
 int fppg_relax_forces(fppg_ctx *ctx, float *amax_host) {
@@ -857,6 +894,10 @@ int fppg_copy_positions_dev(fppg_ctx *ctx, float *xyz_dev) {
 }
 
 // ---- batches ------------------------------------------------------------------
+static bool crowded_body(const fppg_batch *b) {
+    return std::any_of(b->ctxs.begin(), b->ctxs.end(), [](const fppg_ctx *c) { return c->group.crowded; });
+}
+
 int fppg_batch_create(fppg_ctx *const *ctxs, int32_t n, fppg_batch **out) {
     if (!out) return FPPG_ERR_ARG;
     *out = nullptr;
@@ -989,6 +1030,7 @@ int fppg_batch_create(fppg_ctx *const *ctxs, int32_t n, fppg_batch **out) {
         return fail_global(FPPG_ERR_ARG, "batch too large for 32-bit keys");
     }
     d.total_cells = cells;
+    g.crowded = crowded_body(b);
     std::string &err = b->err;
     int r = g.alloc_particles(N, err);
     auto A = [&](void **p, size_t bytes) { return dev_malloc(p, std::max<size_t>(bytes, 16)); };
@@ -1183,12 +1225,25 @@ int fppg_batch_store(fppg_batch *b) {
     return FPPG_OK;
 }
 
+static void batch_crowds(fppg_batch *b, bool crowded) {
+    Group &g = b->group;
+    if (crowded == g.crowded) return;
+    const bool counted = g.d.counted;
+    g.crowded = crowded;
+    g.choose_order();
+    if (g.d.counted != counted && g.graph) {
+        cudaGraphExecDestroy(g.graph);
+        g.graph = nullptr;
+    }
+}
+
 int fppg_batch_load(fppg_batch *b) {
     if (!b) return FPPG_ERR_ARG;
     // (nothing is loaded when a body's count changed)
     for (size_t i = 0; i < b->ctxs.size(); i++)
         if (b->ctxs[i]->n != b->off[i + 1] - b->off[i])
             return fail(b->err, FPPG_ERR_STATE, "a body changed its particle count");
+    batch_crowds(b, crowded_body(b));
     return batch_move(b, false);
 }
 
@@ -1227,6 +1282,9 @@ int fppg_batch_autotune(fppg_batch *b, int32_t iters, int32_t *variant, int32_t 
     const TuneKey key{nb, d.N ? (int)(10 * nv / d.N) : 0, prop.name};
     TuneVal best{g.force_variant, g.force_block, g.search_thread ? 0 : g.search_blocks / std::max(sms, 1),
                  d.counted ? 1 : 0, g.cell_order};
+    // (a crowded set keeps the order of its keys, and what was timed under it is
+    // not for others)
+    const int order0 = best.incremental;
     double best_ms = 0.0;
     bool cached = false;
     {
@@ -1297,7 +1355,8 @@ int fppg_batch_autotune(fppg_batch *b, int32_t iters, int32_t *variant, int32_t 
         }
         // the other ordering of the keys, then the other order of the grid
         // rows, with the fastest kernels
-        if (const int r = consider(best.variant, best.block, best.search_ctas, 1 - inc0, co0)) return r;
+        if (!g.crowded)
+            if (const int r = consider(best.variant, best.block, best.search_ctas, 1 - inc0, co0)) return r;
         if (const int r = consider(best.variant, best.block, best.search_ctas, best.incremental, 1 - co0))
             if (r != FPPG_ERR_ARG) return r;   // a grid too large for the Morton table keeps row-major rows
         g.time_force = tf;
@@ -1309,12 +1368,13 @@ int fppg_batch_autotune(fppg_batch *b, int32_t iters, int32_t *variant, int32_t 
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        g_tune_cache[key] = best;
+        if (!g.crowded) g_tune_cache[key] = best;
     }
     g.force_variant = best.variant;
     g.force_block = best.block;
     g.search_thread = best.search_ctas == 0;
     g.search_blocks = (best.search_ctas == 0 ? 16 : best.search_ctas) * sms;
+    if (g.crowded) best.incremental = order0;
     d.counted = best.incremental != 0;
     if (best.cell_order != g.cell_order) {
         const int r = g.set_cell_order(best.cell_order, s, b->err);
@@ -1335,9 +1395,17 @@ int fppg_batch_autotune(fppg_batch *b, int32_t iters, int32_t *variant, int32_t 
 
 int fppg_batch_set_mobile_classes(fppg_batch *b, int32_t mask) {
     if (!b) return FPPG_ERR_ARG;
-    if (mask & ~((1 << FPPG_S) | (1 << FPPG_V) | (1 << FPPG_F)))
+    if (mask & ~kMovable)
         return fail(b->err, FPPG_ERR_ARG, "only S, V and F can be mobile");
-    for (AsmParams &A : b->group.hp) A.mobile = mask;
+    Group &g = b->group;
+    for (AsmParams &A : g.hp) A.mobile = mask;
+    // classes that stop moving may share keys (the order it had stays when the
+    // bodies are moving again)
+    if (mask != kMovable && !g.crowded && g.d.counted) {
+        bool crowded = false;
+        if (g.find_crowds(b->stream, &crowded, b->err)) return FPPG_ERR_CUDA;
+        batch_crowds(b, crowded);
+    }
     // the kernels read the parameters from device memory: a captured
     // graph sees the new mask without being captured again
     return b->group.upload_params(b->stream, b->err) ? FPPG_ERR_CUDA : FPPG_OK;
@@ -1398,6 +1466,7 @@ int fppg_device_sm_count(int32_t *sms) {
 
 int fppg_set_incremental(fppg_ctx *ctx, int32_t incremental) {
     if (!ctx || incremental < 0 || incremental > 1) return FPPG_ERR_ARG;
+    ctx->group.order_set = true;
     ctx->group.d.counted = incremental != 0;
     return FPPG_OK;
 }
@@ -1405,6 +1474,7 @@ int fppg_set_incremental(fppg_ctx *ctx, int32_t incremental) {
 int fppg_batch_set_incremental(fppg_batch *b, int32_t incremental) {
     if (!b || incremental < 0 || incremental > 1) return FPPG_ERR_ARG;
     Group &g = b->group;
+    g.order_set = true;
     g.d.counted = incremental != 0;
     if (g.graph) {
         cudaGraphExecDestroy(g.graph);

@@ -333,8 +333,8 @@ int Group::alloc_particles_once(int64_t N, std::string &err) {
             CKA(dev_malloc(&g.tile_base, sizeof(uint32_t) * (size_t)nt));
             CKA(dev_malloc(&g.scan_tmp, sizeof(uint32_t) * (size_t)scan_tmp_elems(nt)));
         }
-        g.counted = true;    // the faster form at every size measured (the autotuner may switch)
     }
+    choose_order();
     if (!g.amax) {
         CKA(dev_malloc(&g.amax, sizeof(uint32_t) * (size_t)std::max(g.B, 1)));
         CKA(dev_malloc(&g.maxdisp, sizeof(uint32_t) * (size_t)std::max(g.B, 1)));

@@ -118,6 +118,14 @@ struct Group {
     bool search_thread = false;   // one thread (not a group of lanes) per queued particle
     int search_lanes = 32;        // lanes per queued particle otherwise: 8 or 32 (set_search_lanes)
     void set_search_lanes(int64_t cells, int64_t entries);
+    // order of the keys: the counting sort, but the radix form for a set with
+    // crowded keys, unless the caller chose one (order_set)
+    bool crowded = false, order_set = false;
+    void choose_order() {
+        if (!order_set) d.counted = !crowded;
+    }
+    // whether some key holds more than kCrowd particles now; waits for s
+    int find_crowds(cudaStream_t s, bool *found, std::string &err);
     int force_block = 256;        // threads per block of the force kernel (multiple of 32, <= 256)
     int force_variant = 0;        // 0 per-lane rows, 1 shared-row union
     // order of the neighbour grid's rows: 0 row-major, 1 Morton (Eq. 9 over

@@ -292,6 +292,10 @@ constexpr int64_t start_blocks(int64_t f1) { return (f1 + kStartBlock - 1) / kSt
 constexpr int kCountTile = 4096, kFewTiles = 8, kScanTiles = 16384;
 constexpr int64_t count_tiles(int64_t f1) { return (f1 + kCountTile - 1) / kCountTile; }
 
+// more particles than this on one fine key, fixed ones among them: the keys
+// are ordered by the radix form (relax.cu)
+constexpr uint32_t kCrowd = 512;
+
 struct GridPoint {
     float t[3];
     int c[3];

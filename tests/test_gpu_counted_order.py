@@ -77,3 +77,81 @@ def test_counting_sort_on_a_grid_of_more_tiles_than_a_block_adds_up():
     assert len(a[2]) > 25000
     for x, y in zip(a, b):
         assert np.array_equal(x, y)
+
+
+def test_fixed_particles_on_one_key_take_linear_time():
+    # twice as many on the key: far from four times as long (ranking each
+    # against all takes 3.8 times as long from 100,000 to 200,000)
+    import torch
+    v, t = W.cube_mesh(0.5)
+    took = []
+    for n in (100000, 200000):
+        b = pkg.Body(v, t, 0.02, 0.026, stream=torch.cuda.current_stream())
+        b.set_particles(np.full((n, 3), 0.1234, np.float32), np.full(n, W.CLS_I, np.int32))
+        b.relax(1)
+        runs = []
+        for _ in range(5):
+            t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            t0.record()
+            b.relax(2)
+            t1.record()
+            t1.synchronize()
+            runs.append(t0.elapsed_time(t1))
+        took.append(sorted(runs)[2])
+    assert took[1] < 2.9 * took[0]
+
+
+# a set that crowds a key when it is given takes the radix sort, and only that
+# one: at the edge (512), for a batch when it is made and when it is loaded again
+@pytest.mark.parametrize("m,crowded", [(512, False), (513, True), (20000, True)])
+def test_a_crowded_set_is_ordered_by_the_radix_sort(m, crowded):
+    rng = np.random.default_rng(m)
+    v, t = W.cube_mesh(0.5)
+    loose = rng.uniform(-0.45, 0.45, (25000, 3)).astype(np.float32)
+    tight = loose.copy()
+    tight[rng.permutation(len(loose))[:m]] = 0.49        # (a key that holds no other)
+    cls = np.where(rng.uniform(size=len(loose)) < 0.5, W.CLS_I, W.CLS_P).astype(np.int32)
+
+    def body(x):
+        b = pkg.Body(v, t, 0.05, 0.065)
+        b.set_particles(x, cls)
+        return b
+
+    kernels = pkg.Batch([body(loose)]).kernels_per_iter
+    radix = pkg.Batch([body(loose)])
+    radix.set_incremental(False)
+    assert radix.kernels_per_iter > kernels
+    a, b = body(loose), body(tight)
+    bt = pkg.Batch([a, b])
+    assert (bt.kernels_per_iter == kernels) == (not crowded)
+    b.set_particles(loose, cls)
+    bt.load()
+    assert bt.kernels_per_iter == kernels
+    b.set_particles(tight, cls)
+    bt.load()
+    assert (bt.kernels_per_iter == kernels) == (not crowded)
+    bt.set_graph_iters(2)
+    bt.relax(2, use_graph=True)
+    bt.autotune(1)
+    assert (bt.kernels_per_iter == kernels) == (not crowded)
+    # moving classes on one key that stop moving, in a body and in a batch
+    b = pkg.Body(v, t, 0.05, 0.065)
+    b.set_particles(tight, np.full(len(tight), W.CLS_V, np.int32))
+    moving = pkg.Batch([b])
+    assert moving.kernels_per_iter == kernels
+    moving.set_mobile_classes((W.CLS_S, W.CLS_F))
+    assert (moving.kernels_per_iter == kernels) == (not crowded)
+    b.set_mobile_classes((W.CLS_S, W.CLS_F))
+    assert (pkg.Batch([b]).kernels_per_iter == kernels) == (not crowded)
+    b = pkg.Body(v, t, 0.05, 0.065)
+    b.set_particles(tight, np.full(len(tight), W.CLS_V, np.int32))
+    b.set_ghost_count(len(tight))
+    assert (pkg.Batch([b]).kernels_per_iter == kernels) == (not crowded)
+    b, bt = body(tight), pkg.Batch([a, body(loose)])
+    bt.set_incremental(True)                      # the caller's choice stands
+    bt.load()
+    assert bt.kernels_per_iter == kernels
+    loaded = pkg.Batch([b])
+    loaded.set_incremental(True)
+    loaded.load()
+    assert loaded.kernels_per_iter == kernels
