@@ -119,7 +119,10 @@ struct Group {
     int search_lanes = 32;        // lanes per queued particle otherwise: 8 or 32 (set_search_lanes)
     void set_search_lanes(int64_t cells, int64_t entries);
     // order of the keys: the counting sort, but the radix form for a set with
-    // crowded keys, unless the caller chose one (order_set)
+    // crowded keys, unless the caller chose one (order_set).  An iteration of
+    // fixed particles, counting sort / radix form: 100 of them on 8 k fine keys
+    // 29 / 53 us, on 3.9 M 37 / 79, on 71 M 201 / 377; 50 k on 8 k keys 31 / 64, on
+    // 3.9 M 39 / 88, on 71 M 207 / 265; 4 M on 0.55 M keys 263 / 428, on 71 M 606 / 819
     bool crowded = false, order_set = false;
     void choose_order() {
         if (!order_set) d.counted = !crowded;

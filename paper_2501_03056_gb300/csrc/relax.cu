@@ -1518,7 +1518,11 @@ static void build_counted(DevGroup &d, cudaStream_t s) {
     k_count_starts<<<(unsigned)nt, TPB, 0, s>>>(d.cnt, tiles, nt > kScanTiles, F1, d.fstart, d.amax, d.maxdisp, d.B,
                                                 d.work_count);
     d.id_s = d.key[1];
-    k_place<<<nblocks(d.N), TPB, 0, s>>>(d.key[0], d.id[0], d.fstart, d.N, d.id[1], d.cnt, F1);
+    // a block for every 4096 counts to clear, however few the particles: 100 of
+    // them on 71 M fine keys 4,392 -> 201 us an iteration, on 3.9 M 273 -> 37
+    // (radix form 377 and 79)
+    k_place<<<std::max(nblocks(d.N), nblocks(F1, kCountTile)), TPB, 0, s>>>(d.key[0], d.id[0], d.fstart, d.N, d.id[1],
+                                                                            d.cnt, F1);
     if (d.N < kGatherTwoMinN)
         k_rank_gather<1><<<nblocks(d.N), TPB, 0, s>>>(d.id[1], d.params, d.fstart, d.pos, d.cons, d.N, d.pos_s,
                                                       d.pos_p, d.id_s, d.cons_s);

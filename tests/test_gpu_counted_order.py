@@ -101,6 +101,31 @@ def test_fixed_particles_on_one_key_take_linear_time():
     assert took[1] < 2.9 * took[0]
 
 
+def test_few_particles_on_a_large_grid_are_not_slower_than_by_the_radix_sort():
+    # 3.9 M fine keys, whose counts were cleared by the blocks of the particles:
+    # 273 us an iteration, the radix sort 79
+    import torch
+    v, t = W.cube_mesh(0.5)
+    rng = np.random.default_rng(2)
+    took = []
+    for counted in (None, False):
+        b = pkg.Body(v, t, 0.005, 0.0065, stream=torch.cuda.current_stream())
+        b.set_particles(rng.uniform(-0.5, 0.5, (100, 3)).astype(np.float32), np.full(100, W.CLS_V, np.int32))
+        if counted is not None:
+            b.set_incremental(counted)
+        b.relax(2)
+        runs = []
+        for _ in range(5):
+            t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            t0.record()
+            b.relax(20)
+            t1.record()
+            t1.synchronize()
+            runs.append(t0.elapsed_time(t1))
+        took.append(sorted(runs)[2])
+    assert took[0] < 1.2 * took[1]
+
+
 # a set that crowds a key when it is given takes the radix sort, and only that
 # one: at the edge (512), for a batch when it is made and when it is loaded again
 @pytest.mark.parametrize("m,crowded", [(512, False), (513, True), (20000, True)])
