@@ -442,6 +442,10 @@ int fppg_batch_set_mobile_classes(fppg_batch *b, int32_t mask);
  * (FPPG_ERR_ARG otherwise).  Every choice gives the
  * same bits; only the speed differs.  Drops a captured graph. */
 int fppg_batch_configure(fppg_batch *b, int32_t variant, int32_t block, int32_t search_ctas);
+/* The lanes per queued particle of a batch's triangle search alone: lanes 1, 8
+ * or 32 sets them (dropping a captured graph), 0 leaves them; *used (nullable)
+ * the lanes in force.  FPPG_ERR_ARG otherwise. */
+int fppg_debug_search_lanes(fppg_batch *b, int32_t lanes, int32_t *used);
 /* Kernel launches of one iteration of the batch (A1-A6, all bodies). */
 int32_t fppg_batch_kernels_per_iter(const fppg_batch *b);
 /* Particle count and the last error of the batch. */

@@ -80,6 +80,7 @@ def lib():
                 "fppg_work_counts": [vp, P_(i64), P_(i64), P_(i64)],
                 "fppg_debug_search": [vp, P_(i64), P_(i32)],
                 "fppg_debug_cell_lists": [vp, P_(i64), P_(i64), P_(i64)],
+                "fppg_debug_search_lanes": [vp, i32, P_(i32)],
                 "fppg_batch_load": [vp],
                 "fppg_copy_positions_dev": [vp, vp],
                 "fppg_batch_create": [P_(vp), i32, P_(vp)],
@@ -594,6 +595,13 @@ class Batch:
     def configure(self, force_variant: int = 0, force_block: int = 256, search_ctas_per_sm: int = 16):
         """Set the kernel configuration by hand (the autotuner's choices)."""
         self._chk(lib().fppg_batch_configure(self._h, int(force_variant), int(force_block), int(search_ctas_per_sm)))
+
+    def debug_search_lanes(self, lanes: int = 0) -> int:
+        """Set the lanes per particle of the triangle search (1, 8 or 32; 0
+        leaves them); returns the lanes in force."""
+        used = C.c_int32()
+        self._chk(lib().fppg_debug_search_lanes(self._h, int(lanes), C.byref(used)))
+        return used.value
 
     def phase_ms(self) -> dict:
         """Device ms per iteration of grid build, force pass, step and

@@ -234,7 +234,7 @@ int ctx_group(fppg_ctx *c) {
     g.hp[0].cascade = c->cascade;
     if (g.cell_order) g.hp[0].row_rank = g.d.row_rank;   // the body's table (fppg_set_cell_order)
     g.mesh = view_of(c->body);
-    g.set_search_lanes(c->body.n_dil, c->body.n_cand);
+    g.set_search_lanes(c->body.n_dil, c->body.n_cand + c->body.n_probe, c->body.max_probe, c->n);
     const int r = g.upload_params(c->stream, c->err);
     return r == 0 ? FPPG_OK : (r == 3 ? FPPG_ERR_OOM : FPPG_ERR_CUDA);
 }
@@ -941,6 +941,7 @@ int fppg_batch_create(fppg_ctx *const *ctxs, int32_t n, fppg_batch **out) {
     for (int32_t i = 0; i < n; i++) members[find(i)]++;
     int64_t N = 0, cells = 0, nt = 0, nv = 0, hs = 0, nc = 0, np = 0, ns = 0, nl = 0, ow = 0;
     int64_t dw = 0, dl = 0, dc = 0;   // candidate-list ranks, starts and lists
+    int64_t dp = 0, mp = 0;           // ids of the cells that are probed: in all, at most
     for (int32_t i = 0; i < n; i++) {
         const fppg_ctx *c = ctxs[i];
         const Body &bd = c->body;
@@ -1021,9 +1022,11 @@ int fppg_batch_create(fppg_ctx *const *ctxs, int32_t n, fppg_batch **out) {
         dw += bd.occ_words;
         dl += bd.n_dil + 1;
         dc += bd.n_cand;
+        dp += bd.n_probe;
+        mp = std::max(mp, bd.max_probe);
     }
     b->off.push_back(N);
-    g.set_search_lanes(dl - n, dc);      // (one more list start than cells for every body)
+    g.set_search_lanes(dl - n, dc + dp, mp, N);      // (one more list start than cells for every body)
     if (cells >= ((int64_t)1 << 29) || N > ((int64_t)1 << 31) || ow >= 0xffffffffLL || dl >= 0xffffffffLL ||
         dc >= 0x7fffffffLL) {
         delete b;
@@ -1409,6 +1412,21 @@ int fppg_batch_set_mobile_classes(fppg_batch *b, int32_t mask) {
     // the kernels read the parameters from device memory: a captured
     // graph sees the new mask without being captured again
     return b->group.upload_params(b->stream, b->err) ? FPPG_ERR_CUDA : FPPG_OK;
+}
+
+int fppg_debug_search_lanes(fppg_batch *b, int32_t lanes, int32_t *used) {
+    if (!b || (lanes != 0 && lanes != 1 && lanes != 8 && lanes != 32)) return FPPG_ERR_ARG;
+    Group &g = b->group;
+    if (lanes) {
+        g.search_thread = lanes == 1;
+        if (lanes > 1) g.search_lanes = lanes;
+        if (g.graph) {
+            cudaGraphExecDestroy(g.graph);
+            g.graph = nullptr;
+        }
+    }
+    if (used) *used = g.search_thread ? 1 : g.search_lanes;
+    return FPPG_OK;
 }
 
 int fppg_batch_configure(fppg_batch *b, int32_t variant, int32_t block, int32_t search_ctas) {

@@ -386,13 +386,21 @@ int Group::set_cell_order(int order, cudaStream_t s, std::string &err) {
     return upload_params(s, err);
 }
 
-// Lanes per queued particle from the mean candidate list of the group's
-// meshes (entries over cells).  Search per iteration with 8 and 32 lanes:
-// mean 4.2 (union pair) 8.8 / 8.9 us, 4.6 (64 bodies) 263 / 281, 4.7 (gear)
-// 21 / 45; 12.9 (icosphere + torus) 12.1 / 10.5, 16.2 (vehicle) 26 / 24, 65
-// (eight small bodies) 32 / 15.
-void Group::set_search_lanes(int64_t cells, int64_t entries) {
-    search_lanes = entries < 8 * cells ? 8 : 32;
+// Lanes per queued particle, from what one has to walk on average (entries over
+// cells, the ids of the cells that are probed included) and at most.
+// Long walks feed 32 lanes, short ones leave most of them idle.  Search per
+// iteration with 8 and 32 lanes, by the mean: 4.2 (union pair) 12.5 / 14.4 us,
+// 4.7 (gear, 2.4 M) 39.8 / 54.8, 5.8 (gear, 1.5 M) 32.9 / 46.8, 7.1 (gear, 1.1 M)
+// 24.7 / 26.8, 8.4 (gear, 0.8 M) 24.3 / 22.6, 12.9 (icosphere + torus) 16.6 / 14.4,
+// 65 (eight small bodies) 33.6 / 18.5.
+// A probed cell holds over 512 ids.  Its particles walk them with 8 lanes at
+// about 0.1 us an id, and the launch takes that long unless the others keep the
+// chip busy meanwhile.  Gears and others, longest probe / particles: 734 / 7.1 M
+// 252 / 287 us, 842 / 5.5 M 212 / 242, 842 / 3.3 M 163 / 158, 1226 / 4.7 M 206 / 213,
+// 1376 / 4.2 M 236 / 198, 1792 / 1.8 M 238 / 109, 1376 / 0.5 M 139 / 41: the line
+// lies near 4000 particles for every id.
+void Group::set_search_lanes(int64_t cells, int64_t entries, int64_t longest_probe, int64_t n) {
+    search_lanes = entries < 8 * cells && 4000 * longest_probe <= n ? 8 : 32;
 }
 
 void Group::free_all() {

@@ -51,6 +51,7 @@ struct Body {
     uint32_t *drank = nullptr, *coff = nullptr;
     int32_t *cand = nullptr;
     int64_t n_dil = 0, n_cand = 0;
+    int64_t n_probe = 0, max_probe = 0;   // ids that the probes of the cells without a list walk: in all, at most
     // feature lines (host copies + device segments)
     bool has_features = false;
     std::vector<int32_t> fe;           // [nfe][2] sorted
@@ -117,7 +118,7 @@ struct Group {
     int search_blocks = 152 * 8;  // persistent grid of the search
     bool search_thread = false;   // one thread (not a group of lanes) per queued particle
     int search_lanes = 32;        // lanes per queued particle otherwise: 8 or 32 (set_search_lanes)
-    void set_search_lanes(int64_t cells, int64_t entries);
+    void set_search_lanes(int64_t cells, int64_t entries, int64_t longest_probe, int64_t n);
     // order of the keys: the counting sort, but the radix form for a set with
     // crowded keys, unless the caller chose one (order_set).  An iteration of
     // fixed particles, counting sort / radix form: 100 of them on 8 k fine keys

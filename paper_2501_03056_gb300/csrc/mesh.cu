@@ -334,11 +334,12 @@ constexpr int kListBuf = 512;   // gathered ids per warp (with repeats); more: t
 
 // one warp per dilated cell: gather the 27 cells' triangle ids, keep the
 // first occurrence of each; WRITE = 0 counts (cnt[r], 0 and ovf[r] = 1 on
-// overflow), WRITE = 1 writes the list at off[r]
+// overflow, whose ids probed[0] adds up, probed[1] their largest number), WRITE = 1 writes the list at off[r]
 template <bool WRITE>
 __global__ void __launch_bounds__(256) k_cell_lists(AsmParams A, MeshView M, const uint32_t *__restrict__ dcell,
                                                     int64_t D, uint32_t *__restrict__ cnt, uint8_t *__restrict__ ovf,
-                                                    const uint32_t *__restrict__ off, int32_t *__restrict__ list) {
+                                                    const uint32_t *__restrict__ off, int32_t *__restrict__ list,
+                                                    unsigned long long *__restrict__ probed) {
     __shared__ int32_t sbuf[8][kListBuf];
     int32_t *buf = sbuf[threadIdx.x / 32];
     const int lane = threadIdx.x & 31;
@@ -366,6 +367,8 @@ __global__ void __launch_bounds__(256) k_cell_lists(AsmParams A, MeshView M, con
             if (!WRITE && lane == 0) {
                 cnt[r] = 0;
                 ovf[r] = 1;
+                atomicAdd(probed, (unsigned long long)total);
+                atomicMax(probed + 1, (unsigned long long)total);
             }
             __syncwarp();
             continue;
@@ -484,7 +487,7 @@ void Body::free_mesh() {
         if (p) cudaFree(p);
     drank = coff = nullptr;
     cand = nullptr;
-    n_dil = n_cand = 0;
+    n_dil = n_cand = n_probe = max_probe = 0;
     d_verts = nullptr;
     d_tris = nullptr;
     geo = vx = pn = nullptr;
@@ -693,6 +696,7 @@ int Body::build_mesh(const float *verts_host, int64_t nv_, const int32_t *tris_h
     // ---- candidate lists of the dilated cells -----------------------------
     uint32_t *wpop = nullptr, *dcell = nullptr, *lcnt = nullptr, *ltot = nullptr, *lscr = nullptr;
     uint8_t *lovf = nullptr;
+    unsigned long long *lprobe = nullptr;
     CK(dalloc(&drank, occ_words));
     CK(dalloc(&wpop, occ_words));
     CK(dalloc(&ltot, 1));
@@ -708,6 +712,8 @@ int Body::build_mesh(const float *verts_host, int64_t nv_, const int32_t *tris_h
     CK(dalloc(&lcnt, n_dil));
     CK(dalloc(&lovf, n_dil));
     CK(dalloc(&coff, n_dil + 1));
+    CK(dalloc(&lprobe, 2));
+    CK(cudaMemsetAsync(lprobe, 0, 2 * sizeof(unsigned long long), s));
     k_bit_cells<<<blocks(occ_words), 256, 0, s>>>(occ + occ_words, occ_words, drank, dcell);
     {
         AsmParams A;
@@ -716,23 +722,27 @@ int Body::build_mesh(const float *verts_host, int64_t nv_, const int32_t *tris_h
         A.hash_mask = (uint32_t)(hash_size - 1);
         const MeshView M{geo, vx, pn, hrng, compact, tlist, nullptr, nullptr, occ, nullptr, nullptr, nullptr};
         const unsigned lb = (unsigned)std::min<int64_t>(std::max<int64_t>((n_dil + 7) / 8, 1), 65535);
-        k_cell_lists<false><<<lb, 256, 0, s>>>(A, M, dcell, n_dil, lcnt, lovf, nullptr, nullptr);
+        k_cell_lists<false><<<lb, 256, 0, s>>>(A, M, dcell, n_dil, lcnt, lovf, nullptr, nullptr, lprobe);
         cudaFree(lscr);
         lsc = scan_tmp_elems(std::max<int64_t>(n_dil, 1));
         CK(dalloc(&lscr, lsc));
         exclusive_scan_u32(lcnt, coff, n_dil, coff + n_dil, lscr, lsc, s);
         uint32_t nc_ = 0;
+        unsigned long long np_[2] = {0, 0};
         CK(cudaMemcpyAsync(&nc_, coff + n_dil, 4, cudaMemcpyDeviceToHost, s));
+        CK(cudaMemcpyAsync(np_, lprobe, sizeof(np_), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         n_cand = nc_;
+        n_probe = (int64_t)np_[0];
+        max_probe = (int64_t)np_[1];
         CK(dalloc(&cand, n_cand));
-        k_cell_lists<true><<<lb, 256, 0, s>>>(A, M, dcell, n_dil, lcnt, lovf, coff, cand);
+        k_cell_lists<true><<<lb, 256, 0, s>>>(A, M, dcell, n_dil, lcnt, lovf, coff, cand, nullptr);
         k_flag_overflow<<<blocks(std::max<int64_t>(n_dil, 1)), 256, 0, s>>>(coff, lovf, n_dil);
     }
     CK(cudaStreamSynchronize(s));
     CK(cudaGetLastError());
     {
-        void *lt[] = {wpop, dcell, lcnt, ltot, lscr, lovf};
+        void *lt[] = {wpop, dcell, lcnt, ltot, lscr, lovf, lprobe};
         for (void *p : lt) cudaFree(p);
     }
     void *tmp[] = {cnt, off, total, scratch, pk[0], pk[1], pt[0], pt[1], flag, pos, cmp_unsorted,

@@ -64,3 +64,50 @@ def test_lanes_do_not_change_the_search(kind, cascade):
         got.append([a for b in bs for a in b.get_particles()])
     for other in got[1:]:
         assert all(np.array_equal(a, b) for a, b in zip(got[0], other))
+
+
+# every mesh with every number of lanes, whatever the library would take
+@pytest.mark.parametrize("cascade", [False, True])
+@pytest.mark.parametrize("kind", ["cube", "rims", "sphere", "probe"])
+def test_each_number_of_lanes_gives_the_same_bits(kind, cascade):
+    got = []
+    for lanes in (1, 8, 32):
+        bs = bodies(kind, cascade)
+        bt = pkg.Batch(bs)
+        assert bt.debug_search_lanes(lanes) == lanes
+        bt.relax(4, use_graph=False)
+        bt.store()
+        got.append([a for b in bs for a in b.get_particles()])
+    for other in got[1:]:
+        assert all(np.array_equal(a, b) for a, b in zip(got[0], other))
+
+
+def cloud_in(mesh, dx, n=2000):
+    b = pkg.Body(*mesh, dx, 1.3 * dx)
+    b.set_particles(np.random.default_rng(n).uniform(-0.2, 0.2, (n, 3)).astype(np.float32), np.full(n, W.CLS_V, np.int32))
+    return b
+
+
+def test_cells_too_long_for_a_list_count_with_their_length():
+    short = cloud_in(W.cube_mesh(0.5), 0.06)
+    assert pkg.Batch([short]).debug_search_lanes() == 8
+    # 5,120 triangles within a few cells: no cell has a list, every one is probed
+    dense = cloud_in(W.icosphere_mesh(4, 0.05), 0.2)
+    cells, entries, probed = dense.debug_cell_lists()
+    assert probed > 0 and entries < 8 * cells
+    assert pkg.Batch([dense]).debug_search_lanes() == 32
+    # one such mesh among bodies of short lists: its particles walk longest
+    flat = [cloud_in(W.cube_mesh(2.0), 0.02, 3000) for _ in range(2)]
+    mixed = flat + [dense]
+    c, e = (sum(b.debug_cell_lists()[k] for b in mixed) for k in (0, 1))
+    assert e + 27 * 5120 * probed < 8 * c
+    assert pkg.Batch(flat).debug_search_lanes() == 8
+    assert pkg.Batch(mixed).debug_search_lanes() == 32
+
+
+def test_lanes_are_checked():
+    bt = pkg.Batch([cloud_in(W.cube_mesh(0.5), 0.06)])
+    for bad in (-1, 2, 16, 64):
+        with pytest.raises(pkg.FPPGError) as e:
+            bt.debug_search_lanes(bad)
+        assert e.value.code == pkg.ERR_ARG
