@@ -354,6 +354,19 @@ int fppg_work_counts(fppg_ctx *ctx, int64_t *candidates, int64_t *pairs, int64_t
  * Synchronises the stream. */
 int fppg_energy(fppg_ctx *ctx, const float *y_dev, const float *verts_dev, double *E_host, float *gy_dev,
                 float *gV_dev);
+/* The same in two calls, for a caller that may not want the gradients.  The
+ * forward writes *E_host and leaves in state_dev (fppg_energy_state_bytes of
+ * the particle count, device memory of the caller on a 16-byte boundary) all
+ * that the backward needs of it: the body may be relaxed, given other particles
+ * or set up otherwise in between.  The state holds no address and may be moved.
+ * The backward takes the forward's n, y_dev and verts_dev.  The forward
+ * synchronises the stream, the backward does not.  FPPG_ERR_ARG for a state too
+ * small or off its boundary; fppg_energy_state_bytes is -1 for bad arguments. */
+int64_t fppg_energy_state_bytes(const fppg_ctx *ctx, int64_t n);
+int fppg_energy_forward(fppg_ctx *ctx, const float *y_dev, const float *verts_dev, double *E_host, void *state_dev,
+                        int64_t state_bytes);
+int fppg_energy_backward(fppg_ctx *ctx, int64_t n, const float *y_dev, const float *verts_dev, const void *state_dev,
+                         int64_t state_bytes, float *gy_dev, float *gV_dev);
 /* Current positions [n][3] into a device buffer (for the energy). */
 int fppg_copy_positions_dev(fppg_ctx *ctx, float *xyz_dev);
 

@@ -77,6 +77,8 @@ def lib():
                 "fppg_debug_forces": [vp, P_(f32), P_(i32), P_(f32)],
                 "fppg_project_points": [vp, P_(f32), P_(i32), P_(i32), i64, P_(f32), P_(i32), P_(i32)],
                 "fppg_energy": [vp, vp, vp, P_(f64), vp, vp],
+                "fppg_energy_forward": [vp, vp, vp, P_(f64), vp, i64],
+                "fppg_energy_backward": [vp, i64, vp, vp, vp, i64, vp, vp],
                 "fppg_work_counts": [vp, P_(i64), P_(i64), P_(i64)],
                 "fppg_debug_search": [vp, P_(i64), P_(i32)],
                 "fppg_debug_cell_lists": [vp, P_(i64), P_(i64), P_(i64)],
@@ -126,6 +128,8 @@ def lib():
             L.fppg_batch_last_error.restype = C.c_char_p
             L.fppg_batch_kernels_per_iter.argtypes = [vp]
             L.fppg_batch_kernels_per_iter.restype = C.c_int32
+            L.fppg_energy_state_bytes.argtypes = [vp, i64]
+            L.fppg_energy_state_bytes.restype = i64
             L.fppg_batch_size.argtypes = [vp]
             L.fppg_batch_size.restype = C.c_int64
             _lib = L
@@ -384,6 +388,24 @@ class Body:
         self._chk(lib().fppg_energy(self._h, C.c_void_p(y_ptr), C.c_void_p(verts_ptr or None), C.byref(E),
                                     C.c_void_p(gy_ptr or None), C.c_void_p(gv_ptr or None)))
         return E.value
+
+    def energy_state_bytes(self, n: int) -> int:
+        """Bytes that a forward over n particles leaves for its backward."""
+        return int(lib().fppg_energy_state_bytes(self._h, int(n)))
+
+    def energy_forward_ptr(self, y_ptr: int, verts_ptr: int, state_ptr: int, state_bytes: int) -> float:
+        """Energy from device pointers, with the state of its backward."""
+        E = C.c_double()
+        self._chk(lib().fppg_energy_forward(self._h, C.c_void_p(y_ptr), C.c_void_p(verts_ptr or None), C.byref(E),
+                                            C.c_void_p(state_ptr or None), int(state_bytes)))
+        return E.value
+
+    def energy_backward_ptr(self, n: int, y_ptr: int, verts_ptr: int, state_ptr: int, state_bytes: int,
+                            gy_ptr: int = 0, gv_ptr: int = 0):
+        """Gradients of a forward's energy into device buffers."""
+        self._chk(lib().fppg_energy_backward(self._h, int(n), C.c_void_p(y_ptr or None), C.c_void_p(verts_ptr or None),
+                                             C.c_void_p(state_ptr or None), int(state_bytes),
+                                             C.c_void_p(gy_ptr or None), C.c_void_p(gv_ptr or None)))
 
     def copy_positions_dev(self, ptr: int):
         self._chk(lib().fppg_copy_positions_dev(self._h, C.c_void_p(ptr)))

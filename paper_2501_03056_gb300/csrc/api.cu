@@ -885,6 +885,40 @@ int fppg_energy(fppg_ctx *ctx, const float *y_dev, const float *verts_dev, doubl
     return r == 0 ? FPPG_OK : (r == 3 ? FPPG_ERR_OOM : FPPG_ERR_CUDA);
 }
 
+int64_t fppg_energy_state_bytes(const fppg_ctx *ctx, int64_t n) {
+    if (!ctx || n < 0 || n > (int64_t)1 << 31) return -1;
+    return energy_state_bytes(n, ctx->group.d.total_cells);
+}
+
+int fppg_energy_forward(fppg_ctx *ctx, const float *y_dev, const float *verts_dev, double *E_host, void *state_dev,
+                        int64_t state_bytes) {
+    if (!ctx || !y_dev || !E_host) return FPPG_ERR_ARG;
+    if (!ctx->has_particles) return fail(ctx->err, FPPG_ERR_STATE, "no particles set");
+    if (ctx->n == 0) {
+        *E_host = 0.0;
+        return FPPG_OK;
+    }
+    if (!state_dev || ((uintptr_t)state_dev & 15u) || state_bytes < fppg_energy_state_bytes(ctx, ctx->n))
+        return fail(ctx->err, FPPG_ERR_ARG, "the state needs fppg_energy_state_bytes bytes on a 16-byte boundary");
+    const int r = energy_forward(ctx->group, ctx->body, y_dev, verts_dev, E_host, state_dev, ctx->stream, ctx->err);
+    return r == 0 ? FPPG_OK : (r == 3 ? FPPG_ERR_OOM : FPPG_ERR_CUDA);
+}
+
+int fppg_energy_backward(fppg_ctx *ctx, int64_t n, const float *y_dev, const float *verts_dev, const void *state_dev,
+                         int64_t state_bytes, float *gy_dev, float *gV_dev) {
+    if (!ctx || n < 0 || n > (int64_t)1 << 31 || (n > 0 && !y_dev)) return FPPG_ERR_ARG;
+    if (n == 0) {
+        if (gV_dev)
+            CUDA_OR(ctx->err, cudaMemsetAsync(gV_dev, 0, sizeof(float) * 3 * (size_t)ctx->body.nv, ctx->stream));
+        return FPPG_OK;
+    }
+    if (!state_dev || ((uintptr_t)state_dev & 15u) || state_bytes < fppg_energy_state_bytes(ctx, n))
+        return fail(ctx->err, FPPG_ERR_ARG, "not the state of a forward of this body and count");
+    const int r = energy_backward(ctx->group, ctx->body, n, y_dev, verts_dev, state_dev, gy_dev, gV_dev, ctx->stream,
+                                  ctx->err);
+    return r == 0 ? FPPG_OK : (r == 3 ? FPPG_ERR_OOM : FPPG_ERR_CUDA);
+}
+
 int fppg_copy_positions_dev(fppg_ctx *ctx, float *xyz_dev) {
     if (!ctx || !xyz_dev) return FPPG_ERR_ARG;
     if (!ctx->has_particles) return fail(ctx->err, FPPG_ERR_STATE, "no particles set");

@@ -92,12 +92,18 @@ AsmParams make_params(const Body &b, uint32_t key_base, int p_begin, int p_end, 
 
 // scratch of the energy and its backward (energy.cu), kept between calls
 struct EnergyScratch {
+    AsmParams *params = nullptr;
     float4 *xs = nullptr, *vcon = nullptr;
     double *e_s = nullptr, *part = nullptr;
     uint32_t *vk[2] = {nullptr, nullptr}, *vi[2] = {nullptr, nullptr}, *hist = nullptr, *tot = nullptr;
     int64_t n = 0;   // particles it is sized for
+    // the last backward, which returns before it is done: work on another
+    // stream waits for it
+    cudaEvent_t done = nullptr;
+    cudaStream_t done_on = nullptr;
     void release() {
-        void *p[] = {xs, vcon, e_s, part, vk[0], vk[1], vi[0], vi[1], hist, tot};
+        if (done) cudaEventDestroy(done);
+        void *p[] = {params, xs, vcon, e_s, part, vk[0], vk[1], vi[0], vi[1], hist, tot};
         for (void *q : p)
             if (q) cudaFree(q);
         *this = EnergyScratch();
@@ -211,5 +217,12 @@ void ray_parity(const Group &other, const float4 *pos, int64_t n, int32_t *insid
 // energy and gradients (positions y, vertex coordinates verts of body 0)
 int energy(Group &g, const Body &b, const float *y_dev, const float *verts_dev, double *E, float *gy, float *gV,
            cudaStream_t s, std::string &err);
+// the same in two calls: the forward leaves what the backward needs in `state`
+// (device, energy_state_bytes of the particle count, on 16 bytes)
+int64_t energy_state_bytes(int64_t N, int64_t total_cells);
+int energy_forward(Group &g, const Body &b, const float *y_dev, const float *verts_dev, double *E, void *state,
+                   cudaStream_t s, std::string &err);
+int energy_backward(Group &g, const Body &b, int64_t N, const float *y_dev, const float *verts_dev, const void *state,
+                    float *gy, float *gV, cudaStream_t s, std::string &err);
 
 } // namespace fppg

@@ -226,17 +226,17 @@ __global__ void k_project_frozen(const float *__restrict__ y, const float4 *__re
 // vkey[3k + c] / vcon[3k + c]: vertex and contribution of corner c of the
 // frozen triangle of the particle in key slot k (vertex nv = none)
 __global__ void k_vjp(const float4 *__restrict__ gx_s, const uint32_t *__restrict__ id_s, int64_t N,
-                      const float *__restrict__ y, const float4 *__restrict__ pos, const int32_t *__restrict__ cons,
+                      const float *__restrict__ y, const float4 *__restrict__ pos_s, const int32_t *__restrict__ cons_s,
                       const float *__restrict__ V, const int32_t *__restrict__ T, int nv, float *__restrict__ gy,
                       uint32_t *__restrict__ vkey, float4 *__restrict__ vcon) {
     const int64_t k = (int64_t)blockIdx.x * TPB + threadIdx.x;
     if (k >= N) return;
     const uint32_t i = id_s[k];
     const float3 g = f3(gx_s[k]);
-    const int t = cons[i];
+    const int t = cons_s[k];
     if (vkey)
         for (int c = 0; c < 3; c++) vkey[3 * k + c] = (uint32_t)nv;
-    if (!(cls_of(pos[i].w) == kClsS && t >= 0)) {
+    if (!(cls_of(pos_s[k].w) == kClsS && t >= 0)) {
         if (gy) {
             gy[3 * (size_t)i] = g.x;
             gy[3 * (size_t)i + 1] = g.y;
@@ -293,6 +293,50 @@ __global__ void k_vertex_sum(const uint32_t *__restrict__ vkey_s, const uint32_t
     gV[3 * (size_t)v + 2] = (float)sz;
 }
 
+// a body's parameters into or out of a forward's state, which holds whether the
+// rows were ranked instead of the table's address
+__global__ void k_copy_params(const AsmParams *__restrict__ in, const uint32_t *__restrict__ in_ranked,
+                              const uint32_t *__restrict__ table, AsmParams *__restrict__ out,
+                              uint32_t *__restrict__ out_ranked) {
+    static_assert(sizeof(AsmParams) % 4 == 0, "copied by words");
+    for (int q = threadIdx.x; q < (int)(sizeof(AsmParams) / 4); q += blockDim.x)
+        reinterpret_cast<uint32_t *>(out)[q] = reinterpret_cast<const uint32_t *>(in)[q];
+    __syncthreads();
+    if (threadIdx.x > 0) return;
+    if (out_ranked) *out_ranked = in->row_rank != nullptr;
+    out->row_rank = in_ranked && *in_ranked ? table : nullptr;
+}
+
+// What a backward needs of its forward, in key order: the grid of the projected
+// positions, the kernel sums' coefficients, the constraints and the parameters
+struct ForwardState {
+    AsmParams *params;
+    uint32_t *ranked;          // the rows of the grid were in Morton order
+    float4 *pos_s, *pos_p;
+    float *coef_s, *coef_v;
+    uint32_t *fstart, *id_s;
+    int32_t *cons_s;
+};
+
+// the state's parts in a block at `base`; returns its size in bytes
+int64_t lay_out(int64_t N, int64_t total_cells, char *base, ForwardState *st) {
+    int64_t at = 0;
+    auto take = [&](auto **p, int64_t n) {
+        *p = reinterpret_cast<std::remove_reference_t<decltype(**p)> *>(base + at);
+        at += ((int64_t)sizeof(**p) * n + 15) / 16 * 16;
+    };
+    take(&st->params, 1);
+    take(&st->ranked, 1);
+    take(&st->pos_s, N);
+    take(&st->pos_p, N + 1);
+    take(&st->coef_s, N + 1);
+    take(&st->coef_v, N + 1);
+    take(&st->fstart, kSlabs * total_cells + 1);
+    take(&st->id_s, N);
+    take(&st->cons_s, N);
+    return at;
+}
+
 } // namespace
 
 // the volume particles' coefficients live in the search queue's memory, which
@@ -310,13 +354,15 @@ void energy_accel(Group &g, cudaStream_t s) {
 // The scratch of energy(): kept in the group between calls (allocated on the
 // first call, grown when the particle count grows), so a repeated energy and
 // backward costs no allocation and no implicit device synchronisation.
-static int energy_scratch(Group &g, int64_t N, std::string &err) {
+static int energy_scratch(Group &g, int64_t N, cudaStream_t s, std::string &err) {
     EnergyScratch &e = g.escr;
+    if (e.done_on != s && e.done) cudaStreamWaitEvent(s, e.done, 0);
     if (e.n >= N && e.xs) return 0;
     e.release();
     const int64_t M = 3 * N;
     const size_t n1 = (size_t)std::max<int64_t>(N, 1), m1 = (size_t)std::max<int64_t>(M, 1);
-    if (dev_malloc(&e.xs, sizeof(float4) * n1) != cudaSuccess ||
+    if (cudaEventCreateWithFlags(&e.done, cudaEventDisableTiming) != cudaSuccess ||
+        dev_malloc(&e.params, sizeof(AsmParams)) != cudaSuccess || dev_malloc(&e.xs, sizeof(float4) * n1) != cudaSuccess ||
         dev_malloc(&e.e_s, sizeof(double) * n1) != cudaSuccess ||
         dev_malloc(&e.part, sizeof(double) * (kSumBlocks + 1)) != cudaSuccess ||
         dev_malloc(&e.vcon, sizeof(float4) * m1) != cudaSuccess ||
@@ -332,11 +378,40 @@ static int energy_scratch(Group &g, int64_t N, std::string &err) {
     return 0;
 }
 
+// E from the kernel sums' terms in es.e_s, to the host; waits for s
+static int read_energy(EnergyScratch &es, int64_t N, double *E, cudaStream_t s, std::string &err) {
+    k_sum_fixed<<<kSumBlocks, TPB, 0, s>>>(es.e_s, N, es.part);
+    k_sum_fixed<<<1, TPB, 0, s>>>(es.part, kSumBlocks, es.part + kSumBlocks);
+    cudaMemcpyAsync(E, es.part + kSumBlocks, sizeof(double), cudaMemcpyDeviceToHost, s);
+    cudaError_t e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e != cudaSuccess) {
+        err = std::string("energy: ") + cudaGetErrorString(e);
+        return 4;
+    }
+    return 0;
+}
+
+// the gradients from dE/dx in key order (gx_s)
+static void pull_back(EnergyScratch &es, const Body &b, int64_t N, const float *y_dev, const float *V,
+                      const float4 *gx_s, const uint32_t *id_s, const float4 *pos_s, const int32_t *cons_s, float *gy,
+                      float *gV, cudaStream_t s) {
+    const int64_t M = 3 * N;          // vertex contributions (three per particle)
+    k_vjp<<<nblocks(N), TPB, 0, s>>>(gx_s, id_s, N, y_dev, pos_s, cons_s, V, b.d_tris, b.nv, gy,
+                                      gV ? es.vk[0] : nullptr, es.vcon);
+    if (!gV) return;
+    cudaMemsetAsync(gV, 0, sizeof(float) * 3 * (size_t)b.nv, s);
+    int bits = 1;
+    while (bits < 32 && ((uint64_t)b.nv >> bits) != 0) bits++;
+    const int vb = radix_sort_u32(es.vk, es.vi, true, M, bits, es.hist, es.tot, s);
+    k_vertex_sum<<<nblocks(M), TPB, 0, s>>>(es.vk[vb], es.vi[vb], M, es.vcon, b.nv, gV);
+}
+
 int energy(Group &g, const Body &b, const float *y_dev, const float *verts_dev, double *E, float *gy, float *gV,
            cudaStream_t s, std::string &err) {
     DevGroup &d = g.d;
-    const int64_t N = d.N, M = 3 * N;          // M: vertex contributions (three per particle)
-    if (const int r = energy_scratch(g, N, err)) return r;
+    const int64_t N = d.N;
+    if (const int r = energy_scratch(g, N, s, err)) return r;
     EnergyScratch &es = g.escr;
     const float *V = verts_dev ? verts_dev : b.d_verts;
     float4 *saved = d.pos;
@@ -346,26 +421,68 @@ int energy(Group &g, const Body &b, const float *y_dev, const float *verts_dev, 
     d.pos = saved;
     k_rho<<<nblocks(N + 1), TPB, 0, s>>>(d.pos_s, d.pos_p, N, d.params, d.fstart, d.coef_s,
                                           gy || gV ? volume_coefs(d) : nullptr, es.e_s);
-    k_sum_fixed<<<kSumBlocks, TPB, 0, s>>>(es.e_s, N, es.part);
-    k_sum_fixed<<<1, TPB, 0, s>>>(es.part, kSumBlocks, es.part + kSumBlocks);
     if (gy || gV) {
         k_grad<<<nblocks(N), TPB, 0, s>>>(d.pos_s, d.pos_p, N, d.params, d.fstart, d.coef_s, volume_coefs(d), 1.f,
                                           d.acc_s, nullptr);
-        k_vjp<<<nblocks(N), TPB, 0, s>>>(d.acc_s, d.id_s, N, y_dev, d.pos, d.cons, V, b.d_tris, b.nv, gy,
-                                          gV ? es.vk[0] : nullptr, es.vcon);
-        if (gV) {
-            cudaMemsetAsync(gV, 0, sizeof(float) * 3 * (size_t)b.nv, s);
-            int bits = 1;
-            while (bits < 32 && ((uint64_t)b.nv >> bits) != 0) bits++;
-            const int vb = radix_sort_u32(es.vk, es.vi, true, M, bits, es.hist, es.tot, s);
-            k_vertex_sum<<<nblocks(M), TPB, 0, s>>>(es.vk[vb], es.vi[vb], M, es.vcon, b.nv, gV);
-        }
+        pull_back(es, b, N, y_dev, V, d.acc_s, d.id_s, d.pos_s, d.cons_s, gy, gV, s);
     }
-    cudaMemcpyAsync(E, es.part + kSumBlocks, sizeof(double), cudaMemcpyDeviceToHost, s);
-    cudaError_t e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess) e = cudaGetLastError();
+    return read_energy(es, N, E, s, err);
+}
+
+int64_t energy_state_bytes(int64_t N, int64_t total_cells) {
+    ForwardState st;
+    return lay_out(N, total_cells, nullptr, &st);
+}
+
+// The grid is built in the state (the group's own arrays keep what a split
+// iteration left in them), so the backward starts at k_grad and nothing of it
+// is done before it is asked for: torus, 237 k particles, forward alone
+// 221 us (with the gradients made in it 368, without a state 199), with its
+// backward 520 (584).
+int energy_forward(Group &g, const Body &b, const float *y_dev, const float *verts_dev, double *E, void *state,
+                   cudaStream_t s, std::string &err) {
+    DevGroup &d = g.d;
+    const int64_t N = d.N;
+    if (const int r = energy_scratch(g, N, s, err)) return r;
+    EnergyScratch &es = g.escr;
+    ForwardState st;
+    lay_out(N, d.total_cells, static_cast<char *>(state), &st);
+    const float *V = verts_dev ? verts_dev : b.d_verts;
+    k_copy_params<<<1, 128, 0, s>>>(d.params, nullptr, nullptr, st.params, st.ranked);
+    k_project_frozen<<<nblocks(N), TPB, 0, s>>>(y_dev, d.pos, d.cons, N, V, b.d_tris, es.xs);
+    DevGroup w = d;
+    w.pos = es.xs;
+    w.pos_s = st.pos_s;
+    w.pos_p = st.pos_p;
+    w.fstart = st.fstart;
+    w.cons_s = st.cons_s;
+    w.key[0] = es.vk[0];
+    w.key[1] = d.counted ? st.id_s : es.vk[1];     // (where the counted form leaves the order)
+    w.id[0] = es.vi[0];
+    w.id[1] = es.vi[1];
+    build_grid_dev(w, s);
+    if (w.id_s != st.id_s)
+        cudaMemcpyAsync(st.id_s, w.id_s, sizeof(uint32_t) * (size_t)N, cudaMemcpyDeviceToDevice, s);
+    k_rho<<<nblocks(N + 1), TPB, 0, s>>>(st.pos_s, st.pos_p, N, d.params, st.fstart, st.coef_s, st.coef_v, es.e_s);
+    return read_energy(es, N, E, s, err);
+}
+
+int energy_backward(Group &g, const Body &b, int64_t N, const float *y_dev, const float *verts_dev, const void *state,
+                    float *gy, float *gV, cudaStream_t s, std::string &err) {
+    DevGroup &d = g.d;
+    if (const int r = energy_scratch(g, N, s, err)) return r;
+    EnergyScratch &es = g.escr;
+    ForwardState st;
+    lay_out(N, d.total_cells, static_cast<char *>(const_cast<void *>(state)), &st);
+    k_copy_params<<<1, 128, 0, s>>>(st.params, st.ranked, d.row_rank, es.params, nullptr);
+    k_grad<<<nblocks(N), TPB, 0, s>>>(st.pos_s, st.pos_p, N, es.params, st.fstart, st.coef_s, st.coef_v, 1.f, es.xs,
+                                      nullptr);
+    pull_back(es, b, N, y_dev, verts_dev ? verts_dev : b.d_verts, es.xs, st.id_s, st.pos_s, st.cons_s, gy, gV, s);
+    cudaEventRecord(es.done, s);
+    es.done_on = s;
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
-        err = std::string("energy: ") + cudaGetErrorString(e);
+        err = std::string("energy backward: ") + cudaGetErrorString(e);
         return 4;
     }
     return 0;
