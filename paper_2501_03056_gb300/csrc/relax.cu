@@ -159,11 +159,13 @@ __global__ void __launch_bounds__(TPB) k_keys(const float4 *__restrict__ pos, in
 
 __global__ void __launch_bounds__(TPB) k_keys_count(const float4 *__restrict__ pos, int64_t N,
                                                     const AsmParams *__restrict__ P, uint32_t *__restrict__ key,
-                                                    uint32_t *__restrict__ place, uint32_t *__restrict__ cnt) {
+                                                    uint32_t *__restrict__ place, uint32_t *__restrict__ cnt,
+                                                    int64_t F) {
     const int64_t i = (int64_t)blockIdx.x * TPB + threadIdx.x;
     if (i >= N) return;
     const float4 p = pos[i];
-    const uint32_t k = fine_key_of(P[body_of(p.w)], p.x, p.y, p.z);
+    uint32_t k = fine_key_of(P[body_of(p.w)], p.x, p.y, p.z);
+    if (!FPPG_CHECK(k < F, kChkGather)) k = 0u;
     key[i] = k;
     place[i] = atomicAdd(cnt + k, 1u);
 }
@@ -277,11 +279,13 @@ __global__ void __launch_bounds__(TPB) k_count_starts(const uint32_t *__restrict
 
 // the counts alone, then their maximum where it passes kCrowd, and 0 again
 __global__ void __launch_bounds__(TPB) k_crowd_counts(const float4 *__restrict__ pos, int64_t N,
-                                                      const AsmParams *__restrict__ P, uint32_t *__restrict__ cnt) {
+                                                      const AsmParams *__restrict__ P, uint32_t *__restrict__ cnt,
+                                                      int64_t F) {
     const int64_t i = (int64_t)blockIdx.x * TPB + threadIdx.x;
     if (i >= N) return;
     const float4 p = pos[i];
-    atomicAdd(cnt + fine_key_of(P[body_of(p.w)], p.x, p.y, p.z), 1u);
+    const uint32_t k = fine_key_of(P[body_of(p.w)], p.x, p.y, p.z);
+    if (FPPG_CHECK(k < F, kChkGather)) atomicAdd(cnt + k, 1u);
 }
 
 __global__ void __launch_bounds__(TPB) k_crowd_max(uint32_t *__restrict__ cnt, int64_t F1, uint32_t *__restrict__ most) {
@@ -309,7 +313,7 @@ __global__ void __launch_bounds__(TPB) k_place(const uint32_t *__restrict__ key,
     for (int64_t f = i; f < nv; f += (int64_t)gridDim.x * TPB)
         reinterpret_cast<uint4 *>(cnt)[f] = make_uint4(0u, 0u, 0u, 0u);
     if (i < F1 - 4 * nv) cnt[4 * nv + i] = 0u;
-    if (i >= N) return;
+    if (i >= N || !FPPG_CHECK(key[i] < F1 - 1, kChkGather)) return;
     const uint32_t k = fstart[key[i]] + place[i];
     if (FPPG_CHECK(k < N, kChkGather)) id_a[k] = (uint32_t)i;
 }
@@ -346,7 +350,8 @@ __global__ void __launch_bounds__(TPB) k_rank_gather(const uint32_t *__restrict_
                                                      const uint32_t *__restrict__ fstart,
                                                      const float4 *__restrict__ pos, const int32_t *__restrict__ cons,
                                                      int64_t N, float4 *__restrict__ pos_s, float4 *__restrict__ pos_p,
-                                                     uint32_t *__restrict__ id_s, int32_t *__restrict__ cons_s) {
+                                                     uint32_t *__restrict__ id_s, int32_t *__restrict__ cons_s,
+                                                     int64_t F) {
     constexpr int kGatherTile = kGatherItems * TPB;
     __shared__ float4 s_pos[kGatherTile];
     __shared__ uint32_t s_id[kGatherTile];
@@ -374,8 +379,12 @@ __global__ void __launch_bounds__(TPB) k_rank_gather(const uint32_t *__restrict_
         if (id[u] != kNone) {
             // (the key again: cheaper than a gather of the stored one)
             const uint32_t f = fine_key_of(P[body_of(q[u].w)], q[u].x, q[u].y, q[u].z);
-            s[u] = fstart[f];
-            e[u] = fstart[f + 1u];
+            if (FPPG_CHECK(f < F, kChkGather)) {
+                s[u] = fstart[f];
+                e[u] = fstart[f + 1u];
+            } else {
+                id[u] = kNone;
+            }
         }
     __syncthreads();
 #pragma unroll
@@ -384,6 +393,7 @@ __global__ void __launch_bounds__(TPB) k_rank_gather(const uint32_t *__restrict_
         uint32_t slot = s[u];
         if (e[u] - s[u] > 1u && FPPG_CHECK(s[u] <= e[u] && e[u] <= N, kChkGather))
             for (uint32_t j = s[u]; j < e[u]; j++) slot += id_a[j] < id[u] ? 1u : 0u;
+        if (!FPPG_CHECK(slot < N, kChkGather)) continue;
         const int64_t l = (int64_t)slot - k0;
         if (l >= 0 && l < kGatherTile) {
             s_pos[l] = q[u];
@@ -1505,7 +1515,7 @@ __global__ void k_project_points(const float *__restrict__ y, const int32_t *__r
 // id, id[1] the ids in arrival order, key[1] the ids in key order
 static void build_counted(DevGroup &d, cudaStream_t s) {
     const int64_t F1 = kSlabs * d.total_cells + 1, nt = count_tiles(F1);
-    k_keys_count<<<nblocks(d.N), TPB, 0, s>>>(d.pos, d.N, d.params, d.key[0], d.id[0], d.cnt);
+    k_keys_count<<<nblocks(d.N), TPB, 0, s>>>(d.pos, d.N, d.params, d.key[0], d.id[0], d.cnt, F1 - 1);
     const uint32_t *tiles = nullptr;
     if (nt > kFewTiles) {
         k_tile_sums<<<(unsigned)nt, TPB, 0, s>>>(d.cnt, F1, d.tiles);
@@ -1525,10 +1535,10 @@ static void build_counted(DevGroup &d, cudaStream_t s) {
                                                                             d.cnt, F1);
     if (d.N < kGatherTwoMinN)
         k_rank_gather<1><<<nblocks(d.N), TPB, 0, s>>>(d.id[1], d.params, d.fstart, d.pos, d.cons, d.N, d.pos_s,
-                                                      d.pos_p, d.id_s, d.cons_s);
+                                                      d.pos_p, d.id_s, d.cons_s, F1 - 1);
     else
         k_rank_gather<2><<<nblocks(d.N, 2 * TPB), TPB, 0, s>>>(d.id[1], d.params, d.fstart, d.pos, d.cons, d.N,
-                                                               d.pos_s, d.pos_p, d.id_s, d.cons_s);
+                                                               d.pos_s, d.pos_p, d.id_s, d.cons_s, F1 - 1);
 }
 
 int Group::find_crowds(cudaStream_t s, bool *found, std::string &err) {
@@ -1537,7 +1547,7 @@ int Group::find_crowds(cudaStream_t s, bool *found, std::string &err) {
     if (d.N > kCrowd) {
         const int64_t F1 = kSlabs * d.total_cells + 1;
         e = cudaMemsetAsync(d.totals, 0, sizeof(uint32_t), s);
-        k_crowd_counts<<<nblocks(d.N), TPB, 0, s>>>(d.pos, d.N, d.params, d.cnt);
+        k_crowd_counts<<<nblocks(d.N), TPB, 0, s>>>(d.pos, d.N, d.params, d.cnt, F1 - 1);
         k_crowd_max<<<std::min<unsigned>(nblocks(F1, 16 * TPB), 152 * 8), TPB, 0, s>>>(d.cnt, F1, d.totals);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&most, d.totals, sizeof(most), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
