@@ -696,10 +696,11 @@ int Body::build_mesh(const float *verts_host, int64_t nv_, const int32_t *tris_h
     // ---- candidate lists of the dilated cells -----------------------------
     uint32_t *wpop = nullptr, *dcell = nullptr, *lcnt = nullptr, *ltot = nullptr, *lscr = nullptr;
     uint8_t *lovf = nullptr;
-    unsigned long long *lprobe = nullptr;
     CK(dalloc(&drank, occ_words));
     CK(dalloc(&wpop, occ_words));
-    CK(dalloc(&ltot, 1));
+    CK(dalloc(&ltot, 6));     // a total, (one unused,) the ids of the probed cells: two 64-bit words
+    unsigned long long *const lprobe = reinterpret_cast<unsigned long long *>(ltot + 2);
+    CK(cudaMemsetAsync(lprobe, 0, 2 * sizeof(unsigned long long), s));
     int64_t lsc = scan_tmp_elems(occ_words);
     CK(dalloc(&lscr, lsc));
     k_word_popc<<<blocks(occ_words), 256, 0, s>>>(occ + occ_words, occ_words, wpop);
@@ -712,8 +713,6 @@ int Body::build_mesh(const float *verts_host, int64_t nv_, const int32_t *tris_h
     CK(dalloc(&lcnt, n_dil));
     CK(dalloc(&lovf, n_dil));
     CK(dalloc(&coff, n_dil + 1));
-    CK(dalloc(&lprobe, 2));
-    CK(cudaMemsetAsync(lprobe, 0, 2 * sizeof(unsigned long long), s));
     k_bit_cells<<<blocks(occ_words), 256, 0, s>>>(occ + occ_words, occ_words, drank, dcell);
     {
         AsmParams A;
@@ -742,7 +741,7 @@ int Body::build_mesh(const float *verts_host, int64_t nv_, const int32_t *tris_h
     CK(cudaStreamSynchronize(s));
     CK(cudaGetLastError());
     {
-        void *lt[] = {wpop, dcell, lcnt, ltot, lscr, lovf, lprobe};
+        void *lt[] = {wpop, dcell, lcnt, ltot, lscr, lovf};
         for (void *p : lt) cudaFree(p);
     }
     void *tmp[] = {cnt, off, total, scratch, pk[0], pk[1], pt[0], pt[1], flag, pos, cmp_unsorted,
