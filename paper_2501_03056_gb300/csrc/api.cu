@@ -400,21 +400,14 @@ int fppg_map_particles(fppg_ctx *ctx, const fppg_map_opts *opts, int64_t *n_out)
     ctx->has_particles = false;     // until the new set is complete
     ctx->split = false;
     int r = map_particles(ctx->group, ctx->body, opts->surface, opts->volume, opts->features, opts->band_cells,
-                          opts->band_cells > 0 ? opts->inner_cells : 0, ctx->stream, &n, ctx->cls_host,
+                          opts->band_cells > 0 ? opts->inner_cells : 0, ctx->stream,
+                          ctx->fixed_features || !(ctx->mobile_mask & (1 << FPPG_F)), &n, ctx->cls_host, &ctx->n_still,
                           ctx->err);
     if (r) {
         forget_lost_particles(ctx);
         return r == 1 ? FPPG_ERR_ARG : (r == 3 ? FPPG_ERR_OOM : (r == 6 ? FPPG_ERR_INTERNAL : FPPG_ERR_CUDA));
     }
     ctx->n = n;
-    // (cells and feature points are a spacing apart; only the singular points,
-    // mesh vertices at the front with the features, can share keys)
-    ctx->n_still = 0;
-    for (int32_t c : ctx->cls_host) {
-        if (c != FPPG_F && c != FPPG_P) break;
-        ctx->n_still += c == FPPG_P;
-    }
-    if ((r = ctx_crowds(ctx))) return r;
     ctx->has_particles = true;
     if (n_out) *n_out = n;
     return ctx_group(ctx);

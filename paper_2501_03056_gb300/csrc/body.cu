@@ -90,10 +90,41 @@ void Body::build_lines() {
     nseg_own = nseg;
     nlines = (int)line_first.size();
     has_features = true;
+    sing_crowd = singular_crowd();
+}
+
+// the largest number of singular vertices on one fine key of the neighbour grid
+// (an upper bound while that is at most kCrowd): the x-slabs alone tell for most
+// meshes, the vertices of the fuller ones are sorted by key
+uint32_t Body::singular_crowd() const {
+    if (sing.size() <= (size_t)kCrowd) return (uint32_t)sing.size();
+    auto fine = [&](int32_t v, int k, int per_cell) {
+        const float t = (verts_host[3 * (size_t)v + k] - ng_o[k]) * ng_inv * (float)per_cell;
+        return (uint64_t)std::min(std::max(t, 0.f), (float)(per_cell * ng_n[k] - 1));
+    };
+    std::vector<uint32_t> slab((size_t)kSlabs * (size_t)ng_n[0], 0u);
+    for (int32_t v : sing) slab[fine(v, 0, kSlabs)]++;
+    uint32_t most = *std::max_element(slab.begin(), slab.end());
+    if (most <= kCrowd) return most;
+    std::vector<uint64_t> key;
+    for (int32_t v : sing) {
+        const uint64_t fx = fine(v, 0, kSlabs);
+        if (slab[fx] > kCrowd)
+            key.push_back(fx + (uint64_t)slab.size() * (fine(v, 1, 1) + (uint64_t)ng_n[1] * fine(v, 2, 1)));
+    }
+    std::sort(key.begin(), key.end());
+    most = 0u;
+    uint32_t run = 0u;
+    for (size_t i = 0; i < key.size(); i++) {
+        run = i && key[i] == key[i - 1] ? run + 1 : 1;
+        most = std::max(most, run);
+    }
+    return most;
 }
 
 void Body::drop_features() {
     has_features = false;
+    sing_crowd = 0u;
     fe.clear();
     sing.clear();
     line_first.clear();

@@ -56,6 +56,8 @@ struct Body {
     bool has_features = false;
     std::vector<int32_t> fe;           // [nfe][2] sorted
     std::vector<int32_t> sing;         // singular vertices
+    uint32_t sing_crowd = 0;           // the most of them on one fine key (singular_crowd)
+    uint32_t singular_crowd() const;
     std::vector<int64_t> line_first, line_nseg;
     std::vector<int32_t> line_closed;
     std::vector<int32_t> seg_v;        // [nseg][2]
@@ -134,7 +136,10 @@ struct Group {
     void choose_order() {
         if (!order_set) d.counted = !crowded;
     }
-    // whether some key holds more than kCrowd particles now; waits for s
+    // whether some key holds more than kCrowd particles now; waits for s.  Of the
+    // first n alone, without waiting: the largest number (0 up to kCrowd) in the
+    // device word that count_crowds returns
+    uint32_t *count_crowds(int64_t n, cudaStream_t s);
     int find_crowds(cudaStream_t s, bool *found, std::string &err);
     int force_block = 256;        // threads per block of the force kernel (multiple of 32, <= 256)
     int force_variant = 0;        // 0 per-lane rows, 1 shared-row union
@@ -210,7 +215,8 @@ int stats(Group &g, cudaStream_t s, double *mean, double *sd, double *minpair, d
           std::string &err);
 // initial particles of Sec. 3.2 into the group (features, surface, volume)
 int map_particles(Group &g, Body &b, int surface, int volume, int features, int band_cells, int inner_cells,
-                  cudaStream_t s, int64_t *n_out, std::vector<int32_t> &cls_host, std::string &err);
+                  cudaStream_t s, bool fixed_features, int64_t *n_out, std::vector<int32_t> &cls_host,
+                  int64_t *n_singular, std::string &err);
 // Boolean union: inside[i] (device) = ray parity (Fig. 6, FP64) of point i
 // against body 0 of group `other`
 void ray_parity(const Group &other, const float4 *pos, int64_t n, int32_t *inside, cudaStream_t s);

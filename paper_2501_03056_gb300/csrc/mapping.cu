@@ -472,7 +472,8 @@ void Body::feature_particles(std::vector<float> &xyz, std::vector<int32_t> &cls,
 }
 
 int map_particles(Group &g, Body &b, int surface, int volume, int features, int band_cells, int inner_cells,
-                  cudaStream_t s, int64_t *n_out, std::vector<int32_t> &cls_host, std::string &err) {
+                  cudaStream_t s, bool fixed_features, int64_t *n_out, std::vector<int32_t> &cls_host,
+                  int64_t *n_singular, std::string &err) {
     MapGrid mg;
     for (int k = 0; k < 3; k++) {
         mg.o[k] = b.tg_o[k];
@@ -583,8 +584,10 @@ int map_particles(Group &g, Body &b, int surface, int volume, int features, int 
         return 3;
     }
     std::vector<float4> p4(nf);
+    int64_t np = 0;                // singular points
     if (nf) {
         for (int64_t i = 0; i < nf; i++) {
+            np += fcls[i] == kClsP;
             uint32_t bits = class_bit(fcls[i]);
             float w;
             memcpy(&w, &bits, 4);
@@ -603,13 +606,21 @@ int map_particles(Group &g, Body &b, int surface, int volume, int features, int 
                                                         g.d.pos + nf, g.d.cons + nf);
     k_emit_volume<<<nblk(words), 256, 0, s>>>(vbits, off + words, band, words, first, mg, g.d.pos + nf, g.d.cons + nf,
                                               vcls);
+    // keys with many fixed particles (Group::find_crowds): cells are a spacing
+    // apart, but singular points and the feature points of different lines are not
+    uint32_t most = np ? b.sing_crowd : 0u;
+    uint32_t *const crowd = fixed_features && nf > (int64_t)kCrowd ? g.count_crowds(nf, s) : nullptr;
     std::vector<uint8_t> vc(band ? (size_t)nvol : 0);
     bool done = vc.empty() || ok(cudaMemcpyAsync(vc.data(), vcls, vc.size(), cudaMemcpyDeviceToHost, s));
     // the classes on the host: features as given, then S, then V (or as copied)
     cls_host.resize((size_t)N);
     std::copy(fcls.begin(), fcls.end(), cls_host.begin());
     std::fill(cls_host.begin() + nf, cls_host.begin() + nf + ns, (int32_t)kClsS);
+    if (crowd) done = ok(cudaMemcpyAsync(&most, crowd, sizeof(most), cudaMemcpyDeviceToHost, s)) && done;
     done = ok(cudaStreamSynchronize(s)) && done && ok(cudaGetLastError());
+    g.crowded = most > kCrowd;
+    g.choose_order();
+    *n_singular = np;
     if (vc.empty()) std::fill(cls_host.begin() + nf + ns, cls_host.end(), (int32_t)kClsV);
     else std::copy(vc.begin(), vc.end(), cls_host.begin() + nf + ns);
     cleanup();

@@ -1541,15 +1541,20 @@ static void build_counted(DevGroup &d, cudaStream_t s) {
                                                                d.pos_s, d.pos_p, d.id_s, d.cons_s, F1 - 1);
 }
 
+uint32_t *Group::count_crowds(int64_t n, cudaStream_t s) {
+    const int64_t F1 = kSlabs * d.total_cells + 1;
+    cudaMemsetAsync(d.totals, 0, sizeof(uint32_t), s);
+    k_crowd_counts<<<nblocks(n), TPB, 0, s>>>(d.pos, n, d.params, d.cnt, F1 - 1);
+    k_crowd_max<<<std::min<unsigned>(nblocks(F1, 16 * TPB), 152 * 8), TPB, 0, s>>>(d.cnt, F1, d.totals);
+    return d.totals;
+}
+
 int Group::find_crowds(cudaStream_t s, bool *found, std::string &err) {
     uint32_t most = 0u;
     cudaError_t e = cudaSuccess;
     if (d.N > kCrowd) {
-        const int64_t F1 = kSlabs * d.total_cells + 1;
-        e = cudaMemsetAsync(d.totals, 0, sizeof(uint32_t), s);
-        k_crowd_counts<<<nblocks(d.N), TPB, 0, s>>>(d.pos, d.N, d.params, d.cnt, F1 - 1);
-        k_crowd_max<<<std::min<unsigned>(nblocks(F1, 16 * TPB), 152 * 8), TPB, 0, s>>>(d.cnt, F1, d.totals);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&most, d.totals, sizeof(most), cudaMemcpyDeviceToHost, s);
+        count_crowds(d.N, s);
+        e = cudaMemcpyAsync(&most, d.totals, sizeof(most), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e == cudaSuccess) e = cudaGetLastError();
     }

@@ -180,3 +180,29 @@ def test_a_crowded_set_is_ordered_by_the_radix_sort(m, crowded):
     loaded.set_incremental(True)
     loaded.load()
     assert loaded.kernels_per_iter == kernels
+
+
+@pytest.mark.parametrize("kind,m,fixed,crowded", [
+    ("joined", 400, False, False), ("joined", 600, False, True), ("loose", 600, False, False),
+    ("loose", 600, True, True), ("loose", 400, True, False)])
+def test_features_on_one_key_are_noticed_when_they_are_generated(kind, m, fixed, crowded):
+    # tiny triangles within a thousandth of dx: m pairs joined at a corner, which
+    # is a singular point (fixed), or m loose ones, each a loop with one feature
+    # point (fixed on request)
+    dx = 0.1
+    rng = np.random.default_rng(8)
+    c = rng.uniform(-1e-4, 1e-4, (m, 3)) + 0.03
+    v = np.concatenate([c] + [c + rng.normal(size=(m, 3)) * 1e-5 for _ in range(4)])
+    k = np.arange(m)
+    t = [np.stack([k, k + m, k + 2 * m], 1)] + [np.stack([k, k + 3 * m, k + 4 * m], 1)] * (kind == "joined")
+    t = np.concatenate(t + [[[5 * m, 5 * m + 1, 5 * m + 2]]])
+    v = np.concatenate([v, [[-1.0, -1, -1], [1, 1, 1], [1, -1, 1]]])
+    b = pkg.Body(v.astype(np.float32), t.astype(np.int32), dx, 1.3 * dx)
+    b.set_fixed_features(fixed)
+    b.extract_features(30.0)
+    b.map_particles(surface=False, volume=False)
+    n = np.bincount(b.get_particles()[1], minlength=5)
+    assert n[W.CLS_P] == (m if kind == "joined" else 0) and n[W.CLS_F] >= (0 if kind == "joined" else m)
+    radix = pkg.Batch([b])
+    radix.set_incremental(False)
+    assert (pkg.Batch([b]).kernels_per_iter == radix.kernels_per_iter) == crowded
