@@ -317,8 +317,8 @@ int fppg_project_points(fppg_ctx *ctx, const float *y_host, const int32_t *cls_h
                         int64_t n, float *x_host, int32_t *cons_out_host, int32_t *ok_host);
 
 /* A6 bookkeeping: *queued = particles of the last iteration that went to
- * the triangle search (the others finished in the step: features, nothing
- * within reach, or a volume particle inside its inside certificate, i.e. a
+ * the triangle search (the others finished in the step: features of lines of
+ * at most 8 segments, nothing within reach, or a volume particle inside its inside certificate, i.e. a
  * ball that an earlier search found free of surface and inside a closed
  * mesh); *closed = 1 when every mesh edge has two faces of opposite
  * direction and no face is degenerate (certificates apply), else 0.

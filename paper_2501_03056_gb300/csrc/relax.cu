@@ -341,7 +341,9 @@ __device__ inline void put_slot(uint32_t k, const float4 &q, uint32_t id, int32_
 // by memory: 68 B per particle, with a chain of four dependent loads (id,
 // position, start, the key's ids).  Two particles per thread keep more of
 // them in flight once the blocks fill the chip (18.9 M particles: 278 -> 250
-// us, 7.1 M: 107 -> 97 us); below that one (42 k: 3.1 against 3.9 us).
+// us, 7.1 M: 107 -> 97 us); below that one (42 k: 3.1 against 3.9 us).  Grid build
+// with one and two: 0.24 M 18.1 / 20.2 us, 0.51 M 24.3 / 24.9, 0.86 M 34.4 / 34.5,
+// 1.16 M 43.1 / 42.9, 1.95 M 67.1 / 65.2, 4.0 M 124.8 / 120.5.
 constexpr int64_t kGatherTwoMinN = 1 << 20;
 
 template <int kGatherItems>
@@ -928,17 +930,11 @@ __device__ inline float surface_cert_radius(const AsmParams &A, int n_projectabl
     return fmaxf(r_other * (1.f - 0x1p-10f) - A.dx * 0x1p-12f, 0.f);
 }
 
-// closest projectable triangle (smallest |plane distance|, ties to the lower
-// index) among those binned into the 27 cells around y, or into y's own
-// cell alone (own_cell); -1 when none
-// The candidate triangles of the 27 cells around y's cell from that cell's
-// list (built with the mesh: the distinct triangles of the 27 cells): 1 with
-// [beg, end) into M.cand; 2 when the list was too long to build (probe the
-// cells); 0 when no triangle lies in the 27 cells.  Warp-uniform.
-// The same as a range of triangle cell c: [beg, end) into M.cand, (0, 0)
-// for no triangle, (kProbeCells, kProbeCells) for a list too long to build.
-// The step computes it for every particle it queues, so that the search
-// starts from the list instead of the chain bitmap -> rank -> list start.
+// The candidate triangles of the 27 cells around triangle cell c as a range
+// [beg, end) of M.cand (built with the mesh: the distinct triangles of the 27
+// cells), (0, 0) for no triangle, (kProbeCells, kProbeCells) for a list too long
+// to build.  The step computes it for every particle it queues, so that the
+// search starts from the list instead of the chain bitmap -> rank -> list start.
 constexpr uint32_t kProbeCells = 0xffffffffu;
 
 __device__ inline uint2 cand_range(const MeshView &M, const AsmParams &A, uint32_t c) {
@@ -955,6 +951,8 @@ __device__ inline uint32_t tri_cell_of(const AsmParams &A, float3 y) {
                    cell_coord(y.z, A.tg_o[2], A.tg_inv, A.tg_n[2]));
 }
 
+// the candidates of y's cell: 1 with [beg, end) into M.cand, 2 for cells to be
+// probed, 0 for none; the same for every lane of a group, which holds one y.
 // pre: the range of y's cell when the caller has it (nullptr: look it up)
 __device__ inline int cell_candidates(const MeshView &M, const AsmParams &A, float3 y, uint32_t &beg, uint32_t &end,
                                       const uint2 *pre = nullptr) {
@@ -996,6 +994,9 @@ __device__ inline void for_27_candidates(const MeshView &M, const AsmParams &A, 
     }
 }
 
+// closest projectable triangle (smallest |plane distance|, ties to the lower
+// index) among those binned into the 27 cells around y, or into y's own
+// cell alone (own_cell); -1 when none
 template <int G>
 __device__ int group_project_surface(const MeshView &M, const AsmParams &A, float3 y, float &dist,
                                      bool own_cell = false, const uint2 *pre = nullptr, float *cert_r = nullptr) {
@@ -1204,7 +1205,9 @@ __device__ inline bool near_body(const MeshView &M, const AsmParams &Q, float3 x
                             cell_coord(x.z, Q.tg_o[2], Q.tg_inv, Q.tg_n[2])));
 }
 
-// segments of a feature line that the step walks itself
+// segments of a feature line that the step walks itself.  Cylinder of 105 k
+// particles, step and search together with its lines in the step / the search:
+// lines of 4 segments 20.2 / 20.6 us, 24 23.8 / 20.6, 64 35.2 / 22.1, 128 54.6 / 24.7.
 constexpr int kLaneSegments = 8;
 
 // ---- A5 + A6 -------------------------------------------------------------------
@@ -1383,7 +1386,8 @@ __device__ inline int64_t queue_slot(uint32_t nf, int64_t N, uint32_t e) {
 // particles go to the closest projectable triangle or revert, volume particles
 // are accepted when the pseudonormal sign says inside.  Bound by the latency of
 // its dependent loads, so what counts is how many particles are in flight and
-// how many of a group's lanes the candidate list feeds: SEARCH_NOTE
+// how many of a group's lanes the candidate list feeds (lists of 4.7 on the gear:
+// 39.8 us an iteration with 8 lanes, 54.8 with 32; Group::set_search_lanes).
 // At most 64 registers (four blocks, 32 warps per SM).
 template <int G>
 __global__ void __launch_bounds__(TPB, 4) k_search(const float4 *__restrict__ pos_s,
