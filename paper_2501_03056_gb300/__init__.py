@@ -222,7 +222,8 @@ class Body:
 
     def set_incremental(self, on: bool):
         """Order the keys by the counting sort over the fine keys (True) or by
-        a full stable radix sort (False); both give the same bits."""
+        a full stable radix sort (False); both give the same bits.  Without a
+        call the library chooses (fppg_batch_set_incremental)."""
         self._chk(lib().fppg_set_incremental(self._h, int(bool(on))))
 
     def set_cell_order(self, order: int):
@@ -607,7 +608,8 @@ class Batch:
 
     def set_incremental(self, on: bool):
         """Order the keys by the counting sort over the fine keys (True) or by
-        a full stable radix sort (False); both give the same bits."""
+        a full stable radix sort (False); both give the same bits.  Without a
+        call the library chooses (fppg_batch_set_incremental)."""
         self._chk(lib().fppg_batch_set_incremental(self._h, int(bool(on))))
 
     def set_mobile_classes(self, classes):
