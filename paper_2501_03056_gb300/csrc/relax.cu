@@ -1557,8 +1557,11 @@ int Group::find_crowds(cudaStream_t s, bool *found, std::string &err) {
     uint32_t most = 0u;
     cudaError_t e = cudaSuccess;
     if (d.N > kCrowd) {
-        count_crowds(d.N, s);
-        e = cudaMemcpyAsync(&most, d.totals, sizeof(most), cudaMemcpyDeviceToHost, s);
+        // (the counters may be at work in a relaxation on a stream that the
+        // caller has left)
+        e = cudaDeviceSynchronize();
+        if (e == cudaSuccess) count_crowds(d.N, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&most, d.totals, sizeof(most), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e == cudaSuccess) e = cudaGetLastError();
     }

@@ -206,3 +206,27 @@ def test_features_on_one_key_are_noticed_when_they_are_generated(kind, m, fixed,
     radix = pkg.Batch([b])
     radix.set_incremental(False)
     assert (pkg.Batch([b]).kernels_per_iter == radix.kernels_per_iter) == crowded
+
+
+def test_looking_for_crowds_waits_for_a_relaxation_on_another_stream():
+    # 20,000 fixed particles among moving ones; the classes are set again on
+    # another stream while the body relaxes
+    import torch
+    rng = np.random.default_rng(12)
+    x = rng.uniform(-0.45, 0.45, (40000, 3)).astype(np.float32)
+    cls = np.where(rng.uniform(size=len(x)) < 0.5, W.CLS_I, W.CLS_V).astype(np.int32)
+    got = []
+    for switch in (False, True):
+        b = pkg.Body(*W.cube_mesh(0.5), 0.03, 0.039)
+        b.set_particles(x, cls)
+        one, two = torch.cuda.Stream(), torch.cuda.Stream()
+        b.set_stream(one)
+        b.relax(300)
+        if switch:
+            b.set_stream(two)
+            b.set_mobile_classes((W.CLS_S, W.CLS_V, W.CLS_F))
+            b.set_fixed_features(False)
+        got.append(b.get_particles()[0])
+        b.relax(20)
+        got.append(b.get_particles()[0])
+    assert np.array_equal(got[0], got[2]) and np.array_equal(got[1], got[3])
