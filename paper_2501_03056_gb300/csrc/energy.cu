@@ -201,10 +201,32 @@ __global__ void __launch_bounds__(TPB) k_grad(const float4 *__restrict__ pos_s, 
     }
 }
 
-// x = y - ((y - a) . n) n for S particles with a triangle; w bits kept
+// A body's parameters into or out of a forward's state, which holds whether the
+// rows were ranked instead of the table's address; by one block
+__device__ inline void copy_params(const AsmParams *in, AsmParams *out, const uint32_t *row_rank) {
+    static_assert(sizeof(AsmParams) % 4 == 0, "copied by words");
+    for (int q = threadIdx.x; q < (int)(sizeof(AsmParams) / 4); q += blockDim.x)
+        reinterpret_cast<uint32_t *>(out)[q] = reinterpret_cast<const uint32_t *>(in)[q];
+    __syncthreads();
+    if (threadIdx.x == 0) out->row_rank = row_rank;
+}
+
+__global__ void k_restore_params(const AsmParams *__restrict__ in, const uint32_t *__restrict__ ranked,
+                                 const uint32_t *__restrict__ table, AsmParams *__restrict__ out) {
+    copy_params(in, out, *ranked ? table : nullptr);
+}
+
+// x = y - ((y - a) . n) n for S particles with a triangle; w bits kept.  kept
+// (nullable): the parameters P, and in *ranked whether their rows are ranked
 __global__ void k_project_frozen(const float *__restrict__ y, const float4 *__restrict__ pos,
                                  const int32_t *__restrict__ cons, int64_t N, const float *__restrict__ V,
-                                 const int32_t *__restrict__ T, float4 *__restrict__ out) {
+                                 const int32_t *__restrict__ T, float4 *__restrict__ out,
+                                 const AsmParams *__restrict__ P, AsmParams *__restrict__ kept,
+                                 uint32_t *__restrict__ ranked) {
+    if (kept && blockIdx.x == 0) {
+        copy_params(P, kept, nullptr);
+        if (threadIdx.x == 0) *ranked = P->row_rank != nullptr;
+    }
     const int64_t i = (int64_t)blockIdx.x * TPB + threadIdx.x;
     if (i >= N) return;
     const float4 p = pos[i];
@@ -291,20 +313,6 @@ __global__ void k_vertex_sum(const uint32_t *__restrict__ vkey_s, const uint32_t
     gV[3 * (size_t)v] = (float)sx;
     gV[3 * (size_t)v + 1] = (float)sy;
     gV[3 * (size_t)v + 2] = (float)sz;
-}
-
-// a body's parameters into or out of a forward's state, which holds whether the
-// rows were ranked instead of the table's address
-__global__ void k_copy_params(const AsmParams *__restrict__ in, const uint32_t *__restrict__ in_ranked,
-                              const uint32_t *__restrict__ table, AsmParams *__restrict__ out,
-                              uint32_t *__restrict__ out_ranked) {
-    static_assert(sizeof(AsmParams) % 4 == 0, "copied by words");
-    for (int q = threadIdx.x; q < (int)(sizeof(AsmParams) / 4); q += blockDim.x)
-        reinterpret_cast<uint32_t *>(out)[q] = reinterpret_cast<const uint32_t *>(in)[q];
-    __syncthreads();
-    if (threadIdx.x > 0) return;
-    if (out_ranked) *out_ranked = in->row_rank != nullptr;
-    out->row_rank = in_ranked && *in_ranked ? table : nullptr;
 }
 
 // What a backward needs of its forward, in key order: the grid of the projected
@@ -415,7 +423,7 @@ int energy(Group &g, const Body &b, const float *y_dev, const float *verts_dev, 
     EnergyScratch &es = g.escr;
     const float *V = verts_dev ? verts_dev : b.d_verts;
     float4 *saved = d.pos;
-    k_project_frozen<<<nblocks(N), TPB, 0, s>>>(y_dev, d.pos, d.cons, N, V, b.d_tris, es.xs);
+    k_project_frozen<<<nblocks(N), TPB, 0, s>>>(y_dev, d.pos, d.cons, N, V, b.d_tris, es.xs, nullptr, nullptr, nullptr);
     d.pos = es.xs;
     build_grid(g, s);
     d.pos = saved;
@@ -448,8 +456,8 @@ int energy_forward(Group &g, const Body &b, const float *y_dev, const float *ver
     ForwardState st;
     lay_out(N, d.total_cells, static_cast<char *>(state), &st);
     const float *V = verts_dev ? verts_dev : b.d_verts;
-    k_copy_params<<<1, 128, 0, s>>>(d.params, nullptr, nullptr, st.params, st.ranked);
-    k_project_frozen<<<nblocks(N), TPB, 0, s>>>(y_dev, d.pos, d.cons, N, V, b.d_tris, es.xs);
+    k_project_frozen<<<nblocks(N), TPB, 0, s>>>(y_dev, d.pos, d.cons, N, V, b.d_tris, es.xs, d.params, st.params,
+                                                 st.ranked);
     DevGroup w = d;
     w.pos = es.xs;
     w.pos_s = st.pos_s;
@@ -474,7 +482,7 @@ int energy_backward(Group &g, const Body &b, int64_t N, const float *y_dev, cons
     EnergyScratch &es = g.escr;
     ForwardState st;
     lay_out(N, d.total_cells, static_cast<char *>(const_cast<void *>(state)), &st);
-    k_copy_params<<<1, 128, 0, s>>>(st.params, st.ranked, d.row_rank, es.params, nullptr);
+    k_restore_params<<<1, 128, 0, s>>>(st.params, st.ranked, d.row_rank, es.params);
     k_grad<<<nblocks(N), TPB, 0, s>>>(st.pos_s, st.pos_p, N, es.params, st.fstart, st.coef_s, st.coef_v, 1.f, es.xs,
                                       nullptr);
     pull_back(es, b, N, y_dev, verts_dev ? verts_dev : b.d_verts, es.xs, st.id_s, st.pos_s, st.cons_s, gy, gV, s);
