@@ -208,18 +208,24 @@ void forget_lost_particles(fppg_ctx *c) {
     c->cls_host.clear();
 }
 
-// The order of the keys for the particles as they are (Group::find_crowds).
-// Moving particles repel each other and pay more for their pairs than for their
-// place, so only a set with enough fixed ones is looked at.
-int ctx_crowds(fppg_ctx *c) {
-    Group &g = c->group;
+// Whether the keys of n particles of the classes cls are looked at for crowds
+// (Group::find_crowds): moving particles repel each other and pay more for their
+// pairs than for their place, so only with enough fixed ones.
+bool may_crowd(const fppg_ctx *c, const int32_t *cls, int64_t n) {
     int64_t fixed = c->n_still + c->n_ghost;
     const int moving = c->mobile_mask & (c->fixed_features ? ~(1 << FPPG_F) : ~0);
     const int still = kMovable & ~moving;
-    if (still)
-        for (int32_t cl : c->cls_host) fixed += (still >> cl) & 1;
+    for (int64_t i = 0; still && i < n && fixed <= (int64_t)kCrowd; i++) fixed += (still >> cls[i]) & 1;
+    return fixed > (int64_t)kCrowd;
+}
+
+// the order of the keys for the particles as they are
+int ctx_crowds(fppg_ctx *c) {
+    Group &g = c->group;
     g.crowded = false;
-    if (fixed > (int64_t)kCrowd && g.find_crowds(c->stream, &g.crowded, c->err)) return FPPG_ERR_CUDA;
+    if (may_crowd(c, c->cls_host.data(), (int64_t)c->cls_host.size()) &&
+        g.find_crowds(c->stream, &g.crowded, c->err))
+        return FPPG_ERR_CUDA;
     g.choose_order();
     return FPPG_OK;
 }
@@ -465,14 +471,19 @@ int fppg_set_particles(fppg_ctx *ctx, const float *xyz_host, const int32_t *cls_
         }
     }
     ctx->n = n;
+    ctx->n_still = still.load();
+    const bool look = may_crowd(ctx, cls_host, n);
+    if (look) CUDA_OR(ctx->err, cudaDeviceSynchronize());   // (as in Group::find_crowds)
+    if (n > 0) k_pack<<<nb(n), 256, 0, ctx->stream>>>(dx, dc, n, 0, g.d.pos, g.d.cons);
+    // the keys are counted while the host copies the classes
+    uint32_t most = 0u, *const crowd = look ? g.count_crowds(n, ctx->stream) : nullptr;
     if ((int64_t)ctx->cls_host.size() != n) ctx->cls_host.resize((size_t)n);
     int32_t *ch = ctx->cls_host.data();
     host_parallel(n, [&](int64_t a, int64_t b) { std::copy(cls_host + a, cls_host + b, ch + a); });
-    if (n > 0) k_pack<<<nb(n), 256, 0, ctx->stream>>>(dx, dc, n, 0, g.d.pos, g.d.cons);
-    ctx->n_still = still.load();
-    const int r = ctx_crowds(ctx);
-    if (r) return r;
+    if (crowd) CUDA_OR(ctx->err, cudaMemcpyAsync(&most, crowd, sizeof(most), cudaMemcpyDeviceToHost, ctx->stream));
     CUDA_OR(ctx->err, cudaStreamSynchronize(ctx->stream));
+    g.crowded = most > kCrowd;
+    g.choose_order();
     ctx->has_particles = true;
     return ctx_group(ctx);
 }

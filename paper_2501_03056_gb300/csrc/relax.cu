@@ -1563,7 +1563,6 @@ int Group::find_crowds(cudaStream_t s, bool *found, std::string &err) {
         if (e == cudaSuccess) count_crowds(d.N, s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&most, d.totals, sizeof(most), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e == cudaSuccess) e = cudaGetLastError();
     }
     if (e != cudaSuccess) {
         err = std::string("crowded keys: ") + cudaGetErrorString(e);
